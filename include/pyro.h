@@ -94,8 +94,8 @@ typedef struct {
     uint64_t seed;     /* Philox key */
     void *stream;      /* cudaStream_t to run on; NULL = the library creates one */
     int tile[3];       /* labelling tile in cells: power-of-two edges, each dividing L, at most
-                          512 cells; {0,0,0} = default (Ising 8 x 8 x 4, n-vector 8 x 4 x 4,
-                          each edge reduced to the largest power of two dividing L) */
+                          512 cells; {0,0,0} = default (Ising 8 x 8 x 4, n-vector 8 x 4 x 4 for
+                          most L; power-of-two edges chosen by L that need not divide it) */
     void *workspace;   /* NULL = the library allocates (and frees) the lattice's device memory;
                           else caller-owned device memory (for instance a torch tensor's data_ptr),
                           at least pyro_workspace_bytes(cfg) bytes, 256-byte aligned, from which
@@ -204,8 +204,9 @@ int pyro_set_graphs(pyro_handle h, int on);
 /* Autotuner: equilibrate a scratch lattice for 60 sweeps at beta, then
  * replay the same nsweeps sweeps from that state with every candidate
  * labelling tile (power-of-two edges dividing L, 64 to 512 cells) and
- * return the fastest in tile_out (pass it in pyro_config.tile) and its
- * device ms per sweep (NULL allowed).  Results are cached per (GPU
+ * return the fastest in tile_out (pass it in pyro_config.tile; {0,0,0} if
+ * that is the default tile and its edges do not divide L) and its device ms
+ * per sweep (NULL allowed).  Results are cached per (GPU
  * name, L, model, precision) in the process and, if the environment
  * variable PYRO_AUTOTUNE_CACHE names a file, across processes.  Allocates
  * and frees a scratch lattice per candidate; synchronises the device. */
@@ -298,8 +299,8 @@ int pyro_batch_init(pyro_batch *out, int R, const int *L, const double *beta, in
                     int precision, int start, uint64_t seed);
 
 /* Same with a labelling tile for every replica (power-of-two edges dividing
- * every L; NULL or {0,0,0} = the default of the lattices' common divisor),
- * e.g. from pyro_batch_autotune. */
+ * every L; NULL or {0,0,0} = the default, one tile for all, chosen by the
+ * sizes), e.g. from pyro_batch_autotune. */
 int pyro_batch_init_ex(pyro_batch *out, int R, const int *L, const double *beta, int model,
                        int precision, int start, uint64_t seed, const int tile[3]);
 

@@ -63,8 +63,9 @@ static std::string check_args(int R, const int *Ls, const double *betas, int mod
     if (start != PYRO_START_UP && start != PYRO_START_RANDOM) return "start must be PYRO_START_UP or PYRO_START_RANDOM";
     if (!(J > 0.0) || !std::isfinite(J)) return "J must be positive and finite";
     t = default_tile(Ls, R, model);
-    if (tile && (tile[0] || tile[1] || tile[2])) t = TileShape{tile[0], tile[1], tile[2]};
-    return check_tile(Ls, R, model, prec, t);
+    const bool callers = tile && (tile[0] || tile[1] || tile[2]);
+    if (callers) t = TileShape{tile[0], tile[1], tile[2]};
+    return check_tile(Ls, R, model, prec, t, callers);
 }
 
 static int create(Engine &e, int R, const int *Ls, const double *betas, int model, int prec, int start, double J,
@@ -545,8 +546,17 @@ static int autotune_set(int R, const int *Ls, const double *betas, int model, in
             ref.release();
             return fail(PYRO_E_CUDA, "autotune: reference lattices failed");
         }
-        for (const TileShape &t : tile_candidates(g, model)) {
-            if (!check_tile(Ls, R, model, prec, t).empty()) continue;
+        // the default tile is a candidate of its own where it is no caller's
+        // tile (its edges need not divide L); it is returned as {0, 0, 0}
+        std::vector<TileShape> cand = tile_candidates(g, model);
+        const bool t0_callers = check_tile(Ls, R, model, prec, t0).empty();
+        if (!t0_callers) {
+            cand.push_back(TileShape{0, 0, 0});
+            best = cand.back();
+        }
+        for (const TileShape &ct : cand) {
+            const TileShape t = ct.TX ? ct : t0;
+            if (ct.TX && !check_tile(Ls, R, model, prec, t).empty()) continue;
             Engine e;
             if (e.setup(R, Ls, betas, model, prec, PYRO_START_RANDOM, 1.0, seeds.data(), nullptr, t, err) != cudaSuccess) {
                 cudaGetLastError();
@@ -569,7 +579,7 @@ static int autotune_set(int R, const int *Ls, const double *betas, int model, in
             }
             if (best_ms < 0.0 || ms < best_ms) {
                 best_ms = ms;
-                best = t;
+                best = ct;
             }
         }
         ref.release();

@@ -217,14 +217,6 @@ uint64_t ising_threshold(double beta, double J)
     return tq >= 4294967296.0 ? (1ull << 32) : (uint64_t)tq;
 }
 
-// Largest power of two that divides L and is at most cap.
-static int pow2_divisor_at_most(int L, int cap)
-{
-    int d = 1;
-    while (2 * d <= cap && L % (2 * d) == 0) d *= 2;
-    return d;
-}
-
 static int log2i(int v)
 {
     int l = 0;
@@ -234,21 +226,59 @@ static int log2i(int v)
 
 static bool is_pow2(int v) { return v > 0 && (v & (v - 1)) == 0; }
 
+// Tiles along an axis of L cells with tile edge T (the last may reach past
+// the lattice).
+static int tiles_along(int L, int T) { return (L + T - 1) / T; }
+
+static int64_t tiles_of(int L, const TileShape &t)
+{
+    return (int64_t)tiles_along(L, t.TX) * tiles_along(L, t.TY) * tiles_along(L, t.TZ);
+}
+
+// The tile whose modelled sweep is cheapest over the set of lattices, among
+// the power-of-two tiles of at most 256 cells (Ising) or 128 (n-vector).  The
+// edges need not divide L.  Model: every tile costs its cells, padded to the
+// lattice's edge and to a warp, times 1 + w (1/TX + 1/TY + 1/TZ) over the axes
+// it does not cover, for the crossing unions of its faces; w is the measured
+// cost of the crossing phase per face cell over the local phase's per cell
+// (L = 128, Ising: 186 us over 0.5 face cells per cell against 240 us; n = 3:
+// 183 over 0.625 against 534).  Before, the edges were the largest powers of
+// two dividing L: one-cell tiles of one thread for odd L (Ising L = 45: 951 us
+// a sweep, now 99; Heisenberg FP64 L = 50, tile 2 x 2 x 2: 2,521 us, now 814).
+// Sets of at most 65,536 cells do not fill the GPU and are bound by a block's
+// latency, which grows with its threads: at most 64 cells there (Ising
+// L = 16: 76 us a sweep with 4 x 4 x 4, 84 with 16 x 4 x 4 or 8 x 8 x 4; L = 32:
+// 80 and 92), except where one lattice is hardly more than one tile (L = 8:
+// 71 us with 4 x 4 x 4, 65 with 8 x 8 x 4).
 TileShape default_tile(const int *Ls, int R, int model)
 {
-    int g = Ls[0];
-    for (int r = 1; r < R; ++r) {
-        int a = g, b = Ls[r];
-        while (b) {
-            const int t = a % b;
-            a = b;
-            b = t;
-        }
-        g = a;
-    }
-    if (model == PYRO_ISING)  // 8 x 8 x 4 (8 x 8 x 8 is within 1-2 % at L = 256; the autotuner picks per lattice)
-        return TileShape{pow2_divisor_at_most(g, 8), pow2_divisor_at_most(g, 8), pow2_divisor_at_most(g, 4)};
-    return TileShape{pow2_divisor_at_most(g, 8), pow2_divisor_at_most(g, 4), pow2_divisor_at_most(g, 4)};
+    int64_t cells = 0;
+    for (int r = 0; r < R; ++r) cells += (int64_t)Ls[r] * Ls[r] * Ls[r];
+    const int cap = cells > 512 && cells <= 65536 ? 64 : (model == PYRO_ISING ? 256 : 128);
+    const double w = model == PYRO_ISING ? 1.2 : 0.55;
+    TileShape best{1, 1, 1};
+    double best_cost = -1.0;
+    for (int tx = 32; tx >= 1; tx /= 2)
+        for (int ty = 32; ty >= 1; ty /= 2)
+            for (int tz = 32; tz >= 1; tz /= 2) {
+                const int nt = tx * ty * tz;
+                if (nt > cap) continue;
+                double cost = 0.0;
+                for (int r = 0; r < R; ++r) {
+                    double f = 1.0;
+                    if (tx < Ls[r]) f += w / tx;
+                    if (ty < Ls[r]) f += w / ty;
+                    if (tz < Ls[r]) f += w / tz;
+                    cost += f * (double)tiles_of(Ls[r], TileShape{tx, ty, tz}) * std::max(nt, 32);
+                }
+                // equal costs: fewer threads, then the longer x edge
+                if (best_cost < 0.0 || cost < best_cost * (1.0 - 1e-9) ||
+                    (cost < best_cost * (1.0 + 1e-9) && nt < best.TX * best.TY * best.TZ)) {
+                    best_cost = cost;
+                    best = TileShape{tx, ty, tz};
+                }
+            }
+    return best;
 }
 
 size_t local_smem(int model, int prec, const TileShape &t)
@@ -256,10 +286,11 @@ size_t local_smem(int model, int prec, const TileShape &t)
     return model == PYRO_ISING ? ising_local_smem(t) : vec_local_smem(t, prec);
 }
 
-std::string check_tile(const int *Ls, int R, int model, int prec, const TileShape &t)
+// The edges of a caller's tile divide every L; the default tile's need not.
+std::string check_tile(const int *Ls, int R, int model, int prec, const TileShape &t, bool callers)
 {
     if (!is_pow2(t.TX) || !is_pow2(t.TY) || !is_pow2(t.TZ)) return "tile edges must be powers of two";
-    for (int r = 0; r < R; ++r)
+    for (int r = 0; r < R && callers; ++r)
         if (Ls[r] % t.TX || Ls[r] % t.TY || Ls[r] % t.TZ) return "tile edges must divide every L";
     const int nt = t.TX * t.TY * t.TZ;
     if (nt > 512) return "tile has too many cells (at most 512)";
@@ -284,13 +315,12 @@ size_t workspace_bytes(int R, const int *Ls, int model, int prec, const TileShap
 {
     size_t total = ws_align((size_t)R * sizeof(DevStats));
     int64_t ntiles = 0;
-    const int nt = t.TX * t.TY * t.TZ;
     for (int r = 0; r < R; ++r) {
         const int64_t ncells = (int64_t)Ls[r] * Ls[r] * Ls[r], N = 16 * ncells;
         total += ws_align(spin_bytes_of(model, prec, N)) + ws_align((size_t)N * sizeof(unsigned long long)) +
                  ws_align((size_t)N * sizeof(uint16_t)) + ws_align((size_t)ncells * sizeof(uint16_t)) +
                  ws_align((size_t)ncells * sizeof(uint32_t)) + ws_align((size_t)N * sizeof(int32_t));
-        ntiles += ncells / nt;
+        ntiles += tiles_of(Ls[r], t);
     }
     return total + ws_align((size_t)(ntiles + (int64_t)R * FOLD_GROUPS) * 4 * sizeof(double)) +
            ws_align((size_t)R * sizeof(Rep));
@@ -351,7 +381,6 @@ cudaError_t Engine::setup(int R_, const int *Ls, const double *betas, int model_
     epoch = g_epoch_start;
     ntiles = 0;
     nblocks = 0;
-    const int nt = t.TX * t.TY * t.TZ;
     // every replica's statistics in one block, so that they can be read in
     // one copy
     DevStats *stats = nullptr;
@@ -365,8 +394,8 @@ cudaError_t Engine::setup(int R_, const int *Ls, const double *betas, int model_
         p.L = Ls[r];
         p.ncells = (int64_t)Ls[r] * Ls[r] * Ls[r];
         p.N = 16 * p.ncells;
-        p.ntx = Ls[r] / t.TX;
-        p.nty = Ls[r] / t.TY;
+        p.ntx = tiles_along(Ls[r], t.TX);
+        p.nty = tiles_along(Ls[r], t.TY);
         p.seed = seeds[r];
         p.J = J;
         p.thr = ising_threshold(betas ? betas[r] : 0.0, J);
@@ -374,7 +403,7 @@ cudaError_t Engine::setup(int R_, const int *Ls, const double *betas, int model_
         beta.push_back(betas ? betas[r] : 0.0);
         B.tile_begin[r] = ntiles;
         B.block_begin[r] = nblocks;
-        ntiles += p.ncells / nt;
+        ntiles += tiles_of(Ls[r], t);
         nblocks += (p.ncells + CELL_BLOCK - 1) / CELL_BLOCK;
         struct {
             void **ptr;

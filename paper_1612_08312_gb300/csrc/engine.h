@@ -87,7 +87,8 @@ TileShape default_tile(const int *Ls, int R, int model);
 // Device bytes of every array of a set of lattices (labels included), as
 // the engine lays them out in a caller-owned workspace.
 size_t workspace_bytes(int R, const int *Ls, int model, int prec, const TileShape &t);
-std::string check_tile(const int *Ls, int R, int model, int prec, const TileShape &t);
+// callers: t is a caller's tile (its edges must divide every L), not the default one.
+std::string check_tile(const int *Ls, int R, int model, int prec, const TileShape &t, bool callers = true);
 size_t local_smem(int model, int prec, const TileShape &t);
 
 }  // namespace pyro

@@ -44,7 +44,7 @@ __global__ void __launch_bounds__(512) ising_local_kernel(const __grid_constant_
     uint32_t w[7];
     {
         const int L = c.L;
-        const int x = c.ox + c.lx, y = c.oy + c.ly, z = c.oz + c.lz;
+        const int x = c.x, y = c.y, z = c.z;
         const int xm = wrap_back(x, L), ym = wrap_back(y, L), zm = wrap_back(z, L);
 #pragma unroll
         for (int m = 0; m < 7; ++m) {
@@ -55,11 +55,12 @@ __global__ void __launch_bounds__(512) ising_local_kernel(const __grid_constant_
     __syncthreads();  // table and pair counters ready
     uint32_t anti[3];
     antiparallel_groups(w[0], down_word(w), anti[0], anti[1], anti[2]);
+    const uint32_t vmask = c.valid ? 0xFFFFu : 0u;  // no bond past the lattice
     uint32_t act[3];
     const ByteCompare bc(R.thr);
     if (bc.all || bc.none) {
 #pragma unroll
-        for (int g = 0; g < 3; ++g) act[g] = bc.all ? ~anti[g] & 0xFFFFu : 0u;
+        for (int g = 0; g < 3; ++g) act[g] = bc.all ? ~anti[g] & vmask : 0u;
     } else {
         // bond 48 c + 16 g + 4 f + q: byte 4 f + q of BOND call 3 c + g; the
         // three calls are drawn together (independent chains interleave)
@@ -69,7 +70,7 @@ __global__ void __launch_bounds__(512) ising_local_kernel(const __grid_constant_
         const uint32_t t4 = bc.t8 * 0x01010101u;
 #pragma unroll
         for (int g = 0; g < 3; ++g) {
-            const uint32_t sat = ~anti[g] & 0xFFFFu;
+            const uint32_t sat = ~anti[g] & vmask;
             const uint32_t ww[4] = {wd[g].x, wd[g].y, wd[g].z, wd[g].w};
             uint32_t a = 0;
 #pragma unroll
@@ -97,7 +98,7 @@ __global__ void __launch_bounds__(512) ising_flip_kernel(const __grid_constant__
     const TileCtx c = tile_ctx(B, R, blockIdx.x - B.tile_begin[r]);
     const uint32_t flip = cell_flip_mask(c, R, smem);
     uint16_t *spins = static_cast<uint16_t *>(R.spins);
-    spins[c.cell] = (uint16_t)((uint32_t)spins[c.cell] ^ flip);
+    if (c.valid) spins[c.cell] = (uint16_t)((uint32_t)spins[c.cell] ^ flip);
 }
 
 // Canonical label (global index of the cluster root) of every site.
@@ -108,6 +109,7 @@ __global__ void __launch_bounds__(512) labels_kernel(const __grid_constant__ Bat
     const TileCtx c = tile_ctx(B, R, blockIdx.x - B.tile_begin[r]);
     int root[16];
     uint32_t flip;
+    if (!c.valid) return;
     resolve_cell(c, R, (uint32_t)R.st->last_epoch, root, flip);
     int4 *dst = reinterpret_cast<int4 *>(R.labels + 16 * c.cell);
 #pragma unroll
@@ -128,6 +130,7 @@ __global__ void __launch_bounds__(MEASURE_BLOCK) ising_measure_kernel(const __gr
 #pragma unroll 4
     for (int t = threadIdx.x; t < c.nt; t += blockDim.x) {
         const int x = c.ox + (t & (c.TX - 1)), y = c.oy + ((t >> c.lTX) & (c.TY - 1)), z = c.oz + (t >> (c.lTX + c.lTY));
+        if (max(x, max(y, z)) >= L) continue;
         const int xm = wrap_back(x, L), ym = wrap_back(y, L), zm = wrap_back(z, L);
         uint32_t w[7];
 #pragma unroll
@@ -207,7 +210,8 @@ __global__ void __launch_bounds__(512, 4) boundary_kernel(const __grid_constant_
     if ((int)threadIdx.x < nface) {
         int lx, ly, lz;
         face_cell_coords(B, threadIdx.x, lx, ly, lz);
-        todo = R.dmask[(int64_t)(ox + lx) + (int64_t)L * ((int64_t)(oy + ly) + (int64_t)L * (oz + lz))];
+        if (max(ox + lx, max(oy + ly, oz + lz)) < L)
+            todo = R.dmask[(int64_t)(ox + lx) + (int64_t)L * ((int64_t)(oy + ly) + (int64_t)L * (oz + lz))];
     }
     const int lane = threadIdx.x & 31;
     const int n = __popc(todo);

@@ -106,7 +106,6 @@ extern "C" int pyro_ising_sweep_noalloc(const uint16_t *spins_in, uint16_t *spin
     const cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int Ls[1] = {L};
     const TileShape t = default_tile(Ls, 1, PYRO_ISING);
-    const int nt = t.TX * t.TY * t.TZ;
     unsigned char *base = nullptr;
     uint32_t epoch = 0;
     {
@@ -145,8 +144,8 @@ extern "C" int pyro_ising_sweep_noalloc(const uint16_t *spins_in, uint16_t *spin
     rep.ncells = (int64_t)L * L * L;
     rep.N = 16 * rep.ncells;
     rep.L = L;
-    rep.ntx = L / t.TX;
-    rep.nty = L / t.TY;
+    rep.ntx = (L + t.TX - 1) / t.TX;
+    rep.nty = (L + t.TY - 1) / t.TY;
 
     Batch B;
     std::memset(&B, 0, sizeof(B));
@@ -159,7 +158,7 @@ extern "C" int pyro_ising_sweep_noalloc(const uint16_t *spins_in, uint16_t *spin
     while ((1 << B.lTX) < t.TX) ++B.lTX;
     while ((1 << B.lTY) < t.TY) ++B.lTY;
     while ((1 << B.lTZ) < t.TZ) ++B.lTZ;
-    const int64_t ntiles = rep.ncells / nt;
+    const int64_t ntiles = (int64_t)rep.ntx * rep.nty * ((L + t.TZ - 1) / t.TZ);
     B.tile_begin[1] = ntiles;
     B.block_begin[1] = (rep.ncells + CELL_BLOCK - 1) / CELL_BLOCK;
 

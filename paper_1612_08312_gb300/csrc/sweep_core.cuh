@@ -20,11 +20,17 @@
 namespace pyro {
 
 // Position of the calling thread's cell in its tile and in the lattice.
-// Tile edges are powers of two (shifts, no divisions).
+// Tile edges are powers of two (shifts, no divisions) and need not divide L:
+// the last tile of an axis may reach past the lattice.  A thread whose cell
+// lies there has valid = false; its coordinates are clamped into the lattice
+// (so that its loads stay in bounds), it activates no bond and stores
+// nothing.  A tile that covers a whole axis wraps onto itself along it.
 struct TileCtx {
     int TX, TY, TZ, lTX, lTY, nt, L;
     int ox, oy, oz;
     int lx, ly, lz, t;
+    int x, y, z;  // the cell's coordinates (clamped)
+    bool valid;
     int64_t cell;
     // local cell offset of a backward step along each axis (valid only if
     // the step stays in the tile), and whether it leaves the tile
@@ -52,15 +58,20 @@ __device__ __forceinline__ TileCtx tile_ctx(const Batch &B, const Rep &R, int64_
     c.lx = c.t & (c.TX - 1);
     c.ly = (c.t >> c.lTX) & (c.TY - 1);
     c.lz = c.t >> (c.lTX + c.lTY);
-    const int x = c.ox + c.lx, y = c.oy + c.ly, z = c.oz + c.lz;
-    c.cell = (int64_t)x + (int64_t)c.L * ((int64_t)y + (int64_t)c.L * z);
-    // a tile that spans a whole axis wraps onto itself along it
-    c.bx = c.lx == 0 && c.TX != c.L;
-    c.by = c.ly == 0 && c.TY != c.L;
-    c.bz = c.lz == 0 && c.TZ != c.L;
-    c.dxm = c.lx > 0 ? -1 : c.TX - 1;
-    c.dym = c.ly > 0 ? -c.TX : (c.TY - 1) * c.TX;
-    c.dzm = c.lz > 0 ? -c.TX * c.TY : (c.TZ - 1) * c.TX * c.TY;
+    c.x = c.ox + c.lx;
+    c.y = c.oy + c.ly;
+    c.z = c.oz + c.lz;
+    c.valid = max(c.x, max(c.y, c.z)) < c.L;
+    c.x = min(c.x, c.L - 1);
+    c.y = min(c.y, c.L - 1);
+    c.z = min(c.z, c.L - 1);
+    c.cell = (int64_t)c.x + (int64_t)c.L * ((int64_t)c.y + (int64_t)c.L * c.z);
+    c.bx = c.lx == 0 && c.TX < c.L;
+    c.by = c.ly == 0 && c.TY < c.L;
+    c.bz = c.lz == 0 && c.TZ < c.L;
+    c.dxm = c.lx > 0 ? -1 : c.L - 1;
+    c.dym = c.ly > 0 ? -c.TX : (c.L - 1) * c.TX;
+    c.dzm = c.lz > 0 ? -c.TX * c.TY : (c.L - 1) * c.TX * c.TY;
     return c;
 }
 
@@ -121,6 +132,10 @@ __device__ __forceinline__ int64_t halo_cell(int h, int TX, int TY, int ox, int 
     gx += (gx < 0) ? L : 0;
     gy += (gy < 0) ? L : 0;
     gz += (gz < 0) ? L : 0;
+    // past the lattice (a tile that reaches beyond it): any cell in bounds
+    gx = min(gx, L - 1);
+    gy = min(gy, L - 1);
+    gz = min(gz, L - 1);
     return (int64_t)gx + (int64_t)L * ((int64_t)gy + (int64_t)L * gz);
 }
 
@@ -221,13 +236,13 @@ __device__ __forceinline__ uint32_t tie_bits(uint64_t seed, uint32_t sweep, int6
 
 // The cell's 16 flip bits: bits 16 c .. 16 c + 15 of the FLIP stream (bit i
 // = bit i & 127 of call i >> 7).  One Philox call serves 8 cells; when the
-// 8 cells are 8 consecutive lanes (TX a multiple of 8) one lane draws it.
+// 8 cells are 8 consecutive lanes (TX and L multiples of 8) one lane draws it.
 __device__ __forceinline__ uint32_t cell_flip_bits(const TileCtx &c, uint64_t seed, uint32_t sweep)
 {
     const uint64_t j = (uint64_t)c.cell >> 3;
     const int wsel = (int)((c.cell & 7) >> 1);
     uint32_t word;
-    if ((c.TX & 7) == 0) {
+    if (((c.TX | c.L) & 7) == 0) {
         const unsigned mask = lanes_mask(c.nt);
         uint4 w = make_uint4(0, 0, 0, 0);
         if ((c.lx & 7) == 0) w = philox_call(seed, sweep, TAG_FLIP, j);
@@ -492,10 +507,12 @@ __device__ __forceinline__ void local_core(const TileCtx &c, const Rep &R, const
         packed[2 * f] = root[0] | (root[1] << 16);
         packed[2 * f + 1] = root[2] | (root[3] << 16);
     }
+    const uint32_t fbits = cell_flip_bits(c, R.seed, sweep);
+    if (!c.valid) return;
     uint4 *dst = reinterpret_cast<uint4 *>(R.L16 + 16 * c.cell);
     dst[0] = make_uint4(packed[0], packed[1], packed[2], packed[3]);
     dst[1] = make_uint4(packed[4], packed[5], packed[6], packed[7]);
-    R.F[c.cell] = (uint16_t)cell_flip_bits(c, R.seed, sweep);
+    R.F[c.cell] = (uint16_t)fbits;
     if (c.lx == 0 || c.ly == 0 || c.lz == 0) R.dmask[c.cell] = cross;
 }
 

@@ -130,7 +130,7 @@ __global__ void __launch_bounds__(512, sizeof(T) == 4 ? 2 : 1) vec_local_kernel(
 
     const T K2 = (T)R.K2;
     uint32_t act[3] = {0, 0, 0};
-    if (R.K2 > 0.0) {
+    if (R.K2 > 0.0 && c.valid) {
 #pragma unroll
         for (int g = 0; g < 3; ++g) {
             T xb[16];
@@ -200,7 +200,7 @@ __global__ void __launch_bounds__(512) vec_flip_kernel(const __grid_constant__ B
     __shared__ double s_axis[3];
     if (threadIdx.x == 0) unit_vector_dev<NC>(R.seed, (uint32_t)R.st->sweep, TAG_AXIS, 0, s_axis);
     uint32_t flip = cell_flip_mask(c, R, smem);  // its barrier also publishes s_axis
-    if (!flip) return;
+    if (!flip || !c.valid) return;
     const T r[3] = {(T)s_axis[0], (T)s_axis[1], (T)s_axis[2]};
     T *spins = static_cast<T *>(R.spins);
     const int64_t N = R.N;
@@ -266,7 +266,7 @@ __global__ void __launch_bounds__(512) vec_measure_kernel(const __grid_constant_
     const int L = R.L;
     const int64_t N = R.N;
     const T *sp = static_cast<const T *>(R.spins);
-    const int x = c.ox + c.lx, y = c.oy + c.ly, z = c.oz + c.lz;
+    const int x = c.x, y = c.y, z = c.z;
     int64_t cb[8];
 #pragma unroll
     for (int m = 0; m < 8; ++m) {
@@ -308,8 +308,12 @@ __global__ void __launch_bounds__(512) vec_measure_kernel(const __grid_constant_
             ec += du + dd;
         }
     }
-    const double e = (double)ec, M[3] = {(double)Mc[0], (double)Mc[1], (double)Mc[2]};
-    double tot[4] = {e, M[0], M[1], M[2]};
+    double tot[4] = {0.0, 0.0, 0.0, 0.0};  // a cell past the lattice adds nothing
+    if (c.valid) {
+        tot[0] = (double)ec;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) tot[1 + k] = (double)Mc[k];
+    }
     tile_sum4_f64(tot, c.nt, scratch);
     const double se = tot[0], s0 = tot[1], s1 = tot[2], s2 = tot[3];
     if (threadIdx.x == 0) {
