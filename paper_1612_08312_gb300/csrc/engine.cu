@@ -18,7 +18,7 @@ void ising_launch_init(const Batch &B, int64_t nblocks, int random, cudaStream_t
 void ising_launch_phase(int p, const Batch &B, int64_t ntiles, cudaStream_t s);
 void ising_launch_measure(const Batch &B, int64_t ntiles, cudaStream_t s);
 // vector.cu
-size_t vec_local_smem(const TileShape &t, int prec);
+size_t vec_local_smem(const TileShape &t);
 cudaError_t vec_prepare(int model, int prec, const TileShape &t);
 void vec_launch_init(int model, int prec, const Batch &B, int64_t nblocks, int random, cudaStream_t s);
 void vec_launch_phase(int p, int model, int prec, const Batch &B, int64_t ntiles, cudaStream_t s);
@@ -283,7 +283,7 @@ TileShape default_tile(const int *Ls, int R, int model)
 
 size_t local_smem(int model, int prec, const TileShape &t)
 {
-    return model == PYRO_ISING ? ising_local_smem(t) : vec_local_smem(t, prec);
+    return model == PYRO_ISING ? ising_local_smem(t) : vec_local_smem(t);
 }
 
 // The edges of a caller's tile divide every L; the default tile's need not.

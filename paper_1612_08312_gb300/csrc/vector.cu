@@ -60,23 +60,44 @@ __device__ __forceinline__ void store16(T *p, const T in[16])
     }
 }
 
-// The local kernel's staging area (the halo's projections, then the halo
-// cells' first sites) is dead once the bonds are decided, before the
+// The local kernel's staging area (the halo's projections in FP32, then the
+// halo cells' first sites) is dead once the bonds are decided, before the
 // labelling writes its labels and pair list: when it fits in their room
 // (31 words a cell, the start of the core area) it shares it, which halves
-// the shared memory of the FP32 kernels' common tiles.
-__host__ __device__ constexpr size_t vec_stage_bytes(int TX, int TY, int TZ, size_t es)
+// the shared memory of the common tiles.
+__host__ __device__ constexpr size_t vec_stage_bytes(int TX, int TY, int TZ)
 {
-    return (size_t)16 * halo_cells(TX, TY, TZ) * es + (size_t)halo_cells(TX, TY, TZ) * 4;
+    return (size_t)(16 + 1) * halo_cells(TX, TY, TZ) * 4;
 }
 
-__host__ __device__ constexpr bool vec_stage_shared(int TX, int TY, int TZ, size_t es)
+__host__ __device__ constexpr bool vec_stage_shared(int TX, int TY, int TZ)
 {
-    return vec_stage_bytes(TX, TY, TZ, es) <= (size_t)31 * TX * TY * TZ * 4;
+    return vec_stage_bytes(TX, TY, TZ) <= (size_t)31 * TX * TY * TZ * 4;
 }
 
+// 2^x, relative error at most 2^-22 (PTX ISA, ex2.approx.ftz.f32).
+__device__ __forceinline__ float exp2_approx(float x)
+{
+    float r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// Margin of the bond shortcut below, in units of 1/256 of probability.  The
+// evaluation errs by at most 2e-4 there: 2^-22 of ex2, 2^-22 in its argument
+// y log2 e (which moves exp(-y) by y exp(-y) 2^-22), and the rounding of q.
+// FP64 projections are staged in FP32 as sums of rounded terms, 3e-7 off at
+// most (six roundings of 2^-24), so y = K2 p p' errs by 6e-7 K2 more and q by
+// 1.6e-4 K2.
+template <typename T>
+__device__ __forceinline__ float shortcut_margin(double K2)
+{
+    return sizeof(T) == 4 ? 1e-3f : 1e-3f + 4e-4f * (float)K2;
+}
+
+// Registers: two 512-thread blocks' worth of warps per SM.
 template <int NC, typename T>
-__global__ void __launch_bounds__(512, sizeof(T) == 4 ? 2 : 1) vec_local_kernel(const __grid_constant__ Batch B)
+__global__ void __launch_bounds__(512, 2) vec_local_kernel(const __grid_constant__ Batch B)
 {
     using A = Ar<T>;
     extern __shared__ __align__(16) int smem[];
@@ -84,8 +105,8 @@ __global__ void __launch_bounds__(512, sizeof(T) == 4 ? 2 : 1) vec_local_kernel(
     const Rep &R = B.reps[rep];
     const TileCtx c = tile_ctx(B, R, blockIdx.x - B.tile_begin[rep]);
     const CoreSmem sm = core_smem(smem, c.nt);
-    const bool shared_stage = vec_stage_shared(c.TX, c.TY, c.TZ, sizeof(T));
-    T *proj = reinterpret_cast<T *>(shared_stage ? reinterpret_cast<unsigned char *>(smem) : sm.stage);
+    const bool shared_stage = vec_stage_shared(c.TX, c.TY, c.TZ);
+    float *proj = reinterpret_cast<float *>(shared_stage ? reinterpret_cast<unsigned char *>(smem) : sm.stage);
     const T *spins = static_cast<const T *>(R.spins);
     const int64_t N = R.N;
     const uint32_t sweep = (uint32_t)R.st->sweep;
@@ -97,9 +118,11 @@ __global__ void __launch_bounds__(512, sizeof(T) == 4 ? 2 : 1) vec_local_kernel(
     __shared__ double s_axis[3];
     if (threadIdx.x == 0) unit_vector_dev<NC>(seed, sweep, TAG_AXIS, 0, s_axis);
     __syncthreads();
-    const T r[3] = {(T)s_axis[0], (T)s_axis[1], (T)s_axis[2]};
+    const float rf[3] = {(float)s_axis[0], (float)s_axis[1], (float)s_axis[2]};
 
-    // projections s_i . r of the tile's sites and the backward halo; each
+    // projections s_i . r of the tile's sites and the backward halo, in FP32
+    // (for FP64 spins an approximation that the shortcut's margin covers: FP64
+    // arithmetic here cost more than the whole FP32 kernel); each
     // halo cell's first site is found once (the halo's edges are not powers
     // of two, so this takes divisions) and shared.  Site-major layout (site s
     // of halo cell h at s nh + h): a warp's consecutive cells read
@@ -120,69 +143,97 @@ __global__ void __launch_bounds__(512, sizeof(T) == 4 ? 2 : 1) vec_local_kernel(
         for (int k = 0; k < NC; ++k) load4(spins + k * N + i0, v[k]);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            T pr = A::mul(v[0][q], r[0]);  // in the order of project()
+            float pr = (float)v[0][q] * rf[0];  // in the order of project()
 #pragma unroll
-            for (int k = 1; k < NC; ++k) pr = A::add(pr, A::mul(v[k][q], r[k]));
+            for (int k = 1; k < NC; ++k) pr = Ar<float>::add(pr, Ar<float>::mul((float)v[k][q], rf[k]));
             proj[(s0 + q) * nh + h] = pr;
         }
     }
     __syncthreads();
 
-    const T K2 = (T)R.K2;
     uint32_t act[3] = {0, 0, 0};
     if (R.K2 > 0.0 && c.valid) {
+        // A bond with p = 1 - exp(-K2 p_i p_j) and top byte b of its uniform is
+        // on whatever the low bits if 256 p > b + 1, off if 256 p < b (or p
+        // <= 0): q = 256 p - b from one fast exponential decides all bonds but
+        // those within the margin of [0, 1], about 1 in 250 of the positive
+        // ones.  They take the exact path below, all of them in one loop: with
+        // the exact path expanded at each of the 48 bonds the kernel had
+        // 145 KB of code (now 54) and waited for instructions: L = 128, n = 3, FP32
+        // 534 -> 327 us; FP64, whose projections and exponentials all ran in
+        // FP64, L = 64 862 -> 97 us.
+        const float K2l = (float)R.K2 * 1.44269504f;
+        const float margin = shortcut_margin<T>(R.K2);
+        uint32_t und[3];
+        const int h0 = halo_index(c, 0);
 #pragma unroll
         for (int g = 0; g < 3; ++g) {
-            T xb[16];
-            uint32_t pos = 0;
+            const uint4 wd = philox_call(seed, sweep, TAG_BOND, 3 * (uint64_t)c.cell + g);
+            const uint32_t ww[4] = {wd.x, wd.y, wd.z, wd.w};
+            uint32_t a = 0, u = 0;
 #pragma unroll
             for (int f = 0; f < 4; ++f)
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
                     const int va = slot_a(g, q), vb = slot_b(g, q);
-                    T pa, pb;
+                    float pa, pb;
                     if (slot_up(g, q)) {
-                        pa = proj[(4 * f + va) * nh + halo_index(c, 0)];
-                        pb = proj[(4 * f + vb) * nh + halo_index(c, 0)];
+                        pa = proj[(4 * f + va) * nh + h0];
+                        pb = proj[(4 * f + vb) * nh + h0];
                     } else {
                         pa = proj[down_bit(f, va) * nh + halo_index(c, down_mask(f, va))];
                         pb = proj[down_bit(f, vb) * nh + halo_index(c, down_mask(f, vb))];
                     }
-                    xb[4 * f + q] = A::mul(pa, pb);
-                    pos |= (xb[4 * f + q] > (T)0 ? 1u : 0u) << (4 * f + q);
-                }
-            if (!pos) continue;
-            const uint4 wd = philox_call(seed, sweep, TAG_BOND, 3 * (uint64_t)c.cell + g);
-            const uint32_t ww[4] = {wd.x, wd.y, wd.z, wd.w};
-            uint32_t a = 0;
-#pragma unroll
-            for (int f = 0; f < 4; ++f)
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    if (!((pos >> (4 * f + q)) & 1u)) continue;
-                    const uint32_t byte = (ww[f] >> (8 * q)) & 0xFFu;
-                    if (sizeof(T) == 4) {
-                        // FP32: p = 1 - exp(-y), y = K2 x, exceeds (b + 1) / 256 (so the
-                        // bond is on whatever the low bits) when y > -ln(1 - (b + 1) / 256),
-                        // and stays below b / 256 (off) when y < -ln(1 - b / 256); the
-                        // margins (1e-4 relative, 1e-6 absolute) exceed the errors of
-                        // expm1f (1 ulp of p) and of __logf, so only bonds within them
-                        // take the exact path below, with the same decision either way
-                        const float y = (float)K2 * (float)xb[4 * f + q];
-                        const float ylo = -__logf(1.0f - (float)byte * (1.0f / 256.0f));
-                        const float yhi = -__logf(1.0f - (float)(byte + 1) * (1.0f / 256.0f));  // +inf for 255
-                        if (y > yhi * 1.0001f + 1e-6f) {
-                            a |= 1u << (4 * f + q);
-                            continue;
-                        }
-                        if (y < ylo * 0.9999f - 1e-6f) continue;
-                    }
-                    const ByteCompare bc(prob_threshold(A::bond_p(K2, xb[4 * f + q])));
-                    bool on = bc.all || byte < bc.t8;
-                    if (!bc.all && !bc.none && byte == bc.t8) on = tie_bits(seed, sweep, c.cell, g, f, q) < bc.t24;
-                    a |= (on && !bc.none ? 1u : 0u) << (4 * f + q);
+                    // 256 - b, from the float whose low mantissa bits are b
+                    const float fb = 8388864.0f - __uint_as_float(__byte_perm(ww[f], 0x4B000000u, 0x7440u | (uint32_t)q));
+                    const float e = exp2_approx(-((pa * pb) * K2l));
+                    const float qv = fmaf(-256.0f, e, fb);
+                    const uint32_t bit = 1u << (4 * f + q);
+                    // (a NaN, from an infinite K2l, is neither on nor off)
+                    if (qv > 1.0f + margin) a |= bit;
+                    else if (!(qv < -margin)) u |= bit;
                 }
             act[g] = a;
+            und[g] = u;
+        }
+        const T K2 = (T)R.K2;
+        unsigned long long todo =
+            (unsigned long long)(und[0] | (und[1] << 16)) | ((unsigned long long)und[2] << 32);
+#pragma unroll 1
+        while (todo) {
+            const int k = __ffsll((long long)todo) - 1;
+            todo &= todo - 1;
+            const int g = k >> 4, f = (k >> 2) & 3, q = k & 3;
+            T pr[2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int v = e == 0 ? slot_a(g, q) : slot_b(g, q);
+                const int m = slot_up(g, q) ? 0 : down_mask(f, v);
+                const int s = slot_up(g, q) ? 4 * f + v : down_bit(f, v);
+                if (sizeof(T) == 4) {
+                    pr[e] = (T)proj[s * nh + halo_index(c, m)];
+                } else {
+                    const T r[3] = {(T)s_axis[0], (T)s_axis[1], (T)s_axis[2]};
+                    pr[e] = project<NC, T>(spins, N, (int64_t)hbase[halo_index(c, m)] + s, r);
+                }
+            }
+            const T x = A::mul(pr[0], pr[1]);
+            if (!(x > (T)0)) continue;
+            const ByteCompare bc(prob_threshold(A::bond_p(K2, x)));
+            const uint64_t id = 48 * (uint64_t)c.cell + (uint32_t)k;
+            const uint4 wd = philox_call(seed, sweep, TAG_BOND, id >> 4);
+            const uint32_t byte = (word_of(wd, f) >> (8 * q)) & 0xFFu;
+            bool on = bc.all || byte < bc.t8;
+            if (!on && byte == bc.t8) {
+                const uint4 w4 = philox_call(seed, sweep, TAG_TIE, id >> 2);
+                on = (word_of(w4, q) & 0xFFFFFFu) < bc.t24;
+            }
+            if (on && !bc.none) {
+                const uint32_t bit = 1u << (k & 15);
+                act[0] |= g == 0 ? bit : 0u;
+                act[1] |= g == 1 ? bit : 0u;
+                act[2] |= g == 2 ? bit : 0u;
+            }
         }
     }
     if (shared_stage) __syncthreads();  // the staging area is read no more: the labels may take it
@@ -350,20 +401,19 @@ cudaError_t vec_set_unite_bound(int bound) { return cudaMemcpyToSymbol(c_unite_b
 size_t resolve_smem(const TileShape &t);
 void launch_boundary(const Batch &B, int64_t ntiles, cudaStream_t s);
 
-size_t vec_local_smem(const TileShape &t, int prec)
+size_t vec_local_smem(const TileShape &t)
 {
-    const size_t es = prec == PYRO_FP64 ? 8 : 4;
     const size_t core = core_smem_bytes(t.TX * t.TY * t.TZ);
-    return vec_stage_shared(t.TX, t.TY, t.TZ, es) ? core : core + vec_stage_bytes(t.TX, t.TY, t.TZ, es);
+    return vec_stage_shared(t.TX, t.TY, t.TZ) ? core : core + vec_stage_bytes(t.TX, t.TY, t.TZ);
 }
 
 static size_t vec_measure_smem(const TileShape &t) { return (size_t)4 * t.TX * t.TY * t.TZ * sizeof(double); }
 
 template <int NC, typename T>
 struct VecOps {
-    static cudaError_t prepare(const TileShape &t, int prec)
+    static cudaError_t prepare(const TileShape &t)
     {
-        cudaError_t e = allow_dynamic_smem(vec_local_kernel<NC, T>, vec_local_smem(t, prec));
+        cudaError_t e = allow_dynamic_smem(vec_local_kernel<NC, T>, vec_local_smem(t));
         if (e == cudaSuccess) e = allow_dynamic_smem(vec_flip_kernel<NC, T>, resolve_smem(t));
         return e;
     }
@@ -371,11 +421,11 @@ struct VecOps {
     {
         vec_init_kernel<NC, T><<<(unsigned)nblocks, CELL_BLOCK, 0, s>>>(B, random);
     }
-    static void phase(int p, const Batch &B, int64_t ntiles, int prec, cudaStream_t s)
+    static void phase(int p, const Batch &B, int64_t ntiles, cudaStream_t s)
     {
         const TileShape t{B.TX, B.TY, B.TZ};
         const int nt = B.TX * B.TY * B.TZ;
-        if (p == 0) vec_local_kernel<NC, T><<<(unsigned)ntiles, nt, vec_local_smem(t, prec), s>>>(B);
+        if (p == 0) vec_local_kernel<NC, T><<<(unsigned)ntiles, nt, vec_local_smem(t), s>>>(B);
         else if (p == 1) launch_boundary(B, ntiles, s);
         else vec_flip_kernel<NC, T><<<(unsigned)ntiles, nt, resolve_smem(t), s>>>(B);
     }
@@ -402,8 +452,8 @@ cudaError_t vec_prepare(int model, int prec, const TileShape &t)
     // the labels kernel (compiled with the Ising sweep) serves every model
     const cudaError_t e = ising_prepare(t);
     if (e != cudaSuccess) return e;
-    if (model == PYRO_XY) return prec == PYRO_FP64 ? VecOps<2, double>::prepare(t, prec) : VecOps<2, float>::prepare(t, prec);
-    return prec == PYRO_FP64 ? VecOps<3, double>::prepare(t, prec) : VecOps<3, float>::prepare(t, prec);
+    if (model == PYRO_XY) return prec == PYRO_FP64 ? VecOps<2, double>::prepare(t) : VecOps<2, float>::prepare(t);
+    return prec == PYRO_FP64 ? VecOps<3, double>::prepare(t) : VecOps<3, float>::prepare(t);
 }
 
 void vec_launch_init(int model, int prec, const Batch &B, int64_t nblocks, int random, cudaStream_t s)
@@ -414,7 +464,7 @@ void vec_launch_init(int model, int prec, const Batch &B, int64_t nblocks, int r
 // Phase p of a sweep: 0 local labelling, 1 crossing unions, 2 flip.
 void vec_launch_phase(int p, int model, int prec, const Batch &B, int64_t ntiles, cudaStream_t s)
 {
-    PYRO_VEC_DISPATCH(model, prec, phase(p, B, ntiles, prec, s));
+    PYRO_VEC_DISPATCH(model, prec, phase(p, B, ntiles, s));
 }
 
 void vec_launch_measure(int model, int prec, const Batch &B, int64_t ntiles, cudaStream_t s)
