@@ -24,69 +24,81 @@ void vec_launch_init(int model, int prec, const Batch &B, int64_t nblocks, int r
 void vec_launch_phase(int p, int model, int prec, const Batch &B, int64_t ntiles, cudaStream_t s);
 void vec_launch_measure(int model, int prec, const Batch &B, int64_t ntiles, cudaStream_t s);
 
-// Per replica (one block each): reduce the per-tile partials of the
-// measurement kernel in a fixed order, form E, m = |M|/N, m^2, m^4 (Eq. 1,
-// Eq. 2) and, in mode 1, add them to the Neumaier sums, append the trace
-// record and advance the sweep counter; mode 2 only records them as the last
-// measurement.
+// Threads of an accumulation block.
+constexpr int ACC_THREADS = 128;
+
+// Sums of four values over a block of ACC_THREADS threads in a fixed tree
+// (integers: the first two); results valid in thread 0.
+template <typename V, int NV>
+__device__ __forceinline__ void acc_block_sum(V v[NV], V (*red)[ACC_THREADS])
+{
+    const int t = threadIdx.x;
+#pragma unroll
+    for (int q = 0; q < NV; ++q) red[q][t] = v[q];
+    __syncthreads();
+#pragma unroll
+    for (int o = ACC_THREADS / 2; o > 0; o >>= 1) {
+        if (t < o)
+#pragma unroll
+            for (int q = 0; q < NV; ++q) red[q][t] += red[q][t + o];
+        if (o > 16) __syncthreads();
+        else __syncwarp();
+    }
+#pragma unroll
+    for (int q = 0; q < NV; ++q) v[q] = red[q][0];
+}
+
 // With B.fold groups per replica, a first kernel sums each group of a
 // replica's tile partials (a contiguous range, fixed order) on its own
 // block, so that the accumulation reads B.fold values per replica instead of
 // one per tile; one block reading tens of thousands of partials, in FP64 for
 // the n-vector models, was the accumulation's whole cost.
 template <bool ISING>
-__global__ void __launch_bounds__(256) fold_kernel(const __grid_constant__ Batch B)
+__global__ void __launch_bounds__(ACC_THREADS) fold_kernel(const __grid_constant__ Batch B)
 {
     const int r = blockIdx.x / B.fold, k = blockIdx.x - r * B.fold;
     const int64_t b0 = B.tile_begin[r], n = B.tile_begin[r + 1] - b0;
     const int64_t lo = b0 + n * k / B.fold, hi = b0 + n * (k + 1) / B.fold;
-    const int t = threadIdx.x;
     if (ISING) {
-        __shared__ unsigned long long su[2][256];
-        unsigned long long a = 0, d = 0;
-        for (int64_t b = lo + t; b < hi; b += blockDim.x) {
-            const unsigned long long *p = reinterpret_cast<const unsigned long long *>(B.partials + 4 * b);
-            a += p[0];
-            d += p[1];
+        __shared__ unsigned long long red[2][ACC_THREADS];
+        unsigned long long v[2] = {0, 0};
+#pragma unroll 4
+        for (int64_t b = lo + threadIdx.x; b < hi; b += ACC_THREADS) {
+            const ulonglong2 p = *reinterpret_cast<const ulonglong2 *>(B.partials + 4 * b);
+            v[0] += p.x;
+            v[1] += p.y;
         }
-        su[0][t] = a;
-        su[1][t] = d;
-        __syncthreads();
-        for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-            if (t < o) {
-                su[0][t] += su[0][t + o];
-                su[1][t] += su[1][t + o];
-            }
-            __syncthreads();
-        }
-        if (t == 0) {
-            unsigned long long *o = reinterpret_cast<unsigned long long *>(B.folded + 4 * (int64_t)blockIdx.x);
-            o[0] = su[0][0];
-            o[1] = su[1][0];
-        }
+        acc_block_sum<unsigned long long, 2>(v, red);
+        if (threadIdx.x == 0) *reinterpret_cast<ulonglong2 *>(B.folded + 4 * (int64_t)blockIdx.x) = make_ulonglong2(v[0], v[1]);
     } else {
-        __shared__ double sv[4][256];
+        __shared__ double red[4][ACC_THREADS];
         double v[4] = {0.0, 0.0, 0.0, 0.0};
-        for (int64_t b = lo + t; b < hi; b += blockDim.x)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) v[q] = __dadd_rn(v[q], B.partials[4 * b + q]);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) sv[q][t] = v[q];
-        __syncthreads();
-        for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-            if (t < o)
-#pragma unroll
-                for (int q = 0; q < 4; ++q) sv[q][t] = __dadd_rn(sv[q][t], sv[q][t + o]);
-            __syncthreads();
+#pragma unroll 4
+        for (int64_t b = lo + threadIdx.x; b < hi; b += ACC_THREADS) {
+            const double2 p = *reinterpret_cast<const double2 *>(B.partials + 4 * b);
+            const double2 q = *reinterpret_cast<const double2 *>(B.partials + 4 * b + 2);
+            v[0] += p.x;
+            v[1] += p.y;
+            v[2] += q.x;
+            v[3] += q.y;
         }
-        if (t == 0)
+        acc_block_sum<double, 4>(v, red);
+        if (threadIdx.x == 0)
 #pragma unroll
-            for (int q = 0; q < 4; ++q) B.folded[4 * (int64_t)blockIdx.x + q] = sv[q][0];
+            for (int q = 0; q < 4; ++q) B.folded[4 * (int64_t)blockIdx.x + q] = v[q];
     }
 }
 
+// Per replica (one block each): sum the tiles' partials of the measurement
+// kernel in a fixed order, form E, m = |M|/N, m^2, m^4 (Eq. 1, Eq. 2) and, in
+// mode 1, add them to the Neumaier sums, append the trace record and advance
+// the sweep counter; mode 2 only records them as the last measurement.
+// A block per replica, bound by its own latency: few threads (a replica has
+// at most FOLD_MIN_TILES partials, or its FOLD_GROUPS folded ones) and one
+// tree for all four sums.  With 1,024 threads and a shuffle tree per sum it
+// took 10 us (Ising) and 16 us (n-vector) whatever the lattice.
 template <bool ISING>
-__global__ void __launch_bounds__(1024) accumulate_kernel(const __grid_constant__ Batch B, int mode, int nc)
+__global__ void __launch_bounds__(ACC_THREADS) accumulate_kernel(const __grid_constant__ Batch B, int mode, int nc)
 {
     const int r = blockIdx.x;
     const Rep &R = B.reps[r];
@@ -97,35 +109,32 @@ __global__ void __launch_bounds__(1024) accumulate_kernel(const __grid_constant_
     const int64_t b1 = B.fold ? (int64_t)(r + 1) * B.fold : B.tile_begin[r + 1];
     double tot[4] = {0.0, 0.0, 0.0, 0.0};
     if (ISING) {
-        __shared__ unsigned long long su[2][1024];
-        unsigned long long a = 0, d = 0;
-        for (int64_t b = b0 + threadIdx.x; b < b1; b += blockDim.x) {
-            const unsigned long long *p = reinterpret_cast<const unsigned long long *>(src + 4 * b);
-            a += p[0];
-            d += p[1];
+        __shared__ unsigned long long red[2][ACC_THREADS];
+        unsigned long long v[2] = {0, 0};
+#pragma unroll 4
+        for (int64_t b = b0 + threadIdx.x; b < b1; b += ACC_THREADS) {
+            const ulonglong2 p = *reinterpret_cast<const ulonglong2 *>(src + 4 * b);
+            v[0] += p.x;
+            v[1] += p.y;
         }
-        su[0][threadIdx.x] = a;
-        su[1][threadIdx.x] = d;
-        __syncthreads();
-        for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-            if ((int)threadIdx.x < o) {
-                su[0][threadIdx.x] += su[0][threadIdx.x + o];
-                su[1][threadIdx.x] += su[1][threadIdx.x + o];
-            }
-            __syncthreads();
-        }
+        acc_block_sum<unsigned long long, 2>(v, red);
         if (threadIdx.x != 0) return;
-        const long long anti = (long long)su[0][0];
-        const long long M = R.N - 2 * (long long)su[1][0];
+        const long long anti = (long long)v[0];
+        const long long M = R.N - 2 * (long long)v[1];
         tot[0] = (double)(3 * R.N - 2 * anti);  // sum over bonds of s_i s_j
         tot[1] = (double)M;
     } else {
-        double v[4] = {0.0, 0.0, 0.0, 0.0};
-        for (int64_t b = b0 + threadIdx.x; b < b1; b += blockDim.x)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) v[q] = __dadd_rn(v[q], src[4 * b + q]);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) tot[q] = block_sum_f64(v[q]);
+        __shared__ double red[4][ACC_THREADS];
+#pragma unroll 4
+        for (int64_t b = b0 + threadIdx.x; b < b1; b += ACC_THREADS) {
+            const double2 p = *reinterpret_cast<const double2 *>(src + 4 * b);
+            const double2 q = *reinterpret_cast<const double2 *>(src + 4 * b + 2);
+            tot[0] += p.x;
+            tot[1] += p.y;
+            tot[2] += q.x;
+            tot[3] += q.y;
+        }
+        acc_block_sum<double, 4>(tot, red);
         if (threadIdx.x != 0) return;
     }
     const double E = __dmul_rn(-R.J, tot[0]);
@@ -190,8 +199,8 @@ __global__ void reset_epoch_kernel(const __grid_constant__ Batch B)
 // Host launcher of the accumulation kernel for callers outside this file.
 void launch_accumulate(const Batch &B, bool ising, int mode, int nc, cudaStream_t s)
 {
-    if (ising) accumulate_kernel<true><<<B.R, 1024, 0, s>>>(B, mode, nc);
-    else accumulate_kernel<false><<<B.R, 1024, 0, s>>>(B, mode, nc);
+    if (ising) accumulate_kernel<true><<<B.R, ACC_THREADS, 0, s>>>(B, mode, nc);
+    else accumulate_kernel<false><<<B.R, ACC_THREADS, 0, s>>>(B, mode, nc);
 }
 
 // ------------------------------------------------------------------ host --
@@ -499,11 +508,11 @@ void Engine::enqueue_phase(int p, int mode)
         else vec_launch_measure(model, prec, B, ntiles, stream);
     } else {
         if (B.fold) {
-            if (model == PYRO_ISING) fold_kernel<true><<<R * B.fold, 256, 0, stream>>>(B);
-            else fold_kernel<false><<<R * B.fold, 256, 0, stream>>>(B);
+            if (model == PYRO_ISING) fold_kernel<true><<<R * B.fold, ACC_THREADS, 0, stream>>>(B);
+            else fold_kernel<false><<<R * B.fold, ACC_THREADS, 0, stream>>>(B);
         }
-        if (model == PYRO_ISING) accumulate_kernel<true><<<R, 1024, 0, stream>>>(B, mode, 1);
-        else accumulate_kernel<false><<<R, 1024, 0, stream>>>(B, mode, model);
+        if (model == PYRO_ISING) accumulate_kernel<true><<<R, ACC_THREADS, 0, stream>>>(B, mode, 1);
+        else accumulate_kernel<false><<<R, ACC_THREADS, 0, stream>>>(B, mode, model);
     }
 }
 
