@@ -82,23 +82,20 @@ __device__ __forceinline__ unsigned lanes_mask(int nt)
     return cnt >= 32 ? 0xffffffffu : ((1u << cnt) - 1u);
 }
 
-// Deterministic sums of four doubles over the block's nt threads: a fixed
-// tree in shared memory (any nt), one barrier per level for all four;
-// results valid in thread 0.  scratch holds 4 nt doubles.  (A warp-shuffle
-// tree would add in FP64 on every lane at every level; FP64 adds are scarce
-// on this GPU.)
+// Deterministic sums of the four groups of nt doubles in scratch (written by
+// the block and published by a barrier; group q at q nt): a fixed tree in
+// shared memory (any nt), one barrier per level for all four; results valid
+// in thread 0.  (A warp-shuffle tree would add in FP64 on every lane at every
+// level; FP64 adds are scarce on this GPU.)
 __device__ __forceinline__ void tile_sum4_f64(double v[4], int nt, double *scratch)
 {
-    const int t = threadIdx.x;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) scratch[q * nt + t] = v[q];
-    __syncthreads();
-    int span = 1;
-    while (span < nt) span <<= 1;
-    for (int o = span >> 1; o > 0; o >>= 1) {
-        if (t < o && t + o < nt)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) scratch[q * nt + t] = __dadd_rn(scratch[q * nt + t], scratch[q * nt + t + o]);
+    for (int lo = 30 - __clz(max(2 * nt - 1, 2)); lo >= 0; --lo) {
+        const int o = 1 << lo;  // half the span of nt values still to add
+        // the threads share the 4 o additions of a level
+        for (int e = threadIdx.x; e < 4 * o; e += blockDim.x) {
+            const int q = e >> lo, t = e & (o - 1);
+            if (t + o < nt) scratch[q * nt + t] = __dadd_rn(scratch[q * nt + t], scratch[q * nt + t + o]);
+        }
         __syncthreads();
     }
 #pragma unroll

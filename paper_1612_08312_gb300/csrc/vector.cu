@@ -18,23 +18,12 @@
 // labelling), the global union of tile-crossing clusters (boundary_kernel,
 // shared with the Ising sweep), vec_flip (root, flip, reflection) and
 // vec_measure (E and M per block in FP64).
+#include <algorithm>
+
 #include "nvec.cuh"
 #include "sweep_core.cuh"
 
 namespace pyro {
-
-// 16 consecutive values of T (a cell's sites of one component, 64- or
-// 128-byte aligned) to and from registers in 16-byte accesses.
-template <typename T>
-__device__ __forceinline__ void load16(const T *p, T out[16])
-{
-    const uint4 *q = reinterpret_cast<const uint4 *>(p);
-#pragma unroll
-    for (int k = 0; k < (int)(sizeof(T)); ++k) {
-        const uint4 w = q[k];
-        memcpy(&out[k * 16 / (int)sizeof(T)], &w, 16);
-    }
-}
 
 // 4 consecutive values of T (16-byte aligned) in 16-byte accesses.
 template <typename T>
@@ -45,18 +34,6 @@ __device__ __forceinline__ void load4(const T *p, T out[4])
     for (int k = 0; k < (int)(sizeof(T)) / 4; ++k) {
         const uint4 w = q[k];
         memcpy(&out[k * 16 / (int)sizeof(T)], &w, 16);
-    }
-}
-
-template <typename T>
-__device__ __forceinline__ void store16(T *p, const T in[16])
-{
-    uint4 *q = reinterpret_cast<uint4 *>(p);
-#pragma unroll
-    for (int k = 0; k < (int)(sizeof(T)); ++k) {
-        uint4 w;
-        memcpy(&w, &in[k * 16 / (int)sizeof(T)], 16);
-        q[k] = w;
     }
 }
 
@@ -240,139 +217,315 @@ __global__ void __launch_bounds__(512, 2) vec_local_kernel(const __grid_constant
     local_core(c, R, sm, act[0], act[1], act[2], sweep);
 }
 
+// t <- t / sqrt(t . t), every operation correctly rounded: the bits of sqrt_
+// and div, in fewer operations for the vectors a sweep meets, whose squared
+// length q is within a few units in the last place of 1.  With M mantissa
+// bits and d = bits(q) - bits(1), sqrt(1 + x) = 1 + x/2 - x^2/8 ..: for q d
+// units of 2^-M above 1 (below: -d units of 2^-(M+1)) the correctly rounded
+// root is floor(d / 2) units from 1, the x^2/8 term being far below half a
+// unit for the d taken here; it only breaks the ties of odd d downwards.
+//
+// FP32: the quotients by s = 1 + e follow from one correctly rounded
+// reciprocal r by Markstein's theorem (IBM J. Res. Dev. 34, 1990): with the
+// faithful quotient g = fma(-e, t, t) (e^2 < 2^-27), fma(t - s g, r, g) is the
+// correctly rounded t / s, the residual t - s g being exact in one fma (not
+// for tiny t: those divide).
+template <int NC>
+__device__ __forceinline__ void normalise(float t[NC])
+{
+    float q = t[0] * t[0];
+#pragma unroll
+    for (int k = 1; k < NC; ++k) q = Ar<float>::add(q, Ar<float>::mul(t[k], t[k]));
+    const int d = __float_as_int(q) - 0x3F800000;
+    if (d > -1024 && d < 1024) {
+        const int h = d >> 1;
+        if (h == 0) return;  // the length rounds to 1
+        const float s = __int_as_float(0x3F800000 + h), e = s - 1.0f, r = __frcp_rn(s);
+        bool ok = true;
+        float o[NC];
+#pragma unroll
+        for (int k = 0; k < NC; ++k) {
+            const float g = __fmaf_rn(-e, t[k], t[k]);
+            o[k] = __fmaf_rn(__fmaf_rn(-s, g, t[k]), r, g);
+            ok &= fabsf(t[k]) > 1e-25f;
+        }
+        if (ok) {
+#pragma unroll
+            for (int k = 0; k < NC; ++k) t[k] = o[k];
+            return;
+        }
+    }
+    q = sqrtf(q);
+#pragma unroll
+    for (int k = 0; k < NC; ++k) t[k] = t[k] / q;
+}
+
+// FP64: by integer arithmetic, since roots and quotients took four fifths of
+// the FP64 flip, whose two FP64 lanes a clock per SM bound it.  Quotient of
+// t = T 2^e by s = 1 + h 2^-52, h > 0: T/s = T - T h / (2^52 + h); by
+// s = 1 - k 2^-53: T/s = T + T k / (2^53 - k).  The fraction, rounded to
+// nearest, is its quotient by the power of two alone, rounded, or one step
+// from that (checked by the remainder); no quotient of two floats lies
+// halfway.  A result past the binade of t, a zero and a denormal divide.
+template <int NC>
+__device__ __forceinline__ void normalise(double t[NC])
+{
+    using A = Ar<double>;
+    double q = A::mul(t[0], t[0]);
+#pragma unroll
+    for (int k = 1; k < NC; ++k) q = A::add(q, A::mul(t[k], t[k]));
+    constexpr long long ONE = 0x3FF0000000000000ll, FIELD = (1ll << 52) - 1;
+    const long long d = __double_as_longlong(q) - ONE;
+    if (d > -128 && d < 128) {
+        const int h = (int)d >> 1;
+        if (h == 0) return;  // the length rounds to 1
+        const int m = abs(h), sh = h > 0 ? 52 : 53;
+        const long long D = (1ll << sh) + h;
+        bool ok = true;
+        double o[NC];
+#pragma unroll
+        for (int k = 0; k < NC; ++k) {
+            const long long b = __double_as_longlong(t[k]);
+            const long long mant = b & FIELD;
+            const long long n = (mant | (1ll << 52)) * m;  // below 2^59
+            long long i = (n + (1ll << (sh - 1))) >> sh;
+            const long long r2 = 2 * (n - i * D);
+            if (h > 0) i -= r2 < -D;  // the divisor exceeds the power of two
+            else i += r2 > D;
+            const long long to = h > 0 ? mant - i : mant + i;
+            ok &= to >= 0 && to <= FIELD && ((b >> 53) & 0x3FF) != 0;  // exponent field above 1
+            o[k] = __longlong_as_double(h > 0 ? b - i : b + i);
+        }
+        if (ok) {
+#pragma unroll
+            for (int k = 0; k < NC; ++k) t[k] = o[k];
+            return;
+        }
+    }
+    q = A::sqrt_(q);
+#pragma unroll
+    for (int k = 0; k < NC; ++k) t[k] = A::div(t[k], q);
+}
+
+// s <- the reflection s - 2 (s . r) r, normalised.
+template <int NC, typename T>
+__device__ __forceinline__ void reflect(T t[NC], const T r[3])
+{
+    using A = Ar<T>;
+    T pr = A::mul(t[0], r[0]);  // the projection, in the order of project()
+#pragma unroll
+    for (int k = 1; k < NC; ++k) pr = A::add(pr, A::mul(t[k], r[k]));
+    const T d2 = A::mul((T)2, pr);
+#pragma unroll
+    for (int k = 0; k < NC; ++k) t[k] = A::sub(t[k], A::mul(d2, r[k]));
+    normalise<NC>(t);
+}
+
+// Reflection of the flipped sites.  Every thread first finds its cell's flip
+// mask.  FP32: the block then walks its cells' sites in the order of memory,
+// 16 bytes of every component per thread, so that a warp reads and writes
+// whole lines (a thread per cell stored half sectors, 2.7 times the sectors
+// the spins have) and groups without a flipped site are not touched: bound by
+// HBM, 805 MB in 134 us at L = 128, n = 3 (210 us before).  FP64: bound by the
+// FP64 units, so the flipped sites are listed and every lane takes one.
 template <int NC, typename T>
 __global__ void __launch_bounds__(512) vec_flip_kernel(const __grid_constant__ Batch B)
 {
-    using A = Ar<T>;
     extern __shared__ __align__(16) int smem[];
     const int rep = find_rep(B.tile_begin, B.R, blockIdx.x);
     const Rep &R = B.reps[rep];
     const TileCtx c = tile_ctx(B, R, blockIdx.x - B.tile_begin[rep]);
     __shared__ double s_axis[3];
     if (threadIdx.x == 0) unit_vector_dev<NC>(R.seed, (uint32_t)R.st->sweep, TAG_AXIS, 0, s_axis);
-    uint32_t flip = cell_flip_mask(c, R, smem);  // its barrier also publishes s_axis
-    if (!flip || !c.valid) return;
-    const T r[3] = {(T)s_axis[0], (T)s_axis[1], (T)s_axis[2]};
     T *spins = static_cast<T *>(R.spins);
     const int64_t N = R.N;
-    if (NC * sizeof(T) > 16) {
-        // FP64 Heisenberg: a cell's 48 doubles do not fit the registers;
-        // site by site
-        while (flip) {
-            const int s = __ffs(flip) - 1;
-            flip &= flip - 1;
-            const int64_t i = 16 * c.cell + s;
-            const T pr = project<NC, T>(spins, N, i, r);
-            const T d2 = A::mul((T)2, pr);
-            T t[3];
+    if (sizeof(T) == 8) {
+        // the tile's flipped sites in the order of memory along its rows
+        int *list = smem;
+        __shared__ int wtotal[17];
+        uint32_t mask = cell_flip_mask(c, R, smem + 16 * c.nt);
+        if (!c.valid) mask = 0;
+        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (c.nt + 31) >> 5;
+        const unsigned lanes = lanes_mask(c.nt);
+        const int n = __popc(mask);
+        int incl = n;
 #pragma unroll
-            for (int k = 0; k < NC; ++k) t[k] = A::sub(spins[k * N + i], A::mul(d2, r[k]));
-            T q = A::mul(t[0], t[0]);
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(lanes, incl, o);
+            if (lane >= o) incl += v;
+        }
+        if (lane == 31 || (int)threadIdx.x == c.nt - 1) wtotal[wid] = incl;
+        __syncthreads();  // publishes s_axis too
+        int total = 0, base = 0;
+        for (int w = 0; w < nw; ++w) {
+            if (w == wid) base = total;
+            total += wtotal[w];
+        }
+        int pos = base + incl - n;
+        while (mask) {
+            list[pos++] = (int)(16 * c.cell) + __ffs(mask) - 1;
+            mask &= mask - 1;
+        }
+        __syncthreads();
+        const T r[3] = {(T)s_axis[0], (T)s_axis[1], (T)s_axis[2]};
+        for (int e = threadIdx.x; e < total; e += c.nt) {
+            T *p = spins + list[e];
+            T t[NC];
 #pragma unroll
-            for (int k = 1; k < NC; ++k) q = A::add(q, A::mul(t[k], t[k]));
-            q = A::sqrt_(q);
+            for (int k = 0; k < NC; ++k) t[k] = p[k * N];
+            reflect<NC, T>(t, r);
 #pragma unroll
-            for (int k = 0; k < NC; ++k) spins[k * N + i] = A::div(t[k], q);
+            for (int k = 0; k < NC; ++k) p[k * N] = t[k];
         }
         return;
     }
-    // the cell's 16 sites of every component in registers (16-byte loads)
-    T sv[NC][16];
+    // per cell: its first site and its flip mask (0 past the lattice)
+    int2 *todo = reinterpret_cast<int2 *>(smem);
+    const uint32_t mask = cell_flip_mask(c, R, smem + 2 * c.nt);
+    todo[c.t] = make_int2((int)(16 * c.cell), c.valid ? (int)mask : 0);
+    __syncthreads();  // publishes s_axis too
+    const T r[3] = {(T)s_axis[0], (T)s_axis[1], (T)s_axis[2]};
+    for (int idx = threadIdx.x; idx < 4 * c.nt; idx += blockDim.x) {
+        const int2 cell = todo[idx >> 2];
+        const int s0 = 4 * (idx & 3);
+        const uint32_t flip = ((uint32_t)cell.y >> s0) & 0xFu;
+        if (!flip) continue;
+        T *p = spins + cell.x + s0;
+        T sv[NC][4];
 #pragma unroll
-    for (int k = 0; k < NC; ++k) load16(spins + k * N + 16 * c.cell, sv[k]);
+        for (int k = 0; k < NC; ++k) load4(p + k * N, sv[k]);
 #pragma unroll
-    for (int s = 0; s < 16; ++s) {
-        if (!((flip >> s) & 1u)) continue;
-        T pr = A::mul(sv[0][s], r[0]);  // the projection, in the order of project()
+        for (int s = 0; s < 4; ++s) {
+            if (!((flip >> s) & 1u)) continue;
+            T t[NC];
 #pragma unroll
-        for (int k = 1; k < NC; ++k) pr = A::add(pr, A::mul(sv[k][s], r[k]));
-        const T d2 = A::mul((T)2, pr);
-        T t[3];
+            for (int k = 0; k < NC; ++k) t[k] = sv[k][s];
+            reflect<NC, T>(t, r);
 #pragma unroll
-        for (int k = 0; k < NC; ++k) t[k] = A::sub(sv[k][s], A::mul(d2, r[k]));
-        T q = A::mul(t[0], t[0]);
+            for (int k = 0; k < NC; ++k) sv[k][s] = t[k];
+        }
 #pragma unroll
-        for (int k = 1; k < NC; ++k) q = A::add(q, A::mul(t[k], t[k]));
-        q = A::sqrt_(q);
-#pragma unroll
-        for (int k = 0; k < NC; ++k) sv[k][s] = A::div(t[k], q);
+        for (int k = 0; k < NC; ++k) {
+            uint4 w;
+            memcpy(&w, sv[k], 16);
+            *reinterpret_cast<uint4 *>(p + k * N) = w;
+        }
     }
-#pragma unroll
-    for (int k = 0; k < NC; ++k) store16(spins + k * N + 16 * c.cell, sv[k]);
 }
+
+constexpr int VEC_MEASURE_BLOCK = 128;
 
 // Energy (Eq. 1) and magnetisation of the current configuration: every
 // cell sums the 48 bonds it owns and its 16 spins (FP64 spins in FP64; FP32
 // spins in FP32 within the cell, since FP64 adds and conversions run at a
 // small fraction of the FP32 rate on this GPU), then in FP64; one partial
 // (E, M_x, M_y, M_z) per tile, summed in a fixed order.
+//
+// Four threads per cell, one per FCC point f: a warp's sites are consecutive
+// in memory (one thread per cell read half sectors at a stride of a cell and
+// moved 4.6 times the spins' sectors).  FP32: the cell's sums run over f =
+// 0..3 in turn, handed from thread to thread, and are added in FP64, every
+// lane its own quantity; FP64, bound by the FP64 units: every thread its own
+// sums.  A block of 128 threads takes 32 cells at a time.
 template <int NC, typename T>
-__global__ void __launch_bounds__(512) vec_measure_kernel(const __grid_constant__ Batch B)
+__global__ void __launch_bounds__(VEC_MEASURE_BLOCK) vec_measure_kernel(const __grid_constant__ Batch B)
 {
     extern __shared__ __align__(16) int smem[];
-    double *scratch = reinterpret_cast<double *>(smem);
+    double *scratch = reinterpret_cast<double *>(smem);  // blockDim values (FP64: 4 blockDim)
     const int rep = find_rep(B.tile_begin, B.R, blockIdx.x);
     const Rep &R = B.reps[rep];
-    const TileCtx c = tile_ctx(B, R, blockIdx.x - B.tile_begin[rep]);
-    const int L = R.L;
+    const int L = R.L, TX = B.TX, TY = B.TY, nt = B.TX * B.TY * B.TZ;
+    const uint32_t tile = (uint32_t)(blockIdx.x - B.tile_begin[rep]);
+    const uint32_t txy = tile / (uint32_t)R.ntx;
+    const int ox = (int)(tile - txy * (uint32_t)R.ntx) * TX;
+    const int oy = (int)(txy % (uint32_t)R.nty) * TY;
+    const int oz = (int)(txy / (uint32_t)R.nty) * B.TZ;
     const int64_t N = R.N;
     const T *sp = static_cast<const T *>(R.spins);
-    const int x = c.x, y = c.y, z = c.z;
-    int64_t cb[8];
+    const int f = threadIdx.x & 3;
+    const unsigned lanes = lanes_mask((int)blockDim.x);
+    // FP32: thread f < 3 sums M_f and thread 3 E; FP64: every thread all four
+    double acc[4] = {0.0, 0.0, 0.0, 0.0};
+    // blockDim is a multiple of 4 and at most 4 nt; every thread makes the same rounds
+    for (int c0 = 0; c0 < nt; c0 += blockDim.x >> 2) {
+        const int t = c0 + (threadIdx.x >> 2);
+        const int x = ox + (t & (TX - 1)), y = oy + ((t >> B.lTX) & (TY - 1)), z = oz + (t >> (B.lTX + B.lTY));
+        const bool valid = t < nt && max(x, max(y, z)) < L;
+        T u[NC][4] = {}, w[NC][4] = {};
+        if (valid) {
+            const int own = 16 * (x + L * (y + L * z));
 #pragma unroll
-    for (int m = 0; m < 8; ++m) {
-        const int cx = (m & 1) ? wrap_back(x, L) : x;
-        const int cy = (m & 2) ? wrap_back(y, L) : y;
-        const int cz = (m & 4) ? wrap_back(z, L) : z;
-        cb[m] = 16 * ((int64_t)cx + (int64_t)L * ((int64_t)cy + (int64_t)L * cz));
-    }
-    // the cell's own 16 sites in registers (16-byte loads); the down
-    // tetrahedra's vertices in backward cells are read from global memory
-    T sv[NC][16];
+            for (int k = 0; k < NC; ++k) load4(sp + k * N + own + 4 * f, u[k]);
+            // the down tetrahedron's vertices nu = 1..3: basis nu of FCC point
+            // f ^ nu, a cell back along the axes where a(f) is 0 and a(nu) 1
 #pragma unroll
-    for (int k = 0; k < NC; ++k) load16(sp + k * N + cb[0], sv[k]);
-    using Acc = T;  // the cell's own sums: the spins' precision
-    Acc ec = (Acc)0, Mc[3] = {(Acc)0, (Acc)0, (Acc)0};
+            for (int nu = 1; nu < 4; ++nu) {
+                const int bx = (nu >> 1) & 1 & ~(f >> 1), by = nu & 1 & ~f, bz = ((nu ^ (nu >> 1)) & 1) & ~(f ^ (f >> 1));
+                const int cx = bx ? wrap_back(x, L) : x, cy = by ? wrap_back(y, L) : y, cz = bz ? wrap_back(z, L) : z;
+                const int site = 16 * (cx + L * (cy + L * cz)) + 4 * (f ^ nu) + nu;
 #pragma unroll
-    for (int s = 0; s < 16; ++s)
+                for (int k = 0; k < NC; ++k) w[k][nu] = sp[k * N + site];
+            }
 #pragma unroll
-        for (int k = 0; k < NC; ++k) Mc[k] += (Acc)sv[k][s];
+            for (int k = 0; k < NC; ++k) w[k][0] = u[k][0];
+        }
+        if (sizeof(T) == 8) {
 #pragma unroll
-    for (int f = 0; f < 4; ++f) {
+            for (int k = 0; k < 6; ++k)
+#pragma unroll
+                for (int q = 0; q < NC; ++q) {
+                    acc[0] = fma((double)u[q][pair_a(k)], (double)u[q][pair_b(k)], acc[0]);
+                    acc[0] = fma((double)w[q][pair_a(k)], (double)w[q][pair_b(k)], acc[0]);
+                }
+#pragma unroll
+            for (int k = 0; k < NC; ++k)
+                acc[1 + k] += ((double)u[k][0] + (double)u[k][1]) + ((double)u[k][2] + (double)u[k][3]);
+            continue;
+        }
+        T v[6];
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
             const int va = pair_a(k), vb = pair_b(k);
-            T du = sv[0][4 * f + va] * sv[0][4 * f + vb];
+            T du = u[0][va] * u[0][vb];
 #pragma unroll
-            for (int q = 1; q < NC; ++q) du += sv[q][4 * f + va] * sv[q][4 * f + vb];
-            const int ma = down_mask(f, va), mb = down_mask(f, vb);
-            const int ba = down_bit(f, va), bb = down_bit(f, vb);
-            T xa[3], xb[3];
+            for (int q = 1; q < NC; ++q) du += u[q][va] * u[q][vb];
+            T dd = w[0][va] * w[0][vb];
 #pragma unroll
-            for (int q = 0; q < NC; ++q) {
-                xa[q] = ma == 0 ? sv[q][ba] : sp[q * N + cb[ma] + ba];
-                xb[q] = mb == 0 ? sv[q][bb] : sp[q * N + cb[mb] + bb];
-            }
-            T dd = xa[0] * xb[0];
-#pragma unroll
-            for (int q = 1; q < NC; ++q) dd += xa[q] * xb[q];
-            ec += du + dd;
+            for (int q = 1; q < NC; ++q) dd += w[q][va] * w[q][vb];
+            v[k] = du + dd;
         }
-    }
-    double tot[4] = {0.0, 0.0, 0.0, 0.0};  // a cell past the lattice adds nothing
-    if (c.valid) {
-        tot[0] = (double)ec;
+        T ec = (T)0, Mc[3] = {(T)0, (T)0, (T)0};
 #pragma unroll
-        for (int k = 0; k < 3; ++k) tot[1 + k] = (double)Mc[k];
+        for (int st = 0; st < 4; ++st) {
+            if (f == st) {
+#pragma unroll
+                for (int k = 0; k < 6; ++k) ec += v[k];
+#pragma unroll
+                for (int k = 0; k < NC; ++k)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) Mc[k] += u[k][q];
+            }
+            ec = __shfl_sync(lanes, ec, st, 4);
+#pragma unroll
+            for (int k = 0; k < NC; ++k) Mc[k] = __shfl_sync(lanes, Mc[k], st, 4);
+        }
+        // (a cell past the lattice has zeros)
+        acc[0] += (double)(f == 0 ? Mc[0] : f == 1 ? Mc[1] : f == 2 ? Mc[2] : ec);
     }
-    tile_sum4_f64(tot, c.nt, scratch);
-    const double se = tot[0], s0 = tot[1], s1 = tot[2], s2 = tot[3];
+    const int per = sizeof(T) == 8 ? (int)blockDim.x : (int)blockDim.x >> 2;
+    if (sizeof(T) == 8) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) scratch[q * per + threadIdx.x] = acc[q];
+    } else {
+        scratch[((f + 1) & 3) * per + (threadIdx.x >> 2)] = acc[0];
+    }
+    __syncthreads();
+    double tot[4];
+    tile_sum4_f64(tot, per, scratch);
     if (threadIdx.x == 0) {
         double *o = B.partials + 4 * (int64_t)blockIdx.x;
-        o[0] = se;
-        o[1] = s0;
-        o[2] = s1;
-        o[3] = s2;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) o[q] = tot[q];
     }
 }
 
@@ -407,14 +560,19 @@ size_t vec_local_smem(const TileShape &t)
     return vec_stage_shared(t.TX, t.TY, t.TZ) ? core : core + vec_stage_bytes(t.TX, t.TY, t.TZ);
 }
 
-static size_t vec_measure_smem(const TileShape &t) { return (size_t)4 * t.TX * t.TY * t.TZ * sizeof(double); }
+// FP32: per cell its first site and flip mask; FP64: the flipped sites' list;
+// then the flip stage's own words.
+static size_t vec_flip_smem(const TileShape &t, size_t es)
+{
+    return (es == 8 ? (size_t)64 : (size_t)8) * t.TX * t.TY * t.TZ + resolve_smem(t);
+}
 
 template <int NC, typename T>
 struct VecOps {
     static cudaError_t prepare(const TileShape &t)
     {
         cudaError_t e = allow_dynamic_smem(vec_local_kernel<NC, T>, vec_local_smem(t));
-        if (e == cudaSuccess) e = allow_dynamic_smem(vec_flip_kernel<NC, T>, resolve_smem(t));
+        if (e == cudaSuccess) e = allow_dynamic_smem(vec_flip_kernel<NC, T>, vec_flip_smem(t, sizeof(T)));
         return e;
     }
     static void init(const Batch &B, int64_t nblocks, int random, cudaStream_t s)
@@ -427,12 +585,12 @@ struct VecOps {
         const int nt = B.TX * B.TY * B.TZ;
         if (p == 0) vec_local_kernel<NC, T><<<(unsigned)ntiles, nt, vec_local_smem(t), s>>>(B);
         else if (p == 1) launch_boundary(B, ntiles, s);
-        else vec_flip_kernel<NC, T><<<(unsigned)ntiles, nt, resolve_smem(t), s>>>(B);
+        else vec_flip_kernel<NC, T><<<(unsigned)ntiles, nt, vec_flip_smem(t, sizeof(T)), s>>>(B);
     }
     static void measure(const Batch &B, int64_t ntiles, cudaStream_t s)
     {
-        const TileShape t{B.TX, B.TY, B.TZ};
-        vec_measure_kernel<NC, T><<<(unsigned)ntiles, B.TX * B.TY * B.TZ, vec_measure_smem(t), s>>>(B);
+        const int threads = std::min(VEC_MEASURE_BLOCK, 4 * B.TX * B.TY * B.TZ);
+        vec_measure_kernel<NC, T><<<(unsigned)ntiles, threads, threads * sizeof(double) * (sizeof(T) == 8 ? 4 : 1), s>>>(B);
     }
 };
 
