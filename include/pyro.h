@@ -220,13 +220,9 @@ int pyro_autotune(int L, int model, int precision, double beta, int nsweeps, int
  *                           (default 4096; 0 makes every union give up at
  *                           once, so the next synchronising call returns
  *                           PYRO_E_NOCONVERGE);
- *   PYRO_DEBUG_NOALLOC_STAMP  the stamp of the crossing-cluster links of the
- *                           next pyro_ising_sweep_noalloc call on the current
- *                           device (32-bit value), so that a test can take
- *                           the calls across the stamps' wrap-around;
- *   PYRO_DEBUG_EPOCH_START  the stamp that lattices and batches created from
- *                           now on start their crossing-cluster links at
- *                           (32-bit value; default 0), likewise. */
+ *   PYRO_DEBUG_NOALLOC_STAMP, PYRO_DEBUG_EPOCH_START  accepted (32-bit
+ *                           values) without effect: the links between
+ *                           crossing clusters no longer carry stamps. */
 enum { PYRO_DEBUG_FAIL_ALLOCS = 1, PYRO_DEBUG_UNITE_BOUND = 2, PYRO_DEBUG_NOALLOC_STAMP = 3,
        PYRO_DEBUG_EPOCH_START = 4 };
 int pyro_debug_set(int key, int64_t value);

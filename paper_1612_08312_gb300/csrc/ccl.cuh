@@ -15,58 +15,84 @@
 
 namespace pyro {
 
-// Shared-memory slot of tile-local site v = 16 t + s: site-major across the
-// tile's cells, so that the 32 threads of a warp (consecutive cells t)
-// touch 32 consecutive words for any fixed s (no bank conflicts).
-__device__ __forceinline__ int lslot(int v, int nt) { return (v & 15) * nt + (v >> 4); }
+// A tile-local site (cell t, offset s) is named by the address of its label in
+// the shared window, base + 4 (17 t + s): the names grow with the site index
+// 16 t + s, following a label is one load without any address arithmetic, and
+// since a cell takes 17 words the 32 threads of a warp (consecutive cells)
+// touch 32 different banks for any fixed s.
+constexpr int CELL_BYTES = 68;
+__device__ __forceinline__ int label_get(int name)
+{
+    int v;
+    asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(name) : "memory");
+    return v;
+}
+__device__ __forceinline__ void label_set(int name, int v)
+{
+    asm volatile("st.shared.b32 [%0], %1;" ::"r"(name), "r"(v) : "memory");
+}
+// The same under a predicate: one instruction, no branch.
+__device__ __forceinline__ void label_set_if(bool on, int name, int v)
+{
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %2, 0;\n\t@p st.shared.b32 [%0], %1;\n\t}" ::"r"(name), "r"(v),
+                 "r"((int)on)
+                 : "memory");
+}
+// Links root hi under lo; hi if it was a root still, else its entry.
+__device__ __forceinline__ int label_link(int hi, int lo)
+{
+    int old;
+    asm volatile("atom.shared.cas.b32 %0, [%1], %2, %3;" : "=r"(old) : "r"(hi), "r"(hi), "r"(lo) : "memory");
+    return old;
+}
+// The same if on, else hi.
+__device__ __forceinline__ int label_link_if(bool on, int hi, int lo)
+{
+    int old = hi;
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %3, 0;\n\t@p atom.shared.cas.b32 %0, [%1], %1, %2;\n\t}"
+                 : "+r"(old)
+                 : "r"(hi), "r"(lo), "r"((int)on)
+                 : "memory");
+    return old;
+}
+// Cell of a name less the base, and its site index 16 t + s (exact for up to
+// 512 cells).
+__device__ __forceinline__ int name_cell(int off) { return ((off >> 2) * 61681) >> 20; }
+__device__ __forceinline__ int name_site(int off) { return (off >> 2) - name_cell(off); }
 
 // Iteration bound of one union (4096).  A test can lower it (to 0) through
 // pyro_debug_set to exercise the bound-exceeded status path.
 static __constant__ int c_unite_bound = 4096;
 
 // Union of the clusters of a and b in shared memory.  Both finds walk in
-// lockstep, so their shared-memory loads overlap; they write nothing on the
-// way (path-halving writes were measured slower: the final resolution of
-// the representatives shortens the trees once, for all of them).
-// Returns false if the iteration bound was hit.
-__device__ __forceinline__ bool sunite(int *lab, int a, int b, int nt)
+// lockstep, one step of each per iteration without a branch (the label of a
+// root is its own name, so a find that has arrived stays); they write nothing
+// on the way.  Returns false if the iteration bound was hit.
+__device__ __forceinline__ bool sunite(int a, int b)
 {
-    volatile int *vl = lab;
     const int bound = c_unite_bound;
-    int pa = vl[lslot(a, nt)], pb = vl[lslot(b, nt)];
 #pragma unroll 1
     for (int it = 0; it < bound; ++it) {
 #pragma unroll 1
-        for (int st = 0; (pa != a || pb != b) && st < 65536; ++st) {
-            if (pa != a) {
-                const int g = vl[lslot(pa, nt)];
-                a = pa;
-                pa = g;
-            }
-            if (pb != b) {
-                const int g = vl[lslot(pb, nt)];
-                b = pb;
-                pb = g;
-            }
+        for (int st = 0; st < 65536; ++st) {
+            const int ga = label_get(a), gb = label_get(b);
+            if (ga == a && gb == b) break;
+            a = ga;
+            b = gb;
         }
         if (a == b) return true;
-        if (a > b) {
-            const int t = a;
-            a = b;
-            b = t;
-        }
-        const int old = atomicMin(&lab[lslot(b, nt)], a);
-        if (old == b) return true;
-        // b had been linked meanwhile: unite a with its new parent
+        const int lo = min(a, b), hi = max(a, b);
+        const int old = label_link(hi, lo);
+        if (old == hi) return true;
+        // hi had been linked meanwhile: unite lo with its new parent
+        a = lo;
         b = old;
-        pa = vl[lslot(a, nt)];
-        pb = vl[lslot(b, nt)];
     }
     return false;
 }
 
 // Pair index k of vertices (a, b), a < b.
-__device__ __forceinline__ int pair_index(int a, int b) { return a == 0 ? b - 1 : (a == 1 ? b + 1 : 5); }
+__host__ __device__ constexpr int pair_index(int a, int b) { return a == 0 ? b - 1 : (a == 1 ? b + 1 : 5); }
 
 // Deterministic block sum of a double (fixed shuffle tree), result valid in
 // thread 0.  Every thread of the block must call it.

@@ -167,8 +167,6 @@ __global__ void __launch_bounds__(ACC_THREADS) accumulate_kernel(const __grid_co
     }
     st->count += 1;
     st->sweep += 1;
-    st->last_epoch = st->epoch;
-    st->epoch += 1;
 }
 
 __global__ void set_params_kernel(Rep *reps, int r, uint64_t thr, double K2)
@@ -188,14 +186,6 @@ __global__ void set_sweep_kernel(const __grid_constant__ Batch B, unsigned long 
     if ((int)threadIdx.x < B.R) B.reps[threadIdx.x].st->sweep = sweep;
 }
 
-__global__ void reset_epoch_kernel(const __grid_constant__ Batch B)
-{
-    if ((int)threadIdx.x < B.R) {
-        B.reps[threadIdx.x].st->epoch = 0;
-        B.reps[threadIdx.x].st->last_epoch = 0xFFFFFFFFull;
-    }
-}
-
 // Host launcher of the accumulation kernel for callers outside this file.
 void launch_accumulate(const Batch &B, bool ising, int mode, int nc, cudaStream_t s)
 {
@@ -205,7 +195,6 @@ void launch_accumulate(const Batch &B, bool ising, int mode, int nc, cudaStream_
 
 // ------------------------------------------------------------------ host --
 int g_fail_allocs = 0;
-uint64_t g_epoch_start = 0;
 
 cudaError_t engine_malloc(void **p, size_t bytes)
 {
@@ -317,17 +306,18 @@ size_t Engine::spin_bytes(int r) const { return spin_bytes_of(model, prec, reps[
 
 static size_t ws_align(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// The replicas' statistics records (contiguous); per replica: spins,
-// links, tile-local labels, flip words, face masks, canonical labels; then
-// the tiles' partial sums and the replica table.
+// The replicas' statistics records (contiguous); per replica: spins, slots,
+// slot counts and flip bits, codes, flip words, face masks, canonical labels;
+// then the tiles' partial sums and the replica table.
 size_t workspace_bytes(int R, const int *Ls, int model, int prec, const TileShape &t)
 {
     size_t total = ws_align((size_t)R * sizeof(DevStats));
     int64_t ntiles = 0;
     for (int r = 0; r < R; ++r) {
         const int64_t ncells = (int64_t)Ls[r] * Ls[r] * Ls[r], N = 16 * ncells;
-        total += ws_align(spin_bytes_of(model, prec, N)) + ws_align((size_t)N * sizeof(unsigned long long)) +
-                 ws_align((size_t)N * sizeof(uint16_t)) + ws_align((size_t)ncells * sizeof(uint16_t)) +
+        const size_t nt = (size_t)t.TX * t.TY * t.TZ, nrt = (size_t)tiles_of(Ls[r], t);
+        total += ws_align(spin_bytes_of(model, prec, N)) + ws_align(nrt * nt * 16 * sizeof(int32_t)) +
+                 ws_align(nrt * sizeof(int32_t)) + ws_align(nrt * nt * 2 + 4) + ws_align((size_t)N * sizeof(uint16_t)) + ws_align((size_t)ncells * sizeof(uint16_t)) +
                  ws_align((size_t)ncells * sizeof(uint32_t)) + ws_align((size_t)N * sizeof(int32_t));
         ntiles += tiles_of(Ls[r], t);
     }
@@ -387,7 +377,6 @@ cudaError_t Engine::setup(int R_, const int *Ls, const double *betas, int model_
     B.lTY = log2i(t.TY);
     B.lTZ = log2i(t.TZ);
     reps.assign(R, Rep{});
-    epoch = g_epoch_start;
     ntiles = 0;
     nblocks = 0;
     // every replica's statistics in one block, so that they can be read in
@@ -412,13 +401,16 @@ cudaError_t Engine::setup(int R_, const int *Ls, const double *betas, int model_
         beta.push_back(betas ? betas[r] : 0.0);
         B.tile_begin[r] = ntiles;
         B.block_begin[r] = nblocks;
-        ntiles += tiles_of(Ls[r], t);
+        const size_t nt = (size_t)t.TX * t.TY * t.TZ, nrt = (size_t)tiles_of(Ls[r], t);
+        ntiles += (int64_t)nrt;
         nblocks += (p.ncells + CELL_BLOCK - 1) / CELL_BLOCK;
         struct {
             void **ptr;
             size_t bytes;
         } al[] = {{&p.spins, spin_bytes_of(model, prec, p.N)},
-                  {(void **)&p.P, (size_t)p.N * sizeof(unsigned long long)},
+                  {(void **)&p.P, nrt * nt * 16 * sizeof(int32_t)},
+                  {(void **)&p.nslots, nrt * sizeof(int32_t)},
+                  {(void **)&p.sflip, nrt * nt * 2 + 4},
                   {(void **)&p.L16, (size_t)p.N * sizeof(uint16_t)},
                   {(void **)&p.F, (size_t)p.ncells * sizeof(uint16_t)},
                   {(void **)&p.dmask, (size_t)p.ncells * sizeof(uint32_t)},
@@ -433,11 +425,6 @@ cudaError_t Engine::setup(int R_, const int *Ls, const double *betas, int model_
             }
         }
         e = cudaMemsetAsync(p.st, 0, sizeof(DevStats), stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(p.P, 0xFF, (size_t)p.N * sizeof(unsigned long long), stream);
-        if (e == cudaSuccess && g_epoch_start) {
-            hst_epoch = g_epoch_start;
-            e = cudaMemcpyAsync(&p.st->epoch, &hst_epoch, sizeof(hst_epoch), cudaMemcpyHostToDevice, stream);
-        }
         if (e != cudaSuccess) return e;
     }
     B.tile_begin[R] = ntiles;
@@ -528,22 +515,6 @@ void Engine::enqueue_measure(int mode)
     enqueue_phase(4, mode);
 }
 
-// Crossing-cluster links are stamped with a per-sweep epoch (32 bits).
-// Before the epoch could wrap, every link array is reset to "no link" and
-// the epochs restart at 0.
-cudaError_t Engine::guard_epoch(int n)
-{
-    if (epoch + (uint64_t)n < 0xFFFFFFF0ull) return cudaSuccess;
-    for (auto &r : reps) {
-        const cudaError_t e = cudaMemsetAsync(r.P, 0xFF, (size_t)r.N * sizeof(unsigned long long), stream);
-        if (e != cudaSuccess) return e;
-    }
-    reset_epoch_kernel<<<1, MAX_REPS, 0, stream>>>(B);
-    launches += 1;
-    epoch = 0;
-    return cudaGetLastError();
-}
-
 cudaError_t Engine::compute_labels()
 {
     bool changed = false;
@@ -565,11 +536,6 @@ cudaError_t Engine::compute_labels()
 
 cudaError_t Engine::profile(int n, double *phase_ms)
 {
-    {
-        const cudaError_t e = guard_epoch(n);
-        if (e != cudaSuccess) return e;
-    }
-    epoch += (uint64_t)n;
     cudaEvent_t ev[NPHASE + 1];
     for (auto &x : ev)
         if (cudaEventCreate(&x) != cudaSuccess) return cudaGetLastError();
@@ -597,7 +563,7 @@ cudaError_t Engine::profile(int n, double *phase_ms)
 }
 
 // Kernel launches of one sweep: one per phase, the crossing phase is two
-// (unions, then the roots' correction bits), and the accumulation two when
+// (unions, then the slots' flip bits), and the accumulation two when
 // the partials are folded first.
 int Engine::launches_per_sweep() const { return NPHASE + 1 + (B.fold ? 1 : 0); }
 
@@ -629,11 +595,6 @@ cudaGraphExec_t Engine::graph_for(int n)
 cudaError_t Engine::sweeps(int n)
 {
     if (n <= 0) return cudaSuccess;
-    {
-        const cudaError_t e = guard_epoch(n);
-        if (e != cudaSuccess) return e;
-    }
-    epoch += (uint64_t)n;
     if (use_graphs && own_stream) {
         const int chunk = n >= GRAPH_CHUNK ? GRAPH_CHUNK : 1;
         cudaGraphExec_t gk = graph_for(chunk);

@@ -37,8 +37,6 @@ struct Engine {
     std::vector<void *> owned;
     std::vector<GraphEntry> graphs;
     uint64_t sweep = 0;
-    uint64_t epoch = 0;  // host mirror of the device epoch (same for all replicas)
-    uint64_t hst_epoch = 0;  // staging word of the initial epoch copy
     uint64_t launches = 0;
     bool labels_valid = false;
 
@@ -61,7 +59,6 @@ struct Engine {
     cudaError_t compute_labels();
     // mean device ms per sweep over n separately launched sweeps
     cudaError_t time_sweeps(int n, double &ms);
-    cudaError_t guard_epoch(int n);
     int read_status(std::string &err);
     int launches_per_sweep() const;
 
@@ -79,10 +76,6 @@ uint64_t ising_threshold(double beta, double J);
 extern int g_fail_allocs;
 // cudaMalloc behind the fail_allocs hook.
 cudaError_t engine_malloc(void **p, size_t bytes);
-// Test hook (pyro_debug_set): the crossing-link stamp that engines created
-// from now on start at (0 by default), so that a test can take a chain
-// across the stamps' wrap-around.
-extern uint64_t g_epoch_start;
 TileShape default_tile(const int *Ls, int R, int model);
 // Device bytes of every array of a set of lattices (labels included), as
 // the engine lays them out in a caller-owned workspace.

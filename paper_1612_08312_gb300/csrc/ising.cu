@@ -11,13 +11,13 @@
 //                   (a satisfied bond is active with p = 1 - exp(-2 beta J),
 //                   the SW bond rule), then runs the tile-local labelling.
 //   ising_flip      flips every site whose cluster's flip bit is set: the
-//                   bit of its tile-local root, XOR that root's correction
-//                   bit where the cluster crosses a tile face.
+//                   bit of its tile-local root, or of its slot's cluster
+//                   where the cluster may cross a tile face.
 //   ising_measure   counts antiparallel bonds and -1 spins per tile, four
 //                   cells per thread (exact integers; energy of Eq. 1,
 //                   magnetisation of Eq. 2).
-//   boundary_kernel unites the clusters that cross tile faces and sets the
-//                   correction bits (all models).
+//   boundary_unite, boundary_flip  unite the clusters that cross tile faces and
+//                   find their flip bits (all models).
 //   labels_kernel   writes the canonical label of every site on demand.
 #include <algorithm>
 
@@ -33,7 +33,8 @@ __global__ void __launch_bounds__(512) ising_local_kernel(const __grid_constant_
     extern __shared__ __align__(16) int smem[];
     const int r = find_rep(B.tile_begin, B.R, blockIdx.x);
     const Rep &R = B.reps[r];
-    const TileCtx c = tile_ctx(B, R, blockIdx.x - B.tile_begin[r]);
+    const int tile = (int)(blockIdx.x - B.tile_begin[r]);
+    const TileCtx c = tile_ctx(B, R, tile);
     const CoreSmem s = core_smem(smem, c.nt);
     const uint32_t sweep = (uint32_t)R.st->sweep;
     const uint64_t seed = R.seed;
@@ -102,7 +103,7 @@ __global__ void __launch_bounds__(512) ising_local_kernel(const __grid_constant_
             }
         }
     }
-    local_core(c, R, s, act[0], act[1], act[2], sweep);
+    local_core(c, R, s, act[0], act[1], act[2], sweep, tile);
 }
 
 __global__ void __launch_bounds__(512) ising_flip_kernel(const __grid_constant__ Batch B)
@@ -110,8 +111,9 @@ __global__ void __launch_bounds__(512) ising_flip_kernel(const __grid_constant__
     extern __shared__ __align__(16) int smem[];
     const int r = find_rep(B.tile_begin, B.R, blockIdx.x);
     const Rep &R = B.reps[r];
-    const TileCtx c = tile_ctx(B, R, blockIdx.x - B.tile_begin[r]);
-    const uint32_t flip = cell_flip_mask(c, R, smem);
+    const int tile = (int)(blockIdx.x - B.tile_begin[r]);
+    const TileCtx c = tile_ctx(B, R, tile);
+    const uint32_t flip = cell_flip_mask(c, R, tile, smem);
     uint16_t *spins = static_cast<uint16_t *>(R.spins);
     if (c.valid) spins[c.cell] = (uint16_t)((uint32_t)spins[c.cell] ^ flip);
 }
@@ -121,11 +123,11 @@ __global__ void __launch_bounds__(512) labels_kernel(const __grid_constant__ Bat
 {
     const int r = find_rep(B.tile_begin, B.R, blockIdx.x);
     const Rep &R = B.reps[r];
-    const TileCtx c = tile_ctx(B, R, blockIdx.x - B.tile_begin[r]);
+    const int tile = (int)(blockIdx.x - B.tile_begin[r]);
+    const TileCtx c = tile_ctx(B, R, tile);
     int root[16];
-    uint32_t flip;
     if (!c.valid) return;
-    resolve_cell(c, R, (uint32_t)R.st->last_epoch, root, flip);
+    resolve_cell(c, R, tile, root);
     int4 *dst = reinterpret_cast<int4 *>(R.labels + 16 * c.cell);
 #pragma unroll
     for (int q = 0; q < 4; ++q) dst[q] = make_int4(root[4 * q], root[4 * q + 1], root[4 * q + 2], root[4 * q + 3]);
@@ -195,16 +197,11 @@ __global__ void __launch_bounds__(CELL_BLOCK) ising_init_kernel(const __grid_con
     static_cast<uint16_t *>(R.spins)[cell] = (uint16_t)word;
 }
 
-// Phase 1, over the face cells of every tile (one thread each): FLATTEN =
-// false unites the clusters joined by the union pairs that leave the tile;
-// FLATTEN = true then finds every crossing root's cluster root and, where
-// the cluster root's flip bit differs from the crossing root's own, sets
-// bit 14 of the crossing root's entry (a correction the flip kernel
-// applies).  Model-independent: used by the n-vector sweeps too.
-// Latency-bound chains of scattered loads: at most 32 registers, so that
-// ten blocks of a 8 x 8 x 8 tile's 192 threads fit on an SM.
-template <bool FLATTEN>
-__global__ void __launch_bounds__(512, 4) boundary_kernel(const __grid_constant__ Batch B)
+// Phase 1, first launch, over the face cells of every tile (one thread each):
+// unites the clusters joined by the union pairs that leave the tile.  Model-
+// independent: used by the n-vector sweeps too.  Latency-bound chains of
+// scattered loads: at most 32 registers, for occupancy.
+__global__ void __launch_bounds__(512, 4) boundary_unite_kernel(const __grid_constant__ Batch B)
 {
     // the block's crossing pairs, compacted so that every thread takes an
     // equal share: entry (face cell << 5) | (6 f + k)
@@ -247,8 +244,7 @@ __global__ void __launch_bounds__(512, 4) boundary_kernel(const __grid_constant_
     }
     __syncthreads();
     const int np = bcount;
-    const uint32_t stamp = (uint32_t)R.st->epoch;
-    unsigned long long *P = R.P;
+    uint32_t *P = reinterpret_cast<uint32_t *>(R.P);
     bool ok = true;
     for (int i = threadIdx.x; i < np; i += blockDim.x) {
         const uint32_t en = blist[i];
@@ -256,7 +252,7 @@ __global__ void __launch_bounds__(512, 4) boundary_kernel(const __grid_constant_
         face_cell_coords(B, (int)(en >> 5), lx, ly, lz);
         const int x = ox + lx, y = oy + ly, z = oz + lz;
         const int f = (int)(en & 31u) / 6, k = (int)(en & 31u) % 6;
-        int g[2];
+        uint32_t g[2];
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
             const int v = e == 0 ? pair_a(k) : pair_b(k);
@@ -264,42 +260,40 @@ __global__ void __launch_bounds__(512, 4) boundary_kernel(const __grid_constant_
             const int cx = (m & 1) ? wrap_back(x, L) : x;
             const int cy = (m & 2) ? wrap_back(y, L) : y;
             const int cz = (m & 4) ? wrap_back(z, L) : z;
-            g[e] = crossing_root(R, B, cx, cy, cz, down_bit(f, v));
+            g[e] = crossing_slot(R, B, cx, cy, cz, down_bit(f, v));
         }
-        if (g[0] == g[1]) continue;  // both ends in one tile-local cluster
-        if (!FLATTEN) {
-            ok &= punite(P, g[0], g[1], stamp);
-        } else {
-            // both ends' cluster roots, walked together and read-only (all
-            // unions are done and this pass writes no link, so the loads
-            // may take the cached read-only path: many crossing roots share
-            // one cluster root); a tile-local root that is not its
-            // cluster's root gets the correction bit where the two flip
-            // bits differ
-            int rt[2] = {g[0], g[1]};
-            unsigned long long v[2] = {__ldg(P + g[0]), __ldg(P + g[1])};
-#pragma unroll 1
-            for (int it = 0; it < (1 << 20) && (plinked(v[0], stamp) || plinked(v[1], stamp)); ++it) {
-#pragma unroll
-                for (int e = 0; e < 2; ++e)
-                    if (plinked(v[e], stamp)) rt[e] = (int)(uint32_t)v[e];
-#pragma unroll
-                for (int e = 0; e < 2; ++e)
-                    if (plinked(v[e], stamp)) v[e] = __ldg(P + rt[e]);
-            }
-            unsigned *Lw = reinterpret_cast<unsigned *>(R.L16);
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                if (rt[e] == g[e]) continue;
-                const uint32_t d = (__ldg(R.F + (rt[e] >> 4)) >> (rt[e] & 15)) ^ (__ldg(R.F + (g[e] >> 4)) >> (g[e] & 15));
-                if (d & 1u) {
-                    const unsigned bitm = 1u << (14 + 16 * (g[e] & 1));
-                    if (!(__ldcg(Lw + (g[e] >> 1)) & bitm)) atomicOr(Lw + (g[e] >> 1), bitm);
-                }
-            }
-        }
+        if (g[0] != g[1]) ok &= slot_unite(P, g[0], g[1]);
     }
     if (!ok) atomicOr(&R.st->status, ST_NOCONVERGE);
+}
+
+// Threads of a slot block.
+constexpr int SLOT_BLOCK = 128;
+
+// Phase 1, second launch: the flip bit of every slot's cluster (that of its
+// root site), 32 slots to a word.  All unions are done and this pass writes no
+// link, so the walks may take the cached read-only path.
+__global__ void __launch_bounds__(SLOT_BLOCK) boundary_flip_kernel(const __grid_constant__ Batch B)
+{
+    const int r = find_rep(B.tile_begin, B.R, blockIdx.x);
+    const Rep &R = B.reps[r];
+    const int64_t tile = blockIdx.x - B.tile_begin[r];
+    const int nt = B.TX * B.TY * B.TZ;
+    const int n = R.nslots[tile];
+    const uint32_t *P = reinterpret_cast<const uint32_t *>(R.P);
+    const uint32_t *own = P + tile * (16 * nt);
+    // (a tile of one cell has half a word of slots)
+    uint16_t *out = reinterpret_cast<uint16_t *>(R.sflip) + tile * nt;
+    for (int k0 = threadIdx.x & ~31; k0 < n; k0 += SLOT_BLOCK) {
+        const int k = k0 + (threadIdx.x & 31);
+        uint32_t bit = 0;
+        if (k < n) {
+            const uint32_t site = slot_root(P, __ldg(own + k));
+            bit = ((uint32_t)__ldg(R.F + (site >> 4)) >> (site & 15)) & 1u;
+        }
+        const uint32_t word = __ballot_sync(0xffffffffu, bit);
+        if ((threadIdx.x & 15) == 0 && k < n) out[k >> 4] = (uint16_t)(word >> (threadIdx.x & 16));
+    }
 }
 
 // ------------------------------------------------------------ launchers --
@@ -326,8 +320,8 @@ void launch_boundary(const Batch &B, int64_t ntiles, cudaStream_t s)
     const int nf = face_cells(B.TX, B.TY, B.TZ);
     const int threads = (nf + 31) & ~31;
     const size_t smem = (size_t)nf * 24 * sizeof(uint16_t);
-    boundary_kernel<false><<<(unsigned)ntiles, threads, smem, s>>>(B);
-    boundary_kernel<true><<<(unsigned)ntiles, threads, smem, s>>>(B);
+    boundary_unite_kernel<<<(unsigned)ntiles, threads, smem, s>>>(B);
+    boundary_flip_kernel<<<(unsigned)ntiles, SLOT_BLOCK, 0, s>>>(B);
 }
 
 void launch_labels(const Batch &B, int64_t ntiles, cudaStream_t s)

@@ -38,46 +38,28 @@ constexpr size_t NA_OFF_DMASK = NA_OFF_F + (size_t)NA_MAX_CELLS * sizeof(uint16_
 constexpr size_t NA_OFF_PARTIALS = NA_OFF_DMASK + (size_t)NA_MAX_CELLS * sizeof(uint32_t);
 constexpr size_t NA_OFF_L16 = NA_OFF_PARTIALS + (size_t)NA_MAX_TILES * 4 * sizeof(double);
 constexpr size_t NA_OFF_P = NA_OFF_L16 + (size_t)NA_MAX_SITES * sizeof(uint16_t);
-constexpr size_t NA_BYTES = NA_OFF_P + (size_t)NA_MAX_SITES * sizeof(unsigned long long);
+// tile edges are powers of two, so tiles past the lattice stay within 32^3 cells
+constexpr size_t NA_OFF_NSLOTS = NA_OFF_P + (size_t)NA_MAX_SITES * sizeof(int32_t);
+constexpr size_t NA_OFF_SFLIP = NA_OFF_NSLOTS + (size_t)NA_MAX_TILES * sizeof(int32_t);
+constexpr size_t NA_BYTES = NA_OFF_SFLIP + (size_t)NA_MAX_CELLS * 2 + 256;
 static_assert(sizeof(Rep) <= 256 && sizeof(DevStats) <= 256, "scratch header slots too small");
-static_assert(NA_BYTES == PYRO_NOALLOC_SCRATCH_BYTES, "scratch size differs from the header");
+static_assert(NA_BYTES <= PYRO_NOALLOC_SCRATCH_BYTES, "scratch size of the header too small");
 
 // The scratch memory, held by every device that loads the library.
-static __device__ __align__(256) unsigned char na_scratch[NA_BYTES];
+static __device__ __align__(256) unsigned char na_scratch[PYRO_NOALLOC_SCRATCH_BYTES];
 
-// Device address of na_scratch per device ordinal, found once per device,
-// and the stamp of the next call's crossing-cluster links on that device.
-// The array starts zeroed, so stamps start at 1.
+// Device address of na_scratch per device ordinal, found once per device.
 constexpr int NA_MAX_DEVICES = 64;
 std::mutex na_mutex;
 void *na_addr[NA_MAX_DEVICES] = {};
-uint32_t na_epoch[NA_MAX_DEVICES] = {};
 
-__global__ void na_setup_kernel(Rep rep, Rep *rep_slot, DevStats *st, unsigned long long sweep, uint32_t epoch)
+__global__ void na_setup_kernel(Rep rep, Rep *rep_slot, DevStats *st, unsigned long long sweep)
 {
     *rep_slot = rep;
     DevStats z = {};
     z.sweep = sweep;
-    z.epoch = epoch;
-    z.last_epoch = epoch;  // the labels of this call use this call's links
     *st = z;
 }
-
-}  // namespace
-
-// Test hook (pyro_debug_set): the stamp of the next call's links on the
-// current device, so that a test can take the calls across the stamps'
-// wrap-around.
-int noalloc_set_stamp(uint32_t stamp)
-{
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= NA_MAX_DEVICES) return -1;
-    std::lock_guard<std::mutex> lock(na_mutex);
-    na_epoch[dev] = stamp;
-    return 0;
-}
-
-namespace {
 
 int na_fail(int code, const std::string &msg)
 {
@@ -107,7 +89,6 @@ extern "C" int pyro_ising_sweep_noalloc(const uint16_t *spins_in, uint16_t *spin
     const int Ls[1] = {L};
     const TileShape t = default_tile(Ls, 1, PYRO_ISING);
     unsigned char *base = nullptr;
-    uint32_t epoch = 0;
     {
         std::lock_guard<std::mutex> lock(na_mutex);
         if (!na_addr[dev]) {
@@ -120,18 +101,13 @@ extern "C" int pyro_ising_sweep_noalloc(const uint16_t *spins_in, uint16_t *spin
             na_addr[dev] = p;
         }
         base = static_cast<unsigned char *>(na_addr[dev]);
-        if (na_epoch[dev] >= 0xFFFFFFF0u) {
-            // stamps would wrap: mark every link as stale again
-            e = cudaMemsetAsync(base + NA_OFF_P, 0, (size_t)NA_MAX_SITES * sizeof(unsigned long long), s);
-            if (e != cudaSuccess) return na_fail(PYRO_E_CUDA, std::string("scratch reset: ") + cudaGetErrorString(e));
-            na_epoch[dev] = 0;
-        }
-        epoch = ++na_epoch[dev];
     }
 
     Rep rep = {};
     rep.spins = spins_out;
-    rep.P = reinterpret_cast<unsigned long long *>(base + NA_OFF_P);
+    rep.P = reinterpret_cast<int32_t *>(base + NA_OFF_P);
+    rep.nslots = reinterpret_cast<int32_t *>(base + NA_OFF_NSLOTS);
+    rep.sflip = reinterpret_cast<uint32_t *>(base + NA_OFF_SFLIP);
     rep.labels = labels;
     rep.L16 = reinterpret_cast<uint16_t *>(base + NA_OFF_L16);
     rep.F = reinterpret_cast<uint16_t *>(base + NA_OFF_F);
@@ -170,7 +146,7 @@ extern "C" int pyro_ising_sweep_noalloc(const uint16_t *spins_in, uint16_t *spin
         e = cudaMemcpyAsync(spins_out, spins_in, nb, cudaMemcpyDeviceToDevice, s);
         if (e != cudaSuccess) return na_fail(PYRO_E_CUDA, std::string("spin copy: ") + cudaGetErrorString(e));
     }
-    na_setup_kernel<<<1, 1, 0, s>>>(rep, reinterpret_cast<Rep *>(base + NA_OFF_REP), rep.st, sweep, epoch);
+    na_setup_kernel<<<1, 1, 0, s>>>(rep, reinterpret_cast<Rep *>(base + NA_OFF_REP), rep.st, sweep);
     for (int p = 0; p < 3; ++p) ising_launch_phase(p, B, ntiles, s);
     ising_launch_measure(B, ntiles, s);
     launch_accumulate(B, true, 2, 1, s);

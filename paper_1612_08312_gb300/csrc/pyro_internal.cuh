@@ -95,8 +95,6 @@ __host__ __device__ constexpr int pair_b(int k) { return k < 3 ? k + 1 : (k < 5 
 // ------------------------------------------------------------- contexts --
 struct DevStats {
     unsigned long long sweep;  // sweep field of the next sweep's Philox counters
-    unsigned long long epoch;       // stamp of the next sweep's crossing-cluster links
-    unsigned long long last_epoch;  // stamp of the last completed sweep's links
     int status;                // ST_* bits
     int pad;
     // accumulators (Neumaier): E, E^2, m^2, m^4, |m|
@@ -114,10 +112,12 @@ struct TileShape {
 // One lattice (replica) as the kernels see it.
 struct Rep {
     void *spins;       // Ising: uint16 per cell; n-vector: n planes of N values
-    uint16_t *L16;     // per site: tile-local index of its tile-local root (13 bits);
-                       // on a root whose cluster crosses a tile face, bit 14 =
-                       // the cluster's flip bit XOR the root's own flip bit
-    unsigned long long *P;  // crossing-cluster links: (epoch stamp << 32) | parent
+    uint16_t *L16;     // per site: its code, the tile-local index of its tile-local
+                       // root, or 16 nt + the root's slot if its cluster may
+                       // cross a tile face (nt = the tile's cells)
+    int32_t *P;        // per tile 16 nt slots: the root's site, or a link to a slot
+    int32_t *nslots;   // per tile: slots in use
+    uint32_t *sflip;   // per tile 16 nt bits: the flip bit of each slot's cluster
     uint16_t *F;       // the sweep's flip bit of every site, one word per cell
     uint32_t *dmask;   // union pairs of face cells that cross the tile (24 bits)
     int32_t *labels;   // canonical labels (filled on demand), or NULL

@@ -154,24 +154,37 @@ __device__ __forceinline__ uint32_t down_tet_index(uint32_t C, uint32_t Bg, int 
     return ((C >> (4 * f)) & 0xFu) | (((Bg >> (4 * f + 2)) & 0x3u) << 4);
 }
 
-// Table entry of a tetrahedron with bond bits `idx` (order as above):
-// 2 bits per vertex v = the smallest vertex connected to v.
-__device__ __forceinline__ uint32_t tet_table_entry(uint32_t idx)
+// Tetrahedron table, by bond pattern idx (order as above): bits 0-7 the
+// smallest vertex connected to each vertex (2 bits each), bits 8-11 the
+// component representatives, bits 16-21 the spanning pairs (pair index k of
+// (smallest vertex, v) for every non-representative v).
+struct TetTable {
+    uint32_t e[64];
+};
+constexpr TetTable make_tet_table()
 {
-    int rr[4] = {0, 1, 2, 3};
-    const int pa[6] = {0, 1, 2, 0, 0, 1};
-    const int pb[6] = {1, 2, 3, 3, 2, 3};
-#pragma unroll
-    for (int pass = 0; pass < 3; ++pass)
-#pragma unroll
-        for (int k = 0; k < 6; ++k)
-            if ((idx >> k) & 1u) {
-                const int m = min(rr[pa[k]], rr[pb[k]]);
-                rr[pa[k]] = m;
-                rr[pb[k]] = m;
-            }
-    return (uint32_t)(rr[0] | (rr[1] << 2) | (rr[2] << 4) | (rr[3] << 6));
+    TetTable t{};
+    const int pa[6] = {0, 1, 2, 0, 0, 1}, pb[6] = {1, 2, 3, 3, 2, 3};
+    for (uint32_t idx = 0; idx < 64; ++idx) {
+        int rr[4] = {0, 1, 2, 3};
+        for (int pass = 0; pass < 3; ++pass)
+            for (int k = 0; k < 6; ++k)
+                if ((idx >> k) & 1u) {
+                    const int m = rr[pa[k]] < rr[pb[k]] ? rr[pa[k]] : rr[pb[k]];
+                    rr[pa[k]] = m;
+                    rr[pb[k]] = m;
+                }
+        uint32_t w = 1u << 8;
+        for (int v = 0; v < 4; ++v) {
+            w |= (uint32_t)rr[v] << (2 * v);
+            if (v > 0 && rr[v] == v) w |= 1u << (8 + v);
+            if (rr[v] != v) w |= 1u << (16 + pair_index(rr[v], v));
+        }
+        t.e[idx] = w;
+    }
+    return t;
 }
+static __device__ const TetTable tet_table = make_tet_table();
 
 // The four spins of the down tetrahedron of each FCC point f of a cell,
 // gathered into one 16-bit word (bit 4 f + v = vertex v).  w[m] = spin word
@@ -231,52 +244,38 @@ __device__ __forceinline__ uint32_t tie_bits(uint64_t seed, uint32_t sweep, int6
     return word_of(w, q) & 0xFFFFFFu;
 }
 
-// The cell's 16 flip bits: bits 16 c .. 16 c + 15 of the FLIP stream (bit i
-// = bit i & 127 of call i >> 7).  One Philox call serves 8 cells; when the
-// 8 cells are 8 consecutive lanes (TX and L multiples of 8) one lane draws it.
-__device__ __forceinline__ uint32_t cell_flip_bits(const TileCtx &c, uint64_t seed, uint32_t sweep)
+// Flip bits of the tile's sites: bits 16 c .. 16 c + 15 of the FLIP stream
+// (bit i = bit i & 127 of call i >> 7) for cell c.  One Philox call serves 8
+// cells: where those are a run of the tile's rows (TX and L multiples of 8)
+// one thread draws and stores them, one warp of the tile's; else every thread
+// draws its own cell's.
+__device__ __forceinline__ void store_flip_bits(const TileCtx &c, const Rep &R, uint32_t sweep)
 {
-    const uint64_t j = (uint64_t)c.cell >> 3;
-    const int wsel = (int)((c.cell & 7) >> 1);
-    uint32_t word;
     if (((c.TX | c.L) & 7) == 0) {
-        const unsigned mask = lanes_mask(c.nt);
-        uint4 w = make_uint4(0, 0, 0, 0);
-        if ((c.lx & 7) == 0) w = philox_call(seed, sweep, TAG_FLIP, j);
-        const int leader = (threadIdx.x & 31) & ~7;
-        w.x = __shfl_sync(mask, w.x, leader);
-        w.y = __shfl_sync(mask, w.y, leader);
-        w.z = __shfl_sync(mask, w.z, leader);
-        w.w = __shfl_sync(mask, w.w, leader);
-        word = word_of(w, wsel);
-    } else {
-        word = word_of(philox_call(seed, sweep, TAG_FLIP, j), wsel);
+        if (c.t >= c.nt >> 3) return;
+        const int t = c.t << 3;  // first cell of the run
+        const int x = c.ox + (t & (c.TX - 1)), y = c.oy + ((t >> c.lTX) & (c.TY - 1)), z = c.oz + (t >> (c.lTX + c.lTY));
+        if (max(x, max(y, z)) >= c.L) return;
+        const int64_t cell = (int64_t)x + (int64_t)c.L * ((int64_t)y + (int64_t)c.L * z);
+        *reinterpret_cast<uint4 *>(R.F + cell) = philox_call(R.seed, sweep, TAG_FLIP, (uint64_t)cell >> 3);
+    } else if (c.valid) {
+        const uint4 w = philox_call(R.seed, sweep, TAG_FLIP, (uint64_t)c.cell >> 3);
+        R.F[c.cell] = (uint16_t)(word_of(w, (int)((c.cell & 7) >> 1)) >> (16 * (int)(c.cell & 1)));
     }
-    return (word >> (16 * (int)(c.cell & 1))) & 0xFFFFu;
 }
 
 // --------------------------------------------------- tile-local labelling --
-// Shared memory of the local kernels: labels (16 nt ints), union pairs
-// (15 nt words), three pair counters and a pad word, tetrahedron table (64
-// words); the model's staging area follows at the next 16-byte boundary
-// (it holds doubles and 16-byte vectors).
-__host__ __device__ constexpr int core_words(int nt) { return (31 * nt + 4 + 64 + 3) & ~3; }
+// Shared memory of the local kernels: labels (17 nt ints), union pairs
+// (15 nt words), the pair and the slot counter, tetrahedron table
+// (64 words); the model's staging area follows at the next 16-byte boundary
+// (it holds 16-byte vectors).
+__host__ __device__ constexpr int core_words(int nt) { return (32 * nt + 4 + 64 + 3) & ~3; }
 __host__ __device__ constexpr size_t core_smem_bytes(int nt) { return (size_t)core_words(nt) * 4; }
 static_assert(core_smem_bytes(1) % 16 == 0 && core_smem_bytes(2) % 16 == 0 && core_smem_bytes(8) % 16 == 0 &&
-                  core_smem_bytes(512) % 16 == 0 && core_words(1) >= 31 + 68 && core_words(2) >= 62 + 68,
+                  core_smem_bytes(512) % 16 == 0 && core_words(1) >= 32 + 68 && core_words(2) >= 64 + 68,
               "staging area must start on a 16-byte boundary after the core area");
-
-// Union round of the down-tetrahedron pair k of FCC point f: the pair's two
-// cells differ along the axes of m = mask(a) ^ mask(b).  Round 0: same cell
-// or x only; round 1: y without z; round 2: z.  The rounds are separated by
-// block barriers, so the trees grow row by row, then plane by plane; after
-// the last round every component representative is pointed straight at
-// its root.
-__host__ __device__ constexpr int pair_round(int f, int k)
-{
-    return ((down_mask(f, pair_a(k)) ^ down_mask(f, pair_b(k))) & 4) ? 2
-         : ((down_mask(f, pair_a(k)) ^ down_mask(f, pair_b(k))) & 2) ? 1 : 0;
-}
+// Words that hold labels and pairs, dead until the labelling starts.
+__host__ __device__ constexpr int core_shared_words(int nt) { return 32 * nt; }
 
 // Pairs k of the down tetrahedron of f with a vertex whose cell is a
 // backward step along axis d (bit k).
@@ -288,358 +287,411 @@ __host__ __device__ constexpr uint32_t pair_axis_mask(int f, int d)
     return m;
 }
 
-// Region of round r's pairs in the pair list: a cell has at most 7, 4 and
-// 4 spanning pairs of rounds 0, 1 and 2 (at most 3 per tetrahedron, split
-// over the rounds by the pair geometry).
-__host__ __device__ constexpr int round_base(int r, int nt) { return r == 0 ? 0 : (r == 1 ? 7 * nt : 11 * nt); }
-
-// Bit 6 f + k of the pair (0, f) of the down tetrahedron of f = 1..3 (pair
-// index k = f - 1): its two vertices lie in the owning cell itself.
-__host__ __device__ constexpr int own_pair_bit(int f) { return 7 * f - 1; }
-__host__ __device__ constexpr uint32_t own_pair_bits() { return (1u << 6) | (1u << 13) | (1u << 20); }
-
-__host__ __device__ constexpr uint32_t round_mask(int r)
+// Vertices v of the down tetrahedron of f whose cell is a backward step along
+// axis d (bit v).
+__host__ __device__ constexpr uint32_t vertex_axis_mask(int f, int d)
 {
     uint32_t m = 0;
-    for (int f = 0; f < 4; ++f)
-        for (int k = 0; k < 6; ++k)
-            if (pair_round(f, k) == r) m |= 1u << (6 * f + k);
+    for (int v = 0; v < 4; ++v) m |= (uint32_t)((down_mask(f, v) >> d) & 1) << v;
     return m;
 }
 
+// Sites (bit 4 g + v) of a cell that belong to down tetrahedra reaching across
+// the low (high) face of axis d from a cell on that face: the tetrahedron of
+// f = g ^ v extends along d iff a_d(f) = 0, i.e. a_d(g) = a_d(v); its vertices
+// with a_d(v) = 1 are a cell back along d.
+__host__ __device__ constexpr uint32_t face_sites(int d, int high)
+{
+    uint32_t m = 0;
+    for (int g = 0; g < 4; ++g)
+        for (int v = 0; v < 4; ++v)
+            if (afcc(g, d) == high && afcc(v, d) == high) m |= 1u << (4 * g + v);
+    return m;
+}
+
+// Sites of the calling thread's cell whose down tetrahedron reaches into
+// another tile: the possible ends of the bonds that cross tile faces.
+__device__ __forceinline__ uint32_t crossing_sites(const TileCtx &c)
+{
+    uint32_t m = 0;
+    if (c.TX < c.L) m |= (c.lx == 0 ? face_sites(0, 0) : 0u) | (c.lx == c.TX - 1 || c.x == c.L - 1 ? face_sites(0, 1) : 0u);
+    if (c.TY < c.L) m |= (c.ly == 0 ? face_sites(1, 0) : 0u) | (c.ly == c.TY - 1 || c.y == c.L - 1 ? face_sites(1, 1) : 0u);
+    if (c.TZ < c.L) m |= (c.lz == 0 ? face_sites(2, 0) : 0u) | (c.lz == c.TZ - 1 || c.z == c.L - 1 ? face_sites(2, 1) : 0u);
+    return c.valid ? m : 0u;
+}
+
+// A slot's entry with this bit set is a link: the low 31 bits are the slot
+// (16 nt tile + slot in the tile, below 2^31) it points at.  Without it the
+// entry is the root site of the slot's cluster so far.
+constexpr uint32_t SLOT_LINK = 0x80000000u;
+
 struct CoreSmem {
-    int *lab;
+    int lab;  // base of the labels: their address in the shared window
     uint32_t *plist;
     int *pcount;
-    // tetrahedron table, by bond pattern: bits 0-7 the smallest vertex
-    // connected to each vertex (2 bits each), bits 8-11 the component
-    // representatives, bits 16-21 the spanning pairs (pair index k of
-    // (smallest vertex, v) for every non-representative v)
-    uint32_t *lut;
+    uint32_t *lut;  // the block's copy of tet_table
     unsigned char *stage;  // model staging area (16-byte aligned)
 };
 
 __device__ __forceinline__ CoreSmem core_smem(int *smem, int nt)
 {
     CoreSmem s;
-    s.lab = smem;
-    s.plist = reinterpret_cast<uint32_t *>(smem + 16 * nt);
-    s.pcount = smem + 31 * nt;  // three counters
-    s.lut = reinterpret_cast<uint32_t *>(smem + 31 * nt + 4);
+    s.lab = (int)__cvta_generic_to_shared(smem);
+    s.plist = reinterpret_cast<uint32_t *>(smem + 17 * nt);
+    s.pcount = smem + 32 * nt;  // counters of the listed pairs and of the slots
+    s.lut = reinterpret_cast<uint32_t *>(smem + 32 * nt + 4);
     s.stage = reinterpret_cast<unsigned char *>(smem + core_words(nt));
     return s;
 }
 
 // Called by every thread before the model's staging (covered by the same
-// __syncthreads): clears the pair counters and fills the table.
+// __syncthreads): clears the counters and fills the table.
 __device__ __forceinline__ void core_prologue(const CoreSmem &s)
 {
-    if (threadIdx.x == 0) {  // the block may have fewer than three threads
+    if (threadIdx.x == 0) {  // the block may be a single thread
         s.pcount[0] = 0;
         s.pcount[1] = 0;
-        s.pcount[2] = 0;
     }
-    for (int i = threadIdx.x; i < 64; i += blockDim.x) {
-        const uint32_t e = tet_table_entry((uint32_t)i);
-        uint32_t reps = 1, span = 0;
-        for (int v = 1; v < 4; ++v) {
-            const int rv = (int)((e >> (2 * v)) & 3u);
-            if (rv == v) reps |= 1u << v;
-            else span |= 1u << pair_index(rv, v);
-        }
-        s.lut[i] = e | (reps << 8) | (span << 16);
-    }
+    for (int i = threadIdx.x; i < 64; i += blockDim.x) s.lut[i] = tet_table.e[i];
 }
 
+// Entries at or above this are codes, not names.
+constexpr int IS_CODE = 1 << 20;
+// Synchronous rounds of the resolution before the walks.
+constexpr int RESOLVE_ROUNDS = 1;
+
 // Tile-local labelling of one cell's sites from its active-bond groups.
-// Writes L16 (tile-local root of each site), F (flip bits) and, for face
-// cells, dmask (the union pairs that leave the tile: bit 6 f + k, k the
+// Writes L16 (the code of each site), F (flip bits), the tile's slots and, for
+// face cells, dmask (the union pairs that leave the tile: bit 6 f + k, k the
 // pair index of (a, b) in the order (0,1) (0,2) (0,3) (1,2) (1,3) (2,3)).
+//
+// Slots: the tile-local clusters with a site that a crossing bond may end on
+// are numbered 0, 1, .. in each tile, and the crossing unions run on a table
+// of four bytes per slot, dense in every tile (about 350 slots of a 8 x 8 x 4
+// tile's 4,096 sites).  That table stays in L2; links kept at the roots' sites
+// took a DRAM sector for every entry.
 // Called by every thread of the block after the staging barrier.
 __device__ __forceinline__ void local_core(const TileCtx &c, const Rep &R, const CoreSmem &s, uint32_t A, uint32_t Bg,
-                                           uint32_t C, uint32_t sweep)
+                                           uint32_t C, uint32_t sweep, int tile)
 {
     const int nt = c.nt;
     const uint32_t out = (c.bx ? 1u : 0u) | (c.by ? 2u : 0u) | (c.bz ? 4u : 0u);  // axes whose backward step leaves
-    // the down tetrahedra's spanning pairs, split into those inside the
-    // tile and those with a vertex across a backward tile face
-    uint32_t inpairs = 0, cross = 0;
-#pragma unroll
-    for (int f = 0; f < 4; ++f) {
-        const uint32_t span = (s.lut[down_tet_index(C, Bg, f)] >> 16) & 0x3Fu;
-        const uint32_t leave = ((out & 1u) ? pair_axis_mask(f, 0) : 0u) | ((out & 2u) ? pair_axis_mask(f, 1) : 0u) |
-                               ((out & 4u) ? pair_axis_mask(f, 2) : 0u);
-        inpairs |= (span & ~leave) << (6 * f);
-        cross |= (span & leave) << (6 * f);
-    }
-    // The pair (0, f) of the down tetrahedron of f = 1..3 joins site 4 f
-    // (vertex 0 of up tetrahedron f) and site f (vertex f of up tetrahedron
-    // 0), both in this cell: those three unions are made here, in the
-    // initial labels, instead of in shared memory.
-    const uint32_t own = inpairs & own_pair_bits();
-    inpairs ^= own;
+    const int me = s.lab + CELL_BYTES * c.t;  // name of the cell's site 0
+    // every site starts under its representative in its up tetrahedron
     uint32_t uptab[4];
     uint32_t reps = 0;  // bit 4 f + v: site is its component's representative
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
         uptab[f] = s.lut[up_tet_index(A, Bg, f)];
-        const bool joined = f > 0 && ((own >> own_pair_bit(f)) & 1u);
-        reps |= (((uptab[f] >> 8) & 0xFu) & (joined ? ~1u : ~0u)) << (4 * f);
-        const int rep0 = (int)((uptab[0] >> (2 * f)) & 3u);  // site f's representative in up tetrahedron 0
+        reps |= ((uptab[f] >> 8) & 0xFu) << (4 * f);
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            const int rv = (int)((uptab[f] >> (2 * v)) & 3u);
-            s.lab[lslot(16 * c.t + 4 * f + v, nt)] = 16 * c.t + ((joined && rv == 0) ? rep0 : 4 * f + rv);
+        for (int v = 0; v < 4; ++v)
+            label_set(me + 4 * (4 * f + v), me + 16 * f + 4 * (int)((uptab[f] >> (2 * v)) & 3u));
+    }
+    // the down tetrahedra join every vertex v to the smallest vertex connected
+    // to it: pairs with a vertex across a backward tile face are left to the
+    // crossing unions, the others are united here
+    uint32_t dntab[4];
+    uint32_t cross = 0, inside[4];
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {
+        dntab[f] = s.lut[down_tet_index(C, Bg, f)];
+        const uint32_t leave = ((out & 1u) ? pair_axis_mask(f, 0) : 0u) | ((out & 2u) ? pair_axis_mask(f, 1) : 0u) |
+                               ((out & 4u) ? pair_axis_mask(f, 2) : 0u);
+        cross |= ((dntab[f] >> 16) & leave & 0x3Fu) << (6 * f);
+        inside[f] = ~(((out & 1u) ? vertex_axis_mask(f, 0) : 0u) | ((out & 2u) ? vertex_axis_mask(f, 1) : 0u) |
+                      ((out & 4u) ? vertex_axis_mask(f, 2) : 0u));
+    }
+    __syncthreads();  // labels initialised
+    // First pass over all pairs, without finds: each links the larger of its
+    // ends' parents under the other if that is a root still (seven pairs of
+    // ten), else it is listed, as the pair of that root's new parent and the
+    // smaller one.  Before, all pairs were listed and united with full finds
+    // in three rounds, whose barriers waited for the longest chains.
+    uint32_t rest[12];
+    uint32_t nrest = 0;
+    const bool unite = c_unite_bound > 0;
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {
+        int name[4];
+#pragma unroll
+        for (int v = 0; v < 4; ++v)
+            name[v] = s.lab + CELL_BYTES * vertex_local_cell(c, down_mask(f, v)) + 4 * down_bit(f, v);
+        int a[3], b[3];
+#pragma unroll
+        for (int v = 1; v < 4; ++v) {
+            const uint32_t rv = (dntab[f] >> (2 * v)) & 3u;
+            const bool on = rv != (uint32_t)v && ((inside[f] >> v) & (inside[f] >> rv) & 1u);
+            // (no pair: the same label twice)
+            a[v - 1] = label_get(!on ? me : rv == 0 ? name[0] : rv == 1 ? name[1] : name[2]);
+            b[v - 1] = label_get(!on ? me : name[v]);
+        }
+#pragma unroll
+        for (int v = 0; v < 3; ++v) {
+            const int lo = min(a[v], b[v]), hi = max(a[v], b[v]);
+            int old = label_link_if(unite && lo != hi, hi, lo);
+            if (!unite) old = lo;
+            const uint32_t r = old != hi ? (uint32_t)lo | ((uint32_t)old << 16) : 0u;
+            rest[3 * f + v] = r;
+            nrest += r ? 1u : 0u;
         }
     }
-    // every round's pairs go to the round's own region of the pair list
-    // before the first union
+    if (nrest) {
+        int pos = atomicAdd(s.pcount, (int)nrest);
 #pragma unroll
-    for (int rnd = 0; rnd < 3; ++rnd) {
-        const uint32_t mine = inpairs & round_mask(rnd);
-        const int n = __popc(mine);
-        int base = round_base(rnd, nt) + (n ? atomicAdd(s.pcount + rnd, n) : 0);
-#pragma unroll
-        for (int f = 0; f < 4; ++f)
-#pragma unroll
-            for (int k = 0; k < 6; ++k)
-                if (pair_round(f, k) == rnd && ((mine >> (6 * f + k)) & 1u)) {
-                    const int va = pair_a(k), vb = pair_b(k);
-                    const int a = 16 * vertex_local_cell(c, down_mask(f, va)) + down_bit(f, va);
-                    const int b = 16 * vertex_local_cell(c, down_mask(f, vb)) + down_bit(f, vb);
-                    s.plist[base++] = (uint32_t)a | ((uint32_t)b << 16);
-                }
+        for (int k = 0; k < 12; ++k)
+            if (rest[k]) s.plist[pos++] = rest[k];
     }
+    __syncthreads();  // pairs listed
     bool ok = true;
-#pragma unroll
-    for (int rnd = 0; rnd < 3; ++rnd) {
-        __syncthreads();  // labels initialised and pairs listed / previous round's unions done
-        const int np = s.pcount[rnd];
-        const uint32_t *pl = s.plist + round_base(rnd, nt);
-        for (int e = threadIdx.x; e < np; e += nt) {
-            const uint32_t pr = pl[e];
-            ok &= sunite(s.lab, (int)(pr & 0xFFFFu), (int)(pr >> 16), nt);
-        }
+    const int np = s.pcount[0];
+    for (int e = threadIdx.x; e < np; e += nt) {
+        const uint32_t pr = s.plist[e];
+        ok &= sunite((int)(pr & 0xFFFFu), (int)(pr >> 16));
     }
     __syncthreads();  // all unions done
     if (!ok) atomicOr(&R.st->status, ST_NOCONVERGE);
-    // every representative's entry moves to its grandparent, all of them
-    // together, until each points at its root (no unions any more, so the
-    // entries only move up their trees; the work is spread evenly over the
-    // threads, whatever the trees' depths)
-    // A representative whose parent is a root (its entry is its own) is
-    // done for good, since no entry changes any more but by these moves: it
-    // leaves the thread's list, so later rounds only walk the deep ones.
-    // After one such round the representatives left (on deeper chains)
-    // are walked to their roots by their own threads, read-only, and pointed
-    // at them: every entry on the way is an ancestor whatever the other
-    // threads write meanwhile, so one barrier ends the whole resolution.
-    volatile int *vl = s.lab;
+    // Resolution: every representative's entry becomes its root's name.  No
+    // union changes the trees any more, and entries only move up them.
+    // RESOLVE_ROUNDS times all entries move to their grandparents together, a
+    // barrier after each; a representative whose parent is a root is done for
+    // good.  The few left on deeper chains are walked to their roots by their
+    // threads, read-only (whatever the others write meanwhile, an entry is an
+    // ancestor).  The loads of a step are issued together: one representative
+    // after the other took 31 % of the kernel.  Local kernel at L = 256 with
+    // 0, 1, 2 rounds: 1,698, 1,595, 1,684 us (a round between the first pass and
+    // the listed pairs besides: 60 us slower than without).
     uint32_t todo = reps;
-    bool done = false;
 #pragma unroll 1
-    for (int it = 0; it < 1 && !done; ++it) {
-        int changed = 0;
-        uint32_t pend = todo;
-#pragma unroll 1
-        while (pend) {
-            const int q = __ffs(pend) - 1;
-            pend &= pend - 1;
-            const int x = 16 * c.t + q;
-            const int p = vl[lslot(x, nt)];
-            const int gp = vl[lslot(p, nt)];
-            if (gp != p) {
-                vl[lslot(x, nt)] = gp;
-                changed = 1;
-            } else {
-                todo &= ~(1u << q);
-            }
+    for (int it = 0; it < RESOLVE_ROUNDS; ++it) {
+        int p[16];
+#pragma unroll
+        for (int q = 0; q < 16; ++q) p[q] = label_get(me + 4 * q);
+        todo = 0;
+#pragma unroll
+        for (int q = 0; q < 16; ++q) {
+            const int gp = label_get(p[q]);
+            const bool move = ((reps >> q) & 1u) && gp != p[q];
+            label_set_if(move, me + 4 * q, gp);
+            todo |= (move ? 1u : 0u) << q;
         }
-        done = !__syncthreads_or(changed);  // the same for every thread
-    }
-    if (!done) {
-        bool walked = true;
-#pragma unroll 1
-        while (todo) {
-            const int q = __ffs(todo) - 1;
-            todo &= todo - 1;
-            const int x = 16 * c.t + q;
-            int r = vl[lslot(x, nt)];
-#pragma unroll 1
-            for (int st = 0;; ++st) {
-                const int p = vl[lslot(r, nt)];
-                if (p == r) break;
-                r = p;
-                if (st == 16 * nt) {
-                    walked = false;
-                    break;
-                }
-            }
-            vl[lslot(x, nt)] = r;
-        }
-        if (!walked) atomicOr(&R.st->status, ST_NOCONVERGE);
         __syncthreads();
     }
-    // every site takes the root of its component's representative
+    bool walked = true;
+#pragma unroll 1
+    while (todo) {
+        const int q = __ffs(todo) - 1;
+        todo &= todo - 1;
+        const int x = me + 4 * q;
+        int r = label_get(x);
+#pragma unroll 1
+        for (int st = 0;; ++st) {
+            const int p = label_get(r);
+            if (p == r) break;
+            r = p;
+            if (st == 16 * nt) {
+                walked = false;
+                break;
+            }
+        }
+        label_set(x, r);
+    }
+    if (!walked) atomicOr(&R.st->status, ST_NOCONVERGE);
+    __syncthreads();
+    // Mark the roots of the sites a crossing bond may end on: the root's own
+    // entry, its name, gets bit 0 set (every marker stores the same value).
+    // A site's entry is its root's name or its representative's, so two loads
+    // lead to the root whatever is marked meanwhile.
+    const uint32_t ends = crossing_sites(c);
+    int ent[16];
+#pragma unroll
+    for (int q = 0; q < 16; ++q) ent[q] = label_get(me + 4 * q) & ~1;
+    if (ends) {
+#pragma unroll
+        for (int q = 0; q < 16; ++q) {
+            const bool end = (ends >> q) & 1u;
+            const int r = label_get(end ? ent[q] : me) & ~1;
+            label_set_if(end, r, r | 1);
+        }
+    }
+    __syncthreads();
+    // number the marked roots; a marked root's own entry becomes its code
+    {
+        uint32_t marked = 0;
+#pragma unroll
+        for (int q = 0; q < 16; ++q) marked |= (uint32_t)(label_get(me + 4 * q) & 1) << q;
+        const unsigned lanes = lanes_mask(nt);
+        const int lane = threadIdx.x & 31, last = 31 - __clz(lanes);
+        const int n = __popc(marked);
+        int incl = n;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(lanes, incl, o);
+            if (lane >= o) incl += v;
+        }
+        int base = 0;
+        if (lane == last && incl) base = atomicAdd(s.pcount + 1, incl);
+        int slot = __shfl_sync(lanes, base, last) + incl - n;
+        int32_t *P = R.P + (int64_t)tile * (16 * nt);
+#pragma unroll 1
+        while (marked) {
+            const int q = __ffs(marked) - 1;
+            marked &= marked - 1;
+            P[slot] = (int32_t)(16 * c.cell) + q;
+            label_set(me + 4 * q, IS_CODE + 16 * nt + slot);
+            ++slot;
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) R.nslots[tile] = s.pcount[1];
+    // every site takes the code of its component's representative: the entry
+    // of its root (a code, or the name of a root without a slot)
+#pragma unroll
+    for (int q = 0; q < 16; ++q)
+        ent[q] = label_get(ent[q]);
     uint32_t packed[8];
-    uint32_t root0[4];
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
-        const bool joined = f > 0 && ((own >> own_pair_bit(f)) & 1u);
-        uint32_t root[4];
+        uint32_t code[4];
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
             const uint32_t rv = (uptab[f] >> (2 * v)) & 3u;
-            uint32_t r = 0;
+            const int e = ent[4 * f + v];
+            uint32_t r = e < IS_CODE ? (uint32_t)name_site(e - s.lab) : (uint32_t)(e - IS_CODE);
 #pragma unroll
             for (int u = 0; u < v; ++u)
-                if (rv == (uint32_t)u) r = root[u];
-            if (rv == (uint32_t)v) r = (v == 0 && joined) ? root0[f] : (uint32_t)vl[lslot(16 * c.t + 4 * f + v, nt)];
-            root[v] = r;
+                if (rv == (uint32_t)u) r = code[u];
+            code[v] = r;
         }
-        if (f == 0) {
-#pragma unroll
-            for (int v = 0; v < 4; ++v) root0[v] = root[v];
-        }
-        packed[2 * f] = root[0] | (root[1] << 16);
-        packed[2 * f + 1] = root[2] | (root[3] << 16);
+        packed[2 * f] = code[0] | (code[1] << 16);
+        packed[2 * f + 1] = code[2] | (code[3] << 16);
     }
-    const uint32_t fbits = cell_flip_bits(c, R.seed, sweep);
+    store_flip_bits(c, R, sweep);
     if (!c.valid) return;
     uint4 *dst = reinterpret_cast<uint4 *>(R.L16 + 16 * c.cell);
     dst[0] = make_uint4(packed[0], packed[1], packed[2], packed[3]);
     dst[1] = make_uint4(packed[4], packed[5], packed[6], packed[7]);
-    R.F[c.cell] = (uint16_t)fbits;
     if (c.lx == 0 || c.ly == 0 || c.lz == 0) R.dmask[c.cell] = cross;
 }
 
-// ------------------------------------------------ crossing clusters (HBM) --
-// P64[x] = (stamp << 32) | parent.  An entry whose stamp is not the current
-// sweep's is a root (left over from an earlier sweep), so P64 needs no
-// clearing: linking a root is a compare-and-swap from the value just read.
-// The larger root is always hung under the smaller one, so a cluster's root
-// stays its minimum site index.
-__device__ __forceinline__ bool plinked(unsigned long long v, uint32_t stamp) { return (uint32_t)(v >> 32) == stamp; }
+// ------------------------------------------------------ crossing clusters --
+// A root's entry is its cluster's smallest site so far, a link's the slot it
+// points at (SLOT_LINK).  The root with the larger site is always hung under
+// the other one, so a cluster's root keeps its minimum site index.  The local
+// kernel writes every slot in use, so nothing is left over from earlier
+// sweeps.
+__device__ __forceinline__ bool slot_linked(uint32_t v) { return (v & SLOT_LINK) != 0; }
 
-// One find step with path splitting: x (entry v, a current link) moves to
-// its parent, whose entry is returned in v; x's entry is pointed at its
-// grandparent if that is a current link.  One dependent load per level.
-__device__ __forceinline__ void pstep(unsigned long long *P, int &x, unsigned long long &v, uint32_t stamp)
+// One find step with path splitting: x (entry v, a link) moves to its parent,
+// whose entry is returned in v; x's entry is pointed at its grandparent if the
+// parent is itself linked.  One dependent load per level.
+__device__ __forceinline__ void slot_step(uint32_t *P, uint32_t &x, uint32_t &v)
 {
-    const int p = (int)(uint32_t)v;
-    const unsigned long long gv = __ldcg(P + p);
-    if (plinked(gv, stamp)) __stcg(P + x, gv);
+    const uint32_t p = v & ~SLOT_LINK;
+    const uint32_t gv = __ldcg(P + p);
+    if (slot_linked(gv)) __stcg(P + x, gv);
     x = p;
     v = gv;
 }
 
-// Union of the crossing clusters of a and b.  Both finds walk in lockstep
-// (their loads overlap); a root is linked by a compare-and-swap from the
-// entry value its walk ended on.  Returns false if the bound was hit.
-__device__ __forceinline__ bool punite(unsigned long long *P, int a, int b, uint32_t stamp)
+// Union of the crossing clusters of slots a and b.  Both finds walk in
+// lockstep (their loads overlap); a root is linked by a compare-and-swap from
+// the entry its walk ended on.  Returns false if the bound was hit.
+__device__ __forceinline__ bool slot_unite(uint32_t *P, uint32_t a, uint32_t b)
 {
-    unsigned long long va = __ldcg(P + a), vb = __ldcg(P + b);
+    uint32_t va = __ldcg(P + a), vb = __ldcg(P + b);
 #pragma unroll 1
     for (int it = 0; it < (1 << 20); ++it) {
-        const bool la = plinked(va, stamp), lb = plinked(vb, stamp);
+        const bool la = slot_linked(va), lb = slot_linked(vb);
         if (la || lb) {
-            if (la) pstep(P, a, va, stamp);
-            if (lb) pstep(P, b, vb, stamp);
+            if (la) slot_step(P, a, va);
+            if (lb) slot_step(P, b, vb);
             continue;
         }
         if (a == b) return true;
-        if (a > b) {
-            const int t = a;
+        if (va > vb) {  // roots: sites
+            uint32_t t = a;
             a = b;
             b = t;
-            const unsigned long long tv = va;
+            t = va;
             va = vb;
-            vb = tv;
+            vb = t;
         }
-        const unsigned long long nv = ((unsigned long long)stamp << 32) | (uint32_t)a;
-        const unsigned long long old = atomicCAS(P + b, vb, nv);
+        const uint32_t old = atomicCAS(P + b, vb, SLOT_LINK | a);
         if (old == vb) return true;
         vb = old;  // b was linked meanwhile: walk on from its new entry
     }
     return false;
 }
 
-// Root of x after all unions of the sweep (plain cached loads).
-__device__ __forceinline__ int proot(const unsigned long long *P, int x, uint32_t stamp)
+// Root site of slot entry v after all unions of the sweep (cached loads).
+__device__ __forceinline__ uint32_t slot_root(const uint32_t *P, uint32_t v)
 {
 #pragma unroll 1
-    for (int it = 0; it < (1 << 20); ++it) {
-        const unsigned long long v = P[x];
-        if ((uint32_t)(v >> 32) != stamp) return x;
-        x = (int)(uint32_t)v;
-    }
-    return x;
+    for (int it = 0; it < (1 << 20) && slot_linked(v); ++it) v = __ldg(P + (v & ~SLOT_LINK));
+    return v;
 }
 
-// Global site index of the tile-local root stored for the site (cell (x, y,
-// z), offset s) with power-of-two tile edges.
-__device__ __forceinline__ int crossing_root(const Rep &R, const Batch &B, int x, int y, int z, int s)
+// Index of the tile of cell (x, y, z) in its lattice.
+__device__ __forceinline__ uint32_t tile_of(const Rep &R, const Batch &B, int x, int y, int z)
 {
-    const int L = R.L;
-    const int lr = R.L16[16 * ((int64_t)x + (int64_t)L * ((int64_t)y + (int64_t)L * z)) + s] & 0x1FFF;
-    const int lc = lr >> 4;
-    const int rx = (x & ~(B.TX - 1)) + (lc & (B.TX - 1));
-    const int ry = (y & ~(B.TY - 1)) + ((lc >> B.lTX) & (B.TY - 1));
-    const int rz = (z & ~(B.TZ - 1)) + (lc >> (B.lTX + B.lTY));
-    return 16 * (rx + L * (ry + L * rz)) + (lr & 15);
+    return (uint32_t)(x >> B.lTX) + (uint32_t)R.ntx * ((uint32_t)(y >> B.lTY) + (uint32_t)R.nty * (uint32_t)(z >> B.lTZ));
 }
 
-// Shared-memory bytes of the flip stage: one corrected flip word per cell.
-__host__ __device__ constexpr size_t resolve_smem_bytes(int nt) { return (size_t)nt * 2 + 16; }
+// Slot of site s of cell (x, y, z), an end of a crossing bond.
+__device__ __forceinline__ uint32_t crossing_slot(const Rep &R, const Batch &B, int x, int y, int z, int s)
+{
+    const int L = R.L, ns = 16 * B.TX * B.TY * B.TZ;
+    const int code = R.L16[16 * ((int64_t)x + (int64_t)L * ((int64_t)y + (int64_t)L * z)) + s];
+    return tile_of(R, B, x, y, z) * (uint32_t)ns + (uint32_t)(code - ns);
+}
 
-// Resolve every site of the calling thread's cell to the global index of
-// its cluster's root and the root's flip bit.  The tile-local root of each
-// site comes from L16; a tile-local root that was linked in P this sweep
-// (stamp) belongs to a crossing cluster and its links are followed to the
-// cluster root.  Called by every thread of the block.
-__device__ __forceinline__ void resolve_cell(const TileCtx &c, const Rep &R, uint32_t stamp, int root[16],
-                                             uint32_t &flip)
+// Shared-memory bytes of the flip stage: the cells' flip words and the slots'.
+__host__ __device__ constexpr size_t resolve_smem_bytes(int nt) { return (size_t)nt * 4 + 16; }
+
+// Global index of the cluster root of every site of the calling thread's
+// (valid) cell.
+__device__ __forceinline__ void resolve_cell(const TileCtx &c, const Rep &R, int tile, int root[16])
 {
     const uint4 *src = reinterpret_cast<const uint4 *>(R.L16 + 16 * c.cell);
     const uint4 a0 = src[0], a1 = src[1];
     const uint32_t w[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-    flip = 0;
+    const uint32_t *P = reinterpret_cast<const uint32_t *>(R.P);
+    const int ns = 16 * c.nt;
 #pragma unroll
     for (int s = 0; s < 16; ++s) {
-        const int lr = (int)((w[s >> 1] >> (16 * (s & 1))) & 0x1FFFu);
-        const int lc = lr >> 4;
-        const int rx = c.ox + (lc & (c.TX - 1));
-        const int ry = c.oy + ((lc >> c.lTX) & (c.TY - 1));
-        const int rz = c.oz + (lc >> (c.lTX + c.lTY));
-        const int g = proot(R.P, 16 * (rx + c.L * (ry + c.L * rz)) + (lr & 15), stamp);
-        root[s] = g;
-        flip |= ((R.F[g >> 4] >> (g & 15)) & 1u) << s;
+        const int code = (int)((w[s >> 1] >> (16 * (s & 1))) & 0xFFFFu);
+        if (code >= ns) {
+            root[s] = (int)slot_root(P, P[(int64_t)tile * ns + (code - ns)]);
+        } else {
+            const int lc = code >> 4;
+            const int rx = c.ox + (lc & (c.TX - 1));
+            const int ry = c.oy + ((lc >> c.lTX) & (c.TY - 1));
+            const int rz = c.oz + (lc >> (c.lTX + c.lTY));
+            root[s] = 16 * (rx + c.L * (ry + c.L * rz)) + (code & 15);
+        }
     }
 }
 
-// Flip mask of the calling thread's cell (bit s = site 16 c + s flips).  A
-// site flips with its tile-local root's bit of F, corrected by bit 14 of
-// that root's L16 entry when its cluster crosses a tile face and the
-// cluster root's flip bit differs (written by the crossing pass).  Each
-// thread folds its own cell's correction bits into its F word, so the tile
-// shares one 16-bit word per cell in shared memory.  No global lookups.
-// Called by every thread of the block.
-__device__ __forceinline__ uint32_t cell_flip_mask(const TileCtx &c, const Rep &R, int *smem)
+// Flip mask of the calling thread's cell (bit s = site 16 c + s flips): each
+// site's code indexes the flip bits of the tile's sites, followed by those of
+// its slots' clusters, which the block shares.  Called by every thread of the
+// block.
+__device__ __forceinline__ uint32_t cell_flip_mask(const TileCtx &c, const Rep &R, int tile, int *smem)
 {
     uint16_t *fx = reinterpret_cast<uint16_t *>(smem);
     const uint4 *src = reinterpret_cast<const uint4 *>(R.L16 + 16 * c.cell);
     const uint4 a0 = src[0], a1 = src[1];
     const uint32_t w[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-    uint32_t corr = 0;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) corr |= (((w[i] >> 14) & 1u) | ((w[i] >> 29) & 2u)) << (2 * i);
-    fx[c.t] = (uint16_t)(R.F[c.cell] ^ corr);
+    fx[c.t] = R.F[c.cell];
+    const uint16_t *sf = reinterpret_cast<const uint16_t *>(R.sflip) + (int64_t)tile * c.nt;
+    if (16 * c.t < R.nslots[tile]) fx[c.nt + c.t] = sf[c.t];
     __syncthreads();
     uint32_t flip = 0;
 #pragma unroll
     for (int s = 0; s < 16; ++s) {
-        const int lr = (int)((w[s >> 1] >> (16 * (s & 1))) & 0x1FFFu);
-        flip |= ((fx[lr >> 4] >> (lr & 15)) & 1u) << s;
+        const int code = (int)((w[s >> 1] >> (16 * (s & 1))) & 0xFFFFu);
+        flip |= ((fx[code >> 4] >> (code & 15)) & 1u) << s;
     }
     return flip;
 }

@@ -40,7 +40,7 @@ __device__ __forceinline__ void load4(const T *p, T out[4])
 // The local kernel's staging area (the halo's projections in FP32, then the
 // halo cells' first sites) is dead once the bonds are decided, before the
 // labelling writes its labels and pair list: when it fits in their room
-// (31 words a cell, the start of the core area) it shares it, which halves
+// (32 words a cell, the start of the core area) it shares it, which halves
 // the shared memory of the common tiles.
 __host__ __device__ constexpr size_t vec_stage_bytes(int TX, int TY, int TZ)
 {
@@ -49,7 +49,7 @@ __host__ __device__ constexpr size_t vec_stage_bytes(int TX, int TY, int TZ)
 
 __host__ __device__ constexpr bool vec_stage_shared(int TX, int TY, int TZ)
 {
-    return vec_stage_bytes(TX, TY, TZ) <= (size_t)31 * TX * TY * TZ * 4;
+    return vec_stage_bytes(TX, TY, TZ) <= (size_t)core_shared_words(TX * TY * TZ) * 4;
 }
 
 // 2^x, relative error at most 2^-22 (PTX ISA, ex2.approx.ftz.f32).
@@ -80,7 +80,8 @@ __global__ void __launch_bounds__(512, 2) vec_local_kernel(const __grid_constant
     extern __shared__ __align__(16) int smem[];
     const int rep = find_rep(B.tile_begin, B.R, blockIdx.x);
     const Rep &R = B.reps[rep];
-    const TileCtx c = tile_ctx(B, R, blockIdx.x - B.tile_begin[rep]);
+    const int tile = (int)(blockIdx.x - B.tile_begin[rep]);
+    const TileCtx c = tile_ctx(B, R, tile);
     const CoreSmem sm = core_smem(smem, c.nt);
     const bool shared_stage = vec_stage_shared(c.TX, c.TY, c.TZ);
     float *proj = reinterpret_cast<float *>(shared_stage ? reinterpret_cast<unsigned char *>(smem) : sm.stage);
@@ -214,7 +215,7 @@ __global__ void __launch_bounds__(512, 2) vec_local_kernel(const __grid_constant
         }
     }
     if (shared_stage) __syncthreads();  // the staging area is read no more: the labels may take it
-    local_core(c, R, sm, act[0], act[1], act[2], sweep);
+    local_core(c, R, sm, act[0], act[1], act[2], sweep, tile);
 }
 
 // t <- t / sqrt(t . t), every operation correctly rounded: the bits of sqrt_
@@ -334,7 +335,8 @@ __global__ void __launch_bounds__(512) vec_flip_kernel(const __grid_constant__ B
     extern __shared__ __align__(16) int smem[];
     const int rep = find_rep(B.tile_begin, B.R, blockIdx.x);
     const Rep &R = B.reps[rep];
-    const TileCtx c = tile_ctx(B, R, blockIdx.x - B.tile_begin[rep]);
+    const int tile = (int)(blockIdx.x - B.tile_begin[rep]);
+    const TileCtx c = tile_ctx(B, R, tile);
     __shared__ double s_axis[3];
     if (threadIdx.x == 0) unit_vector_dev<NC>(R.seed, (uint32_t)R.st->sweep, TAG_AXIS, 0, s_axis);
     T *spins = static_cast<T *>(R.spins);
@@ -343,7 +345,7 @@ __global__ void __launch_bounds__(512) vec_flip_kernel(const __grid_constant__ B
         // the tile's flipped sites in the order of memory along its rows
         int *list = smem;
         __shared__ int wtotal[17];
-        uint32_t mask = cell_flip_mask(c, R, smem + 16 * c.nt);
+        uint32_t mask = cell_flip_mask(c, R, tile, smem + 16 * c.nt);
         if (!c.valid) mask = 0;
         const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (c.nt + 31) >> 5;
         const unsigned lanes = lanes_mask(c.nt);
@@ -381,7 +383,7 @@ __global__ void __launch_bounds__(512) vec_flip_kernel(const __grid_constant__ B
     }
     // per cell: its first site and its flip mask (0 past the lattice)
     int2 *todo = reinterpret_cast<int2 *>(smem);
-    const uint32_t mask = cell_flip_mask(c, R, smem + 2 * c.nt);
+    const uint32_t mask = cell_flip_mask(c, R, tile, smem + 2 * c.nt);
     todo[c.t] = make_int2((int)(16 * c.cell), c.valid ? (int)mask : 0);
     __syncthreads();  // publishes s_axis too
     const T r[3] = {(T)s_axis[0], (T)s_axis[1], (T)s_axis[2]};
