@@ -7,6 +7,7 @@
 #include <string>
 
 #include "engine.h"
+#include "nvec.cuh"
 
 namespace pyro {
 
@@ -28,7 +29,7 @@ void vec_launch_measure(int model, int prec, const Batch &B, int64_t ntiles, cud
 constexpr int ACC_THREADS = 128;
 
 // Sums of four values over a block of ACC_THREADS threads in a fixed tree
-// (integers: the first two); results valid in thread 0.
+// (integers: the first two); results valid in the first warp.
 template <typename V, int NV>
 __device__ __forceinline__ void acc_block_sum(V v[NV], V (*red)[ACC_THREADS])
 {
@@ -89,6 +90,18 @@ __global__ void __launch_bounds__(ACC_THREADS) fold_kernel(const __grid_constant
     }
 }
 
+// The n-vector axis of a replica's next sweep, part of its chain's state like
+// the sweep counter: drawn by one thread when the counter moves.  (Every block
+// of the local and the flip kernels drew it before: the FP64 roots and
+// quotients, with a barrier behind them, were 2 to 4 thousand cycles of each.)
+__device__ void draw_axis(const Rep &R, unsigned long long sweep, int nc)
+{
+    double r[3];
+    if (nc == 2) unit_vector_dev<2>(R.seed, (uint32_t)sweep, TAG_AXIS, 0, r);
+    else unit_vector_dev<3>(R.seed, (uint32_t)sweep, TAG_AXIS, 0, r);
+    for (int k = 0; k < 3; ++k) R.st->axis[k] = r[k];
+}
+
 // Per replica (one block each): sum the tiles' partials of the measurement
 // kernel in a fixed order, form E, m = |M|/N, m^2, m^4 (Eq. 1, Eq. 2) and, in
 // mode 1, add them to the Neumaier sums, append the trace record and advance
@@ -107,6 +120,10 @@ __global__ void __launch_bounds__(ACC_THREADS) accumulate_kernel(const __grid_co
     const double *src = B.fold ? B.folded : B.partials;
     const int64_t b0 = B.fold ? (int64_t)r * B.fold : B.tile_begin[r];
     const int64_t b1 = B.fold ? (int64_t)(r + 1) * B.fold : B.tile_begin[r + 1];
+    // the record's fields, read ahead of the sums they are needed after
+    const int t = threadIdx.x;
+    const unsigned long long sweep = st->sweep, count = st->count;
+    double acc_s = t < 5 ? st->acc_s[t] : 0.0, acc_c = t < 5 ? st->acc_c[t] : 0.0;
     double tot[4] = {0.0, 0.0, 0.0, 0.0};
     if (ISING) {
         __shared__ unsigned long long red[2][ACC_THREADS];
@@ -118,13 +135,15 @@ __global__ void __launch_bounds__(ACC_THREADS) accumulate_kernel(const __grid_co
             v[1] += p.y;
         }
         acc_block_sum<unsigned long long, 2>(v, red);
-        if (threadIdx.x != 0) return;
+        if (t >= 32) return;
         const long long anti = (long long)v[0];
         const long long M = R.N - 2 * (long long)v[1];
         tot[0] = (double)(3 * R.N - 2 * anti);  // sum over bonds of s_i s_j
         tot[1] = (double)M;
     } else {
         __shared__ double red[4][ACC_THREADS];
+        // (thread 0 moves the counter after the sums' barriers)
+        if (mode == 1 && threadIdx.x == ACC_THREADS - 1) draw_axis(R, sweep + 1, nc);
 #pragma unroll 4
         for (int64_t b = b0 + threadIdx.x; b < b1; b += ACC_THREADS) {
             const double2 p = *reinterpret_cast<const double2 *>(src + 4 * b);
@@ -135,8 +154,9 @@ __global__ void __launch_bounds__(ACC_THREADS) accumulate_kernel(const __grid_co
             tot[3] += q.y;
         }
         acc_block_sum<double, 4>(tot, red);
-        if (threadIdx.x != 0) return;
+        if (t >= 32) return;
     }
+    // every lane of the first warp forms the observables; lane k < 5 keeps sum k
     const double E = __dmul_rn(-R.J, tot[0]);
     double m;
     if (ISING) {
@@ -148,25 +168,29 @@ __global__ void __launch_bounds__(ACC_THREADS) accumulate_kernel(const __grid_co
     }
     const double m2 = __dmul_rn(m, m);
     const double m4 = __dmul_rn(m2, m2);
-    st->last[0] = E;
-    st->last[1] = m2;
-    st->last[2] = m4;
-    st->last[3] = tot[1];
+    if (t == 0) {
+        st->last[0] = E;
+        st->last[1] = m2;
+        st->last[2] = m4;
+        st->last[3] = tot[1];
+    }
     if (mode != 1) return;
-    nsum_add(st->acc_s[0], st->acc_c[0], E);
-    nsum_add(st->acc_s[1], st->acc_c[1], __dmul_rn(E, E));
-    nsum_add(st->acc_s[2], st->acc_c[2], m2);
-    nsum_add(st->acc_s[3], st->acc_c[3], m4);
-    nsum_add(st->acc_s[4], st->acc_c[4], __dsqrt_rn(m2));
+    if (t < 5) {
+        const double x = t == 0 ? E : t == 1 ? __dmul_rn(E, E) : t == 2 ? m2 : t == 3 ? m4 : __dsqrt_rn(m2);
+        nsum_add(acc_s, acc_c, x);
+        st->acc_s[t] = acc_s;
+        st->acc_c[t] = acc_c;
+    }
+    if (t != 0) return;
     if (R.trace && R.trace_cap > 0) {
-        double *rec = R.trace + 4 * (int64_t)(st->count % (unsigned long long)R.trace_cap);
+        double *rec = R.trace + 4 * (int64_t)(count % (unsigned long long)R.trace_cap);
         rec[0] = E;
         rec[1] = m2;
         rec[2] = m4;
         rec[3] = tot[1];
     }
-    st->count += 1;
-    st->sweep += 1;
+    st->count = count + 1;
+    st->sweep = sweep + 1;
 }
 
 __global__ void set_params_kernel(Rep *reps, int r, uint64_t thr, double K2)
@@ -181,9 +205,11 @@ __global__ void set_trace_kernel(Rep *reps, int r, double *trace, int64_t cap)
     reps[r].trace_cap = cap;
 }
 
-__global__ void set_sweep_kernel(const __grid_constant__ Batch B, unsigned long long sweep)
+__global__ void set_sweep_kernel(const __grid_constant__ Batch B, unsigned long long sweep, int nc)
 {
-    if ((int)threadIdx.x < B.R) B.reps[threadIdx.x].st->sweep = sweep;
+    if ((int)threadIdx.x >= B.R) return;
+    B.reps[threadIdx.x].st->sweep = sweep;
+    if (nc > 1) draw_axis(B.reps[threadIdx.x], sweep, nc);
 }
 
 // Host launcher of the accumulation kernel for callers outside this file.
@@ -451,6 +477,10 @@ cudaError_t Engine::setup(int R_, const int *Ls, const double *betas, int model_
     if (model == PYRO_ISING) ising_launch_init(B, nblocks, start == PYRO_START_RANDOM, stream);
     else vec_launch_init(model, prec, B, nblocks, start == PYRO_START_RANDOM, stream);
     launches += 1;
+    if (model != PYRO_ISING) {  // the first sweep's axis
+        set_sweep_kernel<<<1, MAX_REPS, 0, stream>>>(B, 0, model);
+        launches += 1;
+    }
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
     if (e != cudaSuccess) err = "initial state";
@@ -656,7 +686,7 @@ cudaError_t Engine::measure()
 
 cudaError_t Engine::set_sweep(uint64_t s)
 {
-    set_sweep_kernel<<<1, MAX_REPS, 0, stream>>>(B, s);
+    set_sweep_kernel<<<1, MAX_REPS, 0, stream>>>(B, s, model);
     launches += 1;
     sweep = s;
     return cudaGetLastError();

@@ -103,6 +103,8 @@ struct DevStats {
     unsigned long long count;
     // last measurement: E, m2, m4, M_x
     double last[4];
+    // n-vector: the axis of sweep `sweep`, drawn whenever that counter moves
+    double axis[3];
 };
 
 struct TileShape {

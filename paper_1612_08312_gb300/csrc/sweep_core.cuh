@@ -120,22 +120,6 @@ __device__ __forceinline__ int halo_index(const TileCtx &c, int m)
     return (c.lx + 1 - (m & 1)) + HX * ((c.ly + 1 - ((m >> 1) & 1)) + HY * (c.lz + 1 - ((m >> 2) & 1)));
 }
 
-// Global cell of halo entry h of the tile with origin (ox, oy, oz).
-__device__ __forceinline__ int64_t halo_cell(int h, int TX, int TY, int ox, int oy, int oz, int L)
-{
-    const int HX = TX + 1, HY = TY + 1;
-    const int hx = h % HX, hy = (h / HX) % HY, hz = h / (HX * HY);
-    int gx = ox + hx - 1, gy = oy + hy - 1, gz = oz + hz - 1;
-    gx += (gx < 0) ? L : 0;
-    gy += (gy < 0) ? L : 0;
-    gz += (gz < 0) ? L : 0;
-    // past the lattice (a tile that reaches beyond it): any cell in bounds
-    gx = min(gx, L - 1);
-    gy = min(gy, L - 1);
-    gz = min(gz, L - 1);
-    return (int64_t)gx + (int64_t)L * ((int64_t)gy + (int64_t)L * gz);
-}
-
 // ------------------------------------------------------ bond bit layout --
 // Vertex pair of slot q of group g (see the header comment); up = whether
 // the pair belongs to the up tetrahedron.

@@ -37,14 +37,14 @@ __device__ __forceinline__ void load4(const T *p, T out[4])
     }
 }
 
-// The local kernel's staging area (the halo's projections in FP32, then the
-// halo cells' first sites) is dead once the bonds are decided, before the
-// labelling writes its labels and pair list: when it fits in their room
-// (32 words a cell, the start of the core area) it shares it, which halves
-// the shared memory of the common tiles.
+// The local kernel's staging area (the projections of the tile and its halo,
+// in FP32) is dead once the bonds are decided, before the labelling writes its
+// labels and pair list: when it fits in their room (32 words a cell, the
+// start of the core area) it shares it, which halves the shared memory of the
+// common tiles.
 __host__ __device__ constexpr size_t vec_stage_bytes(int TX, int TY, int TZ)
 {
-    return (size_t)(16 + 1) * halo_cells(TX, TY, TZ) * 4;
+    return (size_t)16 * halo_cells(TX, TY, TZ) * 4;
 }
 
 __host__ __device__ constexpr bool vec_stage_shared(int TX, int TY, int TZ)
@@ -91,41 +91,99 @@ __global__ void __launch_bounds__(512, 2) vec_local_kernel(const __grid_constant
     const uint64_t seed = R.seed;
     core_prologue(sm);
 
-    // the sweep's axis, drawn once per block (FP64 divides and square roots
-    // run at a small fraction of the FP32 rate on this GPU)
-    __shared__ double s_axis[3];
-    if (threadIdx.x == 0) unit_vector_dev<NC>(seed, sweep, TAG_AXIS, 0, s_axis);
-    __syncthreads();
-    const float rf[3] = {(float)s_axis[0], (float)s_axis[1], (float)s_axis[2]};
-
-    // projections s_i . r of the tile's sites and the backward halo, in FP32
+    // Projections s_i . r of the tile's sites and the backward halo, in FP32
     // (for FP64 spins an approximation that the shortcut's margin covers: FP64
-    // arithmetic here cost more than the whole FP32 kernel); each
-    // halo cell's first site is found once (the halo's edges are not powers
-    // of two, so this takes divisions) and shared.  Site-major layout (site s
-    // of halo cell h at s nh + h): a warp's consecutive cells read
-    // consecutive words (nh is odd, so the staging writes of one cell's 16
-    // sites fall in 16 different banks too)
-    const int nh = halo_cells(c.TX, c.TY, c.TZ);
-    int *hbase = reinterpret_cast<int *>(proj + 16 * nh);
-    for (int h = threadIdx.x; h < nh; h += blockDim.x)
-        hbase[h] = (int)(16 * halo_cell(h, c.TX, c.TY, c.ox, c.oy, c.oz, c.L));
-    __syncthreads();
-    // four consecutive sites per thread, each component read in 16-byte
-    // accesses (a cell's sites are 16-byte aligned in every plane)
-    for (int idx = threadIdx.x; idx < 4 * nh; idx += blockDim.x) {
-        const int h = idx >> 2, s0 = 4 * (idx & 3);
-        const int64_t i0 = (int64_t)hbase[h] + s0;
-        T v[NC][4];
+    // arithmetic here cost more than the whole FP32 kernel).  Site-major layout
+    // (site s of halo cell h at s nh + h): a warp's consecutive cells read
+    // consecutive words.  A thread takes four consecutive sites at a time, each
+    // component read in 16 bytes, two loads of each in flight; of a halo cell only the sites a
+    // down tetrahedron of the tile can reach are read: two groups of four across
+    // a face, one across an edge, none at the corner.  One group after the
+    // other, every halo site and the axis drawn here, the staging took a third
+    // of the kernel (337 us at L = 128, n = 3, FP32, now 287).
+    const int nh = halo_cells(c.TX, c.TY, c.TZ), HX = c.TX + 1, HY = c.TY + 1;
+    const int nt = c.nt, L = c.L;
+    constexpr int BATCH = 2;
+    T v[BATCH][NC][4];
+    auto own_load = [&](int b, int k) {
+        const int t = (threadIdx.x + k * nt) >> 2;
+        const int x = min(c.ox + (t & (c.TX - 1)), L - 1), y = min(c.oy + ((t >> c.lTX) & (c.TY - 1)), L - 1),
+                  z = min(c.oz + (t >> (c.lTX + c.lTY)), L - 1);
+        const int i0 = 16 * (x + L * (y + L * z)) + 4 * (threadIdx.x + k * nt & 3);
 #pragma unroll
-        for (int k = 0; k < NC; ++k) load4(spins + k * N + i0, v[k]);
+        for (int m = 0; m < NC; ++m) load4(spins + m * N + i0, v[b][m]);
+    };
+#pragma unroll
+    for (int b = 0; b < BATCH; ++b) own_load(b, b);
+    const double *axis = R.st->axis;
+    const float rf[3] = {(float)axis[0], (float)axis[1], (float)axis[2]};
+    auto put = [&](const T w[NC][4], int h, int s0) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            float pr = (float)v[0][q] * rf[0];  // in the order of project()
+            float pr = (float)w[0][q] * rf[0];  // in the order of project()
 #pragma unroll
-            for (int k = 1; k < NC; ++k) pr = Ar<float>::add(pr, Ar<float>::mul((float)v[k][q], rf[k]));
+            for (int k = 1; k < NC; ++k) pr = Ar<float>::add(pr, Ar<float>::mul((float)w[k][q], rf[k]));
             proj[(s0 + q) * nh + h] = pr;
         }
+    };
+#pragma unroll
+    for (int b0 = 0; b0 < 4; b0 += BATCH) {
+        if (b0 > 0)
+#pragma unroll
+            for (int b = 0; b < BATCH; ++b) own_load(b, b0 + b);
+#pragma unroll
+        for (int b = 0; b < BATCH; ++b) {
+            const int idx = threadIdx.x + (b0 + b) * nt, t = idx >> 2;
+            const int lx = t & (c.TX - 1), ly = (t >> c.lTX) & (c.TY - 1), lz = t >> (c.lTX + c.lTY);
+            put(v[b], lx + 1 + HX * (ly + 1 + HY * (lz + 1)), 4 * (idx & 3));
+        }
+    }
+    // halo: faces x, y, z (two groups a cell), then edges xy, xz, yz
+    const int fx = 2 * c.TY * c.TZ, fy = 2 * c.TX * c.TZ, fz = 2 * c.TX * c.TY;
+    const int nhalo = fx + fy + fz + c.TX + c.TY + c.TZ;
+    auto halo_load = [&](int e, T w[NC][4], int &h, int &s0) {
+        int lx = -1, ly = -1, lz = -1, g;
+        if (e < fx) {
+            ly = (e >> 1) & (c.TY - 1);
+            lz = e >> (1 + c.lTY);
+            g = 2 + (e & 1);
+        } else if ((e -= fx) < fy) {
+            lx = (e >> 1) & (c.TX - 1);
+            lz = e >> (1 + c.lTX);
+            g = 1 + 2 * (e & 1);
+        } else if ((e -= fy) < fz) {
+            lx = (e >> 1) & (c.TX - 1);
+            ly = e >> (1 + c.lTX);
+            g = 1 + (e & 1);
+        } else if ((e -= fz) < c.TZ) {
+            lz = e;
+            g = 3;
+        } else if ((e -= c.TZ) < c.TY) {
+            ly = e;
+            g = 2;
+        } else {
+            lx = e - c.TY;
+            g = 1;
+        }
+        h = lx + 1 + HX * (ly + 1 + HY * (lz + 1));
+        s0 = 4 * g;
+        // a step back from the lattice's first cell wraps, and a tile may
+        // reach past the last
+        int x = c.ox + lx, y = c.oy + ly, z = c.oz + lz;
+        x = x < 0 ? L - 1 : min(x, L - 1);
+        y = y < 0 ? L - 1 : min(y, L - 1);
+        z = z < 0 ? L - 1 : min(z, L - 1);
+        const int i0 = 16 * (x + L * (y + L * z)) + s0;
+#pragma unroll
+        for (int m = 0; m < NC; ++m) load4(spins + m * N + i0, w[m]);
+    };
+    for (int e = threadIdx.x; e < nhalo; e += 2 * nt) {
+        int h[2], s0[2];
+        halo_load(e, v[0], h[0], s0[0]);
+        const bool two = e + nt < nhalo;
+        if (two) halo_load(e + nt, v[1], h[1], s0[1]);
+        put(v[0], h[0], s0[0]);
+        if (two) put(v[1], h[1], s0[1]);
     }
     __syncthreads();
 
@@ -142,38 +200,51 @@ __global__ void __launch_bounds__(512, 2) vec_local_kernel(const __grid_constant
         // FP64, L = 64 862 -> 97 us.
         const float K2l = (float)R.K2 * 1.44269504f;
         const float margin = shortcut_margin<T>(R.K2);
-        uint32_t und[3];
-        const int h0 = halo_index(c, 0);
+        // (three calls together; then tetrahedron by tetrahedron, so that each
+        // projection is loaded once)
+        uint32_t ww[3][4];
 #pragma unroll
         for (int g = 0; g < 3; ++g) {
             const uint4 wd = philox_call(seed, sweep, TAG_BOND, 3 * (uint64_t)c.cell + g);
-            const uint32_t ww[4] = {wd.x, wd.y, wd.z, wd.w};
-            uint32_t a = 0, u = 0;
+            ww[g][0] = wd.x;
+            ww[g][1] = wd.y;
+            ww[g][2] = wd.z;
+            ww[g][3] = wd.w;
+        }
+        uint32_t und[3] = {0, 0, 0};
+        const int h0 = halo_index(c, 0);
 #pragma unroll
-            for (int f = 0; f < 4; ++f)
+        for (int f = 0; f < 4; ++f) {
+            float up[4], dn[4];
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                up[v] = proj[(4 * f + v) * nh + h0];
+                dn[v] = v == 0 ? up[0] : proj[down_bit(f, v) * nh + halo_index(c, down_mask(f, v))];
+            }
+            float ups[3], dns[3];  // the first vertex's, times -K2 log2 e
+#pragma unroll
+            for (int v = 0; v < 3; ++v) {
+                ups[v] = -(up[v] * K2l);
+                dns[v] = -(dn[v] * K2l);
+            }
+#pragma unroll
+            for (int g = 0; g < 3; ++g)
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
                     const int va = slot_a(g, q), vb = slot_b(g, q);
-                    float pa, pb;
-                    if (slot_up(g, q)) {
-                        pa = proj[(4 * f + va) * nh + h0];
-                        pb = proj[(4 * f + vb) * nh + h0];
-                    } else {
-                        pa = proj[down_bit(f, va) * nh + halo_index(c, down_mask(f, va))];
-                        pb = proj[down_bit(f, vb) * nh + halo_index(c, down_mask(f, vb))];
-                    }
-                    // 256 - b, from the float whose low mantissa bits are b
-                    const float fb = 8388864.0f - __uint_as_float(__byte_perm(ww[f], 0x4B000000u, 0x7440u | (uint32_t)q));
-                    const float e = exp2_approx(-((pa * pb) * K2l));
-                    const float qv = fmaf(-256.0f, e, fb);
+                    const float e = exp2_approx(slot_up(g, q) ? fmaf(ups[va], up[vb], 8.0f) : fmaf(dns[va], dn[vb], 8.0f));
+                    // -q: 256 exp(-y) less 256 - b, the latter from the float
+                    // whose low mantissa bits are b
+                    const float nq =
+                        e - (8388864.0f - __uint_as_float(__byte_perm(ww[g][f], 0x4B000000u, 0x7440u | (uint32_t)q)));
                     const uint32_t bit = 1u << (4 * f + q);
                     // (a NaN, from an infinite K2l, is neither on nor off)
-                    if (qv > 1.0f + margin) a |= bit;
-                    else if (!(qv < -margin)) u |= bit;
+                    if (nq < -1.0f - margin) act[g] |= bit;
+                    if (!(nq > margin)) und[g] |= bit;
                 }
-            act[g] = a;
-            und[g] = u;
         }
+#pragma unroll
+        for (int g = 0; g < 3; ++g) und[g] &= ~act[g];
         const T K2 = (T)R.K2;
         unsigned long long todo =
             (unsigned long long)(und[0] | (und[1] << 16)) | ((unsigned long long)und[2] << 32);
@@ -191,8 +262,10 @@ __global__ void __launch_bounds__(512, 2) vec_local_kernel(const __grid_constant
                 if (sizeof(T) == 4) {
                     pr[e] = (T)proj[s * nh + halo_index(c, m)];
                 } else {
-                    const T r[3] = {(T)s_axis[0], (T)s_axis[1], (T)s_axis[2]};
-                    pr[e] = project<NC, T>(spins, N, (int64_t)hbase[halo_index(c, m)] + s, r);
+                    const T r[3] = {(T)axis[0], (T)axis[1], (T)axis[2]};
+                    const int cx = (m & 1) ? wrap_back(c.x, L) : c.x, cy = (m & 2) ? wrap_back(c.y, L) : c.y,
+                              cz = (m & 4) ? wrap_back(c.z, L) : c.z;
+                    pr[e] = project<NC, T>(spins, N, 16 * (int64_t)(cx + L * (cy + L * cz)) + s, r);
                 }
             }
             const T x = A::mul(pr[0], pr[1]);
@@ -337,8 +410,7 @@ __global__ void __launch_bounds__(512) vec_flip_kernel(const __grid_constant__ B
     const Rep &R = B.reps[rep];
     const int tile = (int)(blockIdx.x - B.tile_begin[rep]);
     const TileCtx c = tile_ctx(B, R, tile);
-    __shared__ double s_axis[3];
-    if (threadIdx.x == 0) unit_vector_dev<NC>(R.seed, (uint32_t)R.st->sweep, TAG_AXIS, 0, s_axis);
+    const double *axis = R.st->axis;
     T *spins = static_cast<T *>(R.spins);
     const int64_t N = R.N;
     if (sizeof(T) == 8) {
@@ -357,7 +429,7 @@ __global__ void __launch_bounds__(512) vec_flip_kernel(const __grid_constant__ B
             if (lane >= o) incl += v;
         }
         if (lane == 31 || (int)threadIdx.x == c.nt - 1) wtotal[wid] = incl;
-        __syncthreads();  // publishes s_axis too
+        __syncthreads();
         int total = 0, base = 0;
         for (int w = 0; w < nw; ++w) {
             if (w == wid) base = total;
@@ -369,7 +441,7 @@ __global__ void __launch_bounds__(512) vec_flip_kernel(const __grid_constant__ B
             mask &= mask - 1;
         }
         __syncthreads();
-        const T r[3] = {(T)s_axis[0], (T)s_axis[1], (T)s_axis[2]};
+        const T r[3] = {(T)axis[0], (T)axis[1], (T)axis[2]};
         for (int e = threadIdx.x; e < total; e += c.nt) {
             T *p = spins + list[e];
             T t[NC];
@@ -385,8 +457,8 @@ __global__ void __launch_bounds__(512) vec_flip_kernel(const __grid_constant__ B
     int2 *todo = reinterpret_cast<int2 *>(smem);
     const uint32_t mask = cell_flip_mask(c, R, tile, smem + 2 * c.nt);
     todo[c.t] = make_int2((int)(16 * c.cell), c.valid ? (int)mask : 0);
-    __syncthreads();  // publishes s_axis too
-    const T r[3] = {(T)s_axis[0], (T)s_axis[1], (T)s_axis[2]};
+    __syncthreads();
+    const T r[3] = {(T)axis[0], (T)axis[1], (T)axis[2]};
     for (int idx = threadIdx.x; idx < 4 * c.nt; idx += blockDim.x) {
         const int2 cell = todo[idx >> 2];
         const int s0 = 4 * (idx & 3);

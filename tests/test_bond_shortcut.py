@@ -27,11 +27,12 @@ def test_shortcut_never_contradicts_the_exact_rule(fp64, K2):
         pb = pb.astype(F)
     off = rng.uniform(-3e-7, 3e-7, (2, n)) if fp64 else np.zeros((2, n))
     fa, fb = (pa + off[0]).astype(F), (pb + off[1]).astype(F)
-    arg = -((fa * fb) * K2l)
+    # one fused multiply-add: 8 - y log2 e, so that the exponential is 256 exp(-y)
+    arg = (8.0 - (fa * K2l).astype(np.float64) * fb.astype(np.float64)).astype(F)
     for err in (-1, 0, 1):
         with np.errstate(over="ignore"):
             e = (np.exp2(arg.astype(np.float64)) * (1 + err * 2.0 ** -22)).astype(F)
-            q = (np.float64(256 - b) - 256.0 * e.astype(np.float64)).astype(F)
+            q = -(e - (256 - b).astype(F))
         on, never = q > F(1) + margin, q < -margin
         if fp64:
             xs = pa * pb
