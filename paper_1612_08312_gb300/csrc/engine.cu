@@ -7,6 +7,7 @@
 #include <string>
 
 #include "engine.h"
+#include "launch.cuh"
 #include "nvec.cuh"
 
 namespace pyro {
@@ -57,6 +58,7 @@ __device__ __forceinline__ void acc_block_sum(V v[NV], V (*red)[ACC_THREADS])
 template <bool ISING>
 __global__ void __launch_bounds__(ACC_THREADS) fold_kernel(const __grid_constant__ Batch B)
 {
+    overlap_begin();
     const int r = blockIdx.x / B.fold, k = blockIdx.x - r * B.fold;
     const int64_t b0 = B.tile_begin[r], n = B.tile_begin[r + 1] - b0;
     const int64_t lo = b0 + n * k / B.fold, hi = b0 + n * (k + 1) / B.fold;
@@ -113,6 +115,7 @@ __device__ void draw_axis(const Rep &R, unsigned long long sweep, int nc)
 template <bool ISING>
 __global__ void __launch_bounds__(ACC_THREADS) accumulate_kernel(const __grid_constant__ Batch B, int mode, int nc)
 {
+    overlap_begin();
     const int r = blockIdx.x;
     const Rep &R = B.reps[r];
     DevStats *st = R.st;
@@ -215,8 +218,8 @@ __global__ void set_sweep_kernel(const __grid_constant__ Batch B, unsigned long 
 // Host launcher of the accumulation kernel for callers outside this file.
 void launch_accumulate(const Batch &B, bool ising, int mode, int nc, cudaStream_t s)
 {
-    if (ising) accumulate_kernel<true><<<B.R, ACC_THREADS, 0, s>>>(B, mode, nc);
-    else accumulate_kernel<false><<<B.R, ACC_THREADS, 0, s>>>(B, mode, nc);
+    if (ising) launch_overlapped(accumulate_kernel<true>, B.R, ACC_THREADS, 0, s, B, mode, nc);
+    else launch_overlapped(accumulate_kernel<false>, B.R, ACC_THREADS, 0, s, B, mode, nc);
 }
 
 // ------------------------------------------------------------------ host --
@@ -525,11 +528,11 @@ void Engine::enqueue_phase(int p, int mode)
         else vec_launch_measure(model, prec, B, ntiles, stream);
     } else {
         if (B.fold) {
-            if (model == PYRO_ISING) fold_kernel<true><<<R * B.fold, ACC_THREADS, 0, stream>>>(B);
-            else fold_kernel<false><<<R * B.fold, ACC_THREADS, 0, stream>>>(B);
+            if (model == PYRO_ISING) launch_overlapped(fold_kernel<true>, R * B.fold, ACC_THREADS, 0, stream, B);
+            else launch_overlapped(fold_kernel<false>, R * B.fold, ACC_THREADS, 0, stream, B);
         }
-        if (model == PYRO_ISING) accumulate_kernel<true><<<R, ACC_THREADS, 0, stream>>>(B, mode, 1);
-        else accumulate_kernel<false><<<R, ACC_THREADS, 0, stream>>>(B, mode, model);
+        if (model == PYRO_ISING) launch_overlapped(accumulate_kernel<true>, R, ACC_THREADS, 0, stream, B, mode, 1);
+        else launch_overlapped(accumulate_kernel<false>, R, ACC_THREADS, 0, stream, B, mode, model);
     }
 }
 

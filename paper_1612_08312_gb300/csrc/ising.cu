@@ -31,14 +31,15 @@ constexpr int MEASURE_BLOCK = 128;
 __global__ void __launch_bounds__(512) ising_local_kernel(const __grid_constant__ Batch B)
 {
     extern __shared__ __align__(16) int smem[];
+    const CoreSmem s = core_smem(smem, B.TX * B.TY * B.TZ);
+    core_prologue(s);
+    overlap_wait();
     const int r = find_rep(B.tile_begin, B.R, blockIdx.x);
     const Rep &R = B.reps[r];
     const int tile = (int)(blockIdx.x - B.tile_begin[r]);
     const TileCtx c = tile_ctx(B, R, tile);
-    const CoreSmem s = core_smem(smem, c.nt);
     const uint32_t sweep = (uint32_t)R.st->sweep;
     const uint64_t seed = R.seed;
-    core_prologue(s);
     // the cell's spin word and those of the cells one step back along the
     // axes of each mask m (read straight from global memory, L1-cached)
     const uint16_t *spins = static_cast<const uint16_t *>(R.spins);
@@ -109,6 +110,7 @@ __global__ void __launch_bounds__(512) ising_local_kernel(const __grid_constant_
 __global__ void __launch_bounds__(512) ising_flip_kernel(const __grid_constant__ Batch B)
 {
     extern __shared__ __align__(16) int smem[];
+    overlap_begin();
     const int r = find_rep(B.tile_begin, B.R, blockIdx.x);
     const Rep &R = B.reps[r];
     const int tile = (int)(blockIdx.x - B.tile_begin[r]);
@@ -137,6 +139,7 @@ __global__ void __launch_bounds__(512) labels_kernel(const __grid_constant__ Bat
 // tile, written to the tile's partial slot.
 __global__ void __launch_bounds__(MEASURE_BLOCK) ising_measure_kernel(const __grid_constant__ Batch B)
 {
+    overlap_begin();
     const int r = find_rep(B.tile_begin, B.R, blockIdx.x);
     const Rep &R = B.reps[r];
     const TileCtx c = tile_ctx(B, R, blockIdx.x - B.tile_begin[r]);  // the tile's origin
@@ -207,6 +210,7 @@ __global__ void __launch_bounds__(512, 4) boundary_unite_kernel(const __grid_con
     // equal share: entry (face cell << 5) | (6 f + k)
     extern __shared__ uint16_t blist[];
     __shared__ int bcount;
+    overlap_begin();
     const int r = find_rep(B.tile_begin, B.R, blockIdx.x);
     const Rep &R = B.reps[r];
     const int nface = face_cells(B.TX, B.TY, B.TZ);
@@ -275,6 +279,7 @@ constexpr int SLOT_BLOCK = 128;
 // link, so the walks may take the cached read-only path.
 __global__ void __launch_bounds__(SLOT_BLOCK) boundary_flip_kernel(const __grid_constant__ Batch B)
 {
+    overlap_begin();
     const int r = find_rep(B.tile_begin, B.R, blockIdx.x);
     const Rep &R = B.reps[r];
     const int64_t tile = blockIdx.x - B.tile_begin[r];
@@ -320,8 +325,8 @@ void launch_boundary(const Batch &B, int64_t ntiles, cudaStream_t s)
     const int nf = face_cells(B.TX, B.TY, B.TZ);
     const int threads = (nf + 31) & ~31;
     const size_t smem = (size_t)nf * 24 * sizeof(uint16_t);
-    boundary_unite_kernel<<<(unsigned)ntiles, threads, smem, s>>>(B);
-    boundary_flip_kernel<<<(unsigned)ntiles, SLOT_BLOCK, 0, s>>>(B);
+    launch_overlapped(boundary_unite_kernel, (unsigned)ntiles, threads, smem, s, B);
+    launch_overlapped(boundary_flip_kernel, (unsigned)ntiles, SLOT_BLOCK, 0, s, B);
 }
 
 void launch_labels(const Batch &B, int64_t ntiles, cudaStream_t s)
@@ -334,16 +339,16 @@ void ising_launch_phase(int p, const Batch &B, int64_t ntiles, cudaStream_t s)
 {
     const TileShape t{B.TX, B.TY, B.TZ};
     const int nt = B.TX * B.TY * B.TZ;
-    if (p == 0) ising_local_kernel<<<(unsigned)ntiles, nt, ising_local_smem(t), s>>>(B);
+    if (p == 0) launch_overlapped(ising_local_kernel, (unsigned)ntiles, nt, ising_local_smem(t), s, B);
     else if (p == 1) launch_boundary(B, ntiles, s);
-    else ising_flip_kernel<<<(unsigned)ntiles, nt, resolve_smem(t), s>>>(B);
+    else launch_overlapped(ising_flip_kernel, (unsigned)ntiles, nt, resolve_smem(t), s, B);
 }
 
 void ising_launch_measure(const Batch &B, int64_t ntiles, cudaStream_t s)
 {
     const int nt = B.TX * B.TY * B.TZ;
     const int threads = std::min(MEASURE_BLOCK, std::max(32, ((nt + 3) / 4 + 31) & ~31));
-    ising_measure_kernel<<<(unsigned)ntiles, threads, 0, s>>>(B);
+    launch_overlapped(ising_measure_kernel, (unsigned)ntiles, threads, 0, s, B);
 }
 
 }  // namespace pyro

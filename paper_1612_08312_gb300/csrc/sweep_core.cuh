@@ -16,6 +16,7 @@
 #pragma once
 
 #include "ccl.cuh"
+#include "launch.cuh"
 
 namespace pyro {
 

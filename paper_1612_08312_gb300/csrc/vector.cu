@@ -78,18 +78,20 @@ __global__ void __launch_bounds__(512, 2) vec_local_kernel(const __grid_constant
 {
     using A = Ar<T>;
     extern __shared__ __align__(16) int smem[];
+    const CoreSmem sm = core_smem(smem, B.TX * B.TY * B.TZ);
+    core_prologue(sm);
+    overlap_wait();
+    if (sizeof(T) == 8) overlap_next();  // (FP32: 0.4 % slower; FP64 L = 50: 211 us a sweep with, 220 without)
     const int rep = find_rep(B.tile_begin, B.R, blockIdx.x);
     const Rep &R = B.reps[rep];
     const int tile = (int)(blockIdx.x - B.tile_begin[rep]);
     const TileCtx c = tile_ctx(B, R, tile);
-    const CoreSmem sm = core_smem(smem, c.nt);
     const bool shared_stage = vec_stage_shared(c.TX, c.TY, c.TZ);
     float *proj = reinterpret_cast<float *>(shared_stage ? reinterpret_cast<unsigned char *>(smem) : sm.stage);
     const T *spins = static_cast<const T *>(R.spins);
     const int64_t N = R.N;
     const uint32_t sweep = (uint32_t)R.st->sweep;
     const uint64_t seed = R.seed;
-    core_prologue(sm);
 
     // Projections s_i . r of the tile's sites and the backward halo, in FP32
     // (for FP64 spins an approximation that the shortcut's margin covers: FP64
@@ -406,6 +408,7 @@ template <int NC, typename T>
 __global__ void __launch_bounds__(512) vec_flip_kernel(const __grid_constant__ Batch B)
 {
     extern __shared__ __align__(16) int smem[];
+    overlap_begin();
     const int rep = find_rep(B.tile_begin, B.R, blockIdx.x);
     const Rep &R = B.reps[rep];
     const int tile = (int)(blockIdx.x - B.tile_begin[rep]);
@@ -505,6 +508,7 @@ template <int NC, typename T>
 __global__ void __launch_bounds__(VEC_MEASURE_BLOCK) vec_measure_kernel(const __grid_constant__ Batch B)
 {
     extern __shared__ __align__(16) int smem[];
+    overlap_begin();
     double *scratch = reinterpret_cast<double *>(smem);  // blockDim values (FP64: 4 blockDim)
     const int rep = find_rep(B.tile_begin, B.R, blockIdx.x);
     const Rep &R = B.reps[rep];
@@ -657,14 +661,15 @@ struct VecOps {
     {
         const TileShape t{B.TX, B.TY, B.TZ};
         const int nt = B.TX * B.TY * B.TZ;
-        if (p == 0) vec_local_kernel<NC, T><<<(unsigned)ntiles, nt, vec_local_smem(t), s>>>(B);
+        if (p == 0) launch_overlapped(vec_local_kernel<NC, T>, (unsigned)ntiles, nt, vec_local_smem(t), s, B);
         else if (p == 1) launch_boundary(B, ntiles, s);
-        else vec_flip_kernel<NC, T><<<(unsigned)ntiles, nt, vec_flip_smem(t, sizeof(T)), s>>>(B);
+        else launch_overlapped(vec_flip_kernel<NC, T>, (unsigned)ntiles, nt, vec_flip_smem(t, sizeof(T)), s, B);
     }
     static void measure(const Batch &B, int64_t ntiles, cudaStream_t s)
     {
         const int threads = std::min(VEC_MEASURE_BLOCK, 4 * B.TX * B.TY * B.TZ);
-        vec_measure_kernel<NC, T><<<(unsigned)ntiles, threads, threads * sizeof(double) * (sizeof(T) == 8 ? 4 : 1), s>>>(B);
+        launch_overlapped(vec_measure_kernel<NC, T>, (unsigned)ntiles, threads,
+                          threads * sizeof(double) * (sizeof(T) == 8 ? 4 : 1), s, B);
     }
 };
 
