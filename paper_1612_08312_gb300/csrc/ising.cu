@@ -207,9 +207,12 @@ __global__ void __launch_bounds__(CELL_BLOCK) ising_init_kernel(const __grid_con
 __global__ void __launch_bounds__(512, 4) boundary_unite_kernel(const __grid_constant__ Batch B)
 {
     // the block's crossing pairs, compacted so that every thread takes an
-    // equal share: entry (face cell << 5) | (6 f + k)
-    extern __shared__ uint16_t blist[];
+    // equal share: entry lx | ly << 5 | lz << 10 | (6 f + k) << 16 (at most three
+    // pairs per tetrahedron span it)
+    extern __shared__ uint32_t blist[];
     __shared__ int bcount;
+    __shared__ uint32_t ends[24];
+    if (threadIdx.x < 24) ends[threadIdx.x] = pair_table.e[threadIdx.x];
     overlap_begin();
     const int r = find_rep(B.tile_begin, B.R, blockIdx.x);
     const Rep &R = B.reps[r];
@@ -222,12 +225,13 @@ __global__ void __launch_bounds__(512, 4) boundary_unite_kernel(const __grid_con
     const int oz = (int)(txy / (uint32_t)R.nty) * B.TZ;
     if (threadIdx.x == 0) bcount = 0;
     __syncthreads();
-    uint32_t todo = 0;
+    uint32_t todo = 0, here = 0;
     if ((int)threadIdx.x < nface) {
         int lx, ly, lz;
         face_cell_coords(B, threadIdx.x, lx, ly, lz);
         if (max(ox + lx, max(oy + ly, oz + lz)) < L)
             todo = R.dmask[(int64_t)(ox + lx) + (int64_t)L * ((int64_t)(oy + ly) + (int64_t)L * (oz + lz))];
+        here = (uint32_t)(lx | (ly << 5) | (lz << 10));
     }
     const int lane = threadIdx.x & 31;
     const int n = __popc(todo);
@@ -244,7 +248,7 @@ __global__ void __launch_bounds__(512, 4) boundary_unite_kernel(const __grid_con
     while (todo) {
         const int bit = __ffs(todo) - 1;
         todo &= todo - 1;
-        blist[pos++] = (uint16_t)((threadIdx.x << 5) | bit);
+        blist[pos++] = here | ((uint32_t)bit << 16);
     }
     __syncthreads();
     const int np = bcount;
@@ -252,19 +256,16 @@ __global__ void __launch_bounds__(512, 4) boundary_unite_kernel(const __grid_con
     bool ok = true;
     for (int i = threadIdx.x; i < np; i += blockDim.x) {
         const uint32_t en = blist[i];
-        int lx, ly, lz;
-        face_cell_coords(B, (int)(en >> 5), lx, ly, lz);
-        const int x = ox + lx, y = oy + ly, z = oz + lz;
-        const int f = (int)(en & 31u) / 6, k = (int)(en & 31u) % 6;
+        const int x = ox + (int)(en & 31u), y = oy + (int)((en >> 5) & 31u), z = oz + (int)((en >> 10) & 31u);
+        uint32_t pr = ends[en >> 16];
         uint32_t g[2];
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
-            const int v = e == 0 ? pair_a(k) : pair_b(k);
-            const int m = down_mask(f, v);
-            const int cx = (m & 1) ? wrap_back(x, L) : x;
-            const int cy = (m & 2) ? wrap_back(y, L) : y;
-            const int cz = (m & 4) ? wrap_back(z, L) : z;
-            g[e] = crossing_slot(R, B, cx, cy, cz, down_bit(f, v));
+            const int cx = (pr & 1u) ? wrap_back(x, L) : x;
+            const int cy = (pr & 2u) ? wrap_back(y, L) : y;
+            const int cz = (pr & 4u) ? wrap_back(z, L) : z;
+            g[e] = crossing_slot(R, B, cx, cy, cz, (int)((pr >> 4) & 15u));
+            pr >>= 16;
         }
         if (g[0] != g[1]) ok &= slot_unite(P, g[0], g[1]);
     }
@@ -289,15 +290,29 @@ __global__ void __launch_bounds__(SLOT_BLOCK) boundary_flip_kernel(const __grid_
     const uint32_t *own = P + tile * (16 * nt);
     // (a tile of one cell has half a word of slots)
     uint16_t *out = reinterpret_cast<uint16_t *>(R.sflip) + tile * nt;
-    for (int k0 = threadIdx.x & ~31; k0 < n; k0 += SLOT_BLOCK) {
-        const int k = k0 + (threadIdx.x & 31);
-        uint32_t bit = 0;
-        if (k < n) {
-            const uint32_t site = slot_root(P, __ldg(own + k));
-            bit = ((uint32_t)__ldg(R.F + (site >> 4)) >> (site & 15)) & 1u;
+    // three slots per thread at a time, their walks in lockstep
+    const int lane = threadIdx.x & 31;
+    for (int k0 = threadIdx.x & ~31; k0 < n; k0 += 3 * SLOT_BLOCK) {
+        uint32_t v[3];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const int k = k0 + j * SLOT_BLOCK + lane;
+            v[j] = k < n ? __ldg(own + k) : 0u;
         }
-        const uint32_t word = __ballot_sync(0xffffffffu, bit);
-        if ((threadIdx.x & 15) == 0 && k < n) out[k >> 4] = (uint16_t)(word >> (threadIdx.x & 16));
+#pragma unroll 1
+        for (int it = 0; it < (1 << 20) && ((v[0] | v[1] | v[2]) & SLOT_LINK); ++it)
+#pragma unroll
+            for (int j = 0; j < 3; ++j)
+                if (slot_linked(v[j])) v[j] = __ldg(P + (v[j] & ~SLOT_LINK));
+        uint32_t bit[3];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) bit[j] = ((uint32_t)__ldg(R.F + (v[j] >> 4)) >> (v[j] & 15)) & 1u;
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const int k = k0 + j * SLOT_BLOCK + lane;
+            const uint32_t word = __ballot_sync(0xffffffffu, bit[j]);
+            if ((lane & 15) == 0 && k < n) out[k >> 4] = (uint16_t)(word >> (lane & 16));
+        }
     }
 }
 
@@ -323,8 +338,13 @@ void ising_launch_init(const Batch &B, int64_t nblocks, int random, cudaStream_t
 void launch_boundary(const Batch &B, int64_t ntiles, cudaStream_t s)
 {
     const int nf = face_cells(B.TX, B.TY, B.TZ);
-    const int threads = (nf + 31) & ~31;
-    const size_t smem = (size_t)nf * 24 * sizeof(uint16_t);
+    // a thread per face cell where the grid fills the GPU; up to four per cell
+    // (a pair each) where it does not and the longest thread's chain of finds
+    // is the kernel's time (L = 16: 41 -> 36 us a sweep, L = 45: 62 -> 53; four
+    // at L = 256: crossing 685 -> 955 us)
+    int threads = (nf + 31) & ~31;
+    while (2 * threads <= 512 && 2 * threads <= 4 * ((nf + 31) & ~31) && ntiles * (2 * threads) <= 152 * 2048) threads *= 2;
+    const size_t smem = (size_t)nf * 12 * sizeof(uint32_t);
     launch_overlapped(boundary_unite_kernel, (unsigned)ntiles, threads, smem, s, B);
     launch_overlapped(boundary_flip_kernel, (unsigned)ntiles, SLOT_BLOCK, 0, s, B);
 }

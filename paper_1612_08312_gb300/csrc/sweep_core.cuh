@@ -272,6 +272,23 @@ __host__ __device__ constexpr uint32_t pair_axis_mask(int f, int d)
     return m;
 }
 
+// Ends of pair 6 f + k of a cell's down tetrahedra: the cells' shift masks
+// (bits 0-2 and 16-18) and sites (bits 4-7 and 20-23).
+struct PairTable {
+    uint32_t e[24];
+};
+constexpr PairTable make_pair_table()
+{
+    PairTable t{};
+    for (int f = 0; f < 4; ++f)
+        for (int k = 0; k < 6; ++k) {
+            const int a = pair_a(k), b = pair_b(k);
+            t.e[6 * f + k] = (uint32_t)(down_mask(f, a) | (down_bit(f, a) << 4) | (down_mask(f, b) << 16) | (down_bit(f, b) << 20));
+        }
+    return t;
+}
+static __device__ const PairTable pair_table = make_pair_table();
+
 // Vertices v of the down tetrahedron of f whose cell is a backward step along
 // axis d (bit v).
 __host__ __device__ constexpr uint32_t vertex_axis_mask(int f, int d)
@@ -573,7 +590,7 @@ __device__ __forceinline__ bool slot_linked(uint32_t v) { return (v & SLOT_LINK)
 __device__ __forceinline__ void slot_step(uint32_t *P, uint32_t &x, uint32_t &v)
 {
     const uint32_t p = v & ~SLOT_LINK;
-    const uint32_t gv = __ldcg(P + p);
+    const uint32_t gv = __ldca(P + p);
     if (slot_linked(gv)) __stcg(P + x, gv);
     x = p;
     v = gv;
@@ -584,7 +601,7 @@ __device__ __forceinline__ void slot_step(uint32_t *P, uint32_t &x, uint32_t &v)
 // the entry its walk ended on.  Returns false if the bound was hit.
 __device__ __forceinline__ bool slot_unite(uint32_t *P, uint32_t a, uint32_t b)
 {
-    uint32_t va = __ldcg(P + a), vb = __ldcg(P + b);
+    uint32_t va = __ldca(P + a), vb = __ldca(P + b);
 #pragma unroll 1
     for (int it = 0; it < (1 << 20); ++it) {
         const bool la = slot_linked(va), lb = slot_linked(vb);
@@ -626,9 +643,9 @@ __device__ __forceinline__ uint32_t tile_of(const Rep &R, const Batch &B, int x,
 // Slot of site s of cell (x, y, z), an end of a crossing bond.
 __device__ __forceinline__ uint32_t crossing_slot(const Rep &R, const Batch &B, int x, int y, int z, int s)
 {
-    const int L = R.L, ns = 16 * B.TX * B.TY * B.TZ;
-    const int code = R.L16[16 * ((int64_t)x + (int64_t)L * ((int64_t)y + (int64_t)L * z)) + s];
-    return tile_of(R, B, x, y, z) * (uint32_t)ns + (uint32_t)(code - ns);
+    const uint32_t L = (uint32_t)R.L, ns = 16u * B.TX * B.TY * B.TZ;  // (N < 2^31)
+    const uint32_t code = R.L16[16 * ((uint32_t)x + L * ((uint32_t)y + L * (uint32_t)z)) + (uint32_t)s];
+    return tile_of(R, B, x, y, z) * ns + (code - ns);
 }
 
 // Shared-memory bytes of the flip stage: the cells' flip words and the slots'.
