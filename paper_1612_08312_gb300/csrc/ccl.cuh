@@ -94,25 +94,30 @@ __device__ __forceinline__ bool sunite(int a, int b)
 // Pair index k of vertices (a, b), a < b.
 __host__ __device__ constexpr int pair_index(int a, int b) { return a == 0 ? b - 1 : (a == 1 ? b + 1 : 5); }
 
-// Deterministic block sum of a double (fixed shuffle tree), result valid in
-// thread 0.  Every thread of the block must call it.
-__device__ __forceinline__ double block_sum_f64(double v)
+// Threads of an accumulation block.
+constexpr int ACC_THREADS = 128;
+
+// Sums of NV values over a block of THREADS (a power of two from 64) threads,
+// a fixed tree in shared memory, one barrier per level for all; results valid
+// in the first warp.  (A shuffle tree adds in FP64 on every lane at every
+// level; FP64 adds are scarce on this GPU.)
+template <typename V, int NV, int THREADS>
+__device__ __forceinline__ void block_sums(V v[NV], V (*red)[THREADS])
 {
-    __shared__ double red_f64[32];
+    const int t = threadIdx.x;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = __dadd_rn(v, __shfl_xor_sync(0xffffffffu, v, o));
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int nw = (blockDim.x + 31) >> 5;
+    for (int q = 0; q < NV; ++q) red[q][t] = v[q];
     __syncthreads();
-    if (lane == 0) red_f64[wid] = v;
-    __syncthreads();
-    double r = 0.0;
-    if (wid == 0) {
-        r = lane < nw ? red_f64[lane] : 0.0;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) r = __dadd_rn(r, __shfl_xor_sync(0xffffffffu, r, o));
+    for (int o = THREADS / 2; o > 0; o >>= 1) {
+        if (t < o)
+#pragma unroll
+            for (int q = 0; q < NV; ++q) red[q][t] += red[q][t + o];
+        if (o > 16) __syncthreads();
+        else __syncwarp();
     }
-    return r;
+#pragma unroll
+    for (int q = 0; q < NV; ++q) v[q] = red[q][0];
 }
 
 // Neumaier step with explicitly rounded operations (no contraction).

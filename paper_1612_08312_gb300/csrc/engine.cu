@@ -26,30 +26,6 @@ void vec_launch_init(int model, int prec, const Batch &B, int64_t nblocks, int r
 void vec_launch_phase(int p, int model, int prec, const Batch &B, int64_t ntiles, cudaStream_t s);
 void vec_launch_measure(int model, int prec, const Batch &B, int64_t ntiles, cudaStream_t s);
 
-// Threads of an accumulation block.
-constexpr int ACC_THREADS = 128;
-
-// Sums of four values over a block of ACC_THREADS threads in a fixed tree
-// (integers: the first two); results valid in the first warp.
-template <typename V, int NV>
-__device__ __forceinline__ void acc_block_sum(V v[NV], V (*red)[ACC_THREADS])
-{
-    const int t = threadIdx.x;
-#pragma unroll
-    for (int q = 0; q < NV; ++q) red[q][t] = v[q];
-    __syncthreads();
-#pragma unroll
-    for (int o = ACC_THREADS / 2; o > 0; o >>= 1) {
-        if (t < o)
-#pragma unroll
-            for (int q = 0; q < NV; ++q) red[q][t] += red[q][t + o];
-        if (o > 16) __syncthreads();
-        else __syncwarp();
-    }
-#pragma unroll
-    for (int q = 0; q < NV; ++q) v[q] = red[q][0];
-}
-
 // With B.fold groups per replica, a first kernel sums each group of a
 // replica's tile partials (a contiguous range, fixed order) on its own
 // block, so that the accumulation reads B.fold values per replica instead of
@@ -71,7 +47,7 @@ __global__ void __launch_bounds__(ACC_THREADS) fold_kernel(const __grid_constant
             v[0] += p.x;
             v[1] += p.y;
         }
-        acc_block_sum<unsigned long long, 2>(v, red);
+        block_sums<unsigned long long, 2, ACC_THREADS>(v, red);
         if (threadIdx.x == 0) *reinterpret_cast<ulonglong2 *>(B.folded + 4 * (int64_t)blockIdx.x) = make_ulonglong2(v[0], v[1]);
     } else {
         __shared__ double red[4][ACC_THREADS];
@@ -85,7 +61,7 @@ __global__ void __launch_bounds__(ACC_THREADS) fold_kernel(const __grid_constant
             v[2] += q.x;
             v[3] += q.y;
         }
-        acc_block_sum<double, 4>(v, red);
+        block_sums<double, 4, ACC_THREADS>(v, red);
         if (threadIdx.x == 0)
 #pragma unroll
             for (int q = 0; q < 4; ++q) B.folded[4 * (int64_t)blockIdx.x + q] = v[q];
@@ -137,7 +113,7 @@ __global__ void __launch_bounds__(ACC_THREADS) accumulate_kernel(const __grid_co
             v[0] += p.x;
             v[1] += p.y;
         }
-        acc_block_sum<unsigned long long, 2>(v, red);
+        block_sums<unsigned long long, 2, ACC_THREADS>(v, red);
         if (t >= 32) return;
         const long long anti = (long long)v[0];
         const long long M = R.N - 2 * (long long)v[1];
@@ -156,7 +132,7 @@ __global__ void __launch_bounds__(ACC_THREADS) accumulate_kernel(const __grid_co
             tot[2] += q.x;
             tot[3] += q.y;
         }
-        acc_block_sum<double, 4>(tot, red);
+        block_sums<double, 4, ACC_THREADS>(tot, red);
         if (t >= 32) return;
     }
     // every lane of the first warp forms the observables; lane k < 5 keeps sum k

@@ -29,7 +29,9 @@
 #include <string>
 #include <vector>
 
+#include "bonds.cuh"
 #include "engine.h"
+#include "launch.cuh"
 #include "nvec.cuh"
 
 namespace pyro {
@@ -89,41 +91,35 @@ __device__ __forceinline__ void bond_ends(const GraphDev &G, int64_t e, int &i, 
 __device__ __forceinline__ bool bit_of(const uint32_t *set, int64_t k) { return (set[k >> 5] >> (k & 31)) & 1u; }
 
 // Union of the clusters of a and b in the global array (path halving in
-// both finds).  False if the union's iteration bound was hit.
-__device__ bool gunite(int32_t *lab, int a, int b)
+// both finds).  The finds read through L1: a stale entry still names an
+// ancestor, links are decided by the atomic, and from L2 all finds met at the
+// entry of the largest cluster's root.  False if the union's iteration bound
+// was hit.
+__device__ __forceinline__ bool gunite(int32_t *lab, int a, int b)
 {
-    volatile int32_t *vl = lab;
     const int bound = c_unite_bound;
-    int pa = vl[a], pb = vl[b];
+    int pa = __ldca(lab + a), pb = __ldca(lab + b);
 #pragma unroll 1
     for (int it = 0; it < bound; ++it) {
 #pragma unroll 1
         for (int st = 0; (pa != a || pb != b) && st < (1 << 20); ++st) {
-            if (pa != a) {
-                const int g = vl[pa];
-                if (g != pa) vl[a] = g;
-                a = pa;
-                pa = g;
-            }
-            if (pb != b) {
-                const int g = vl[pb];
-                if (g != pb) vl[b] = g;
-                b = pb;
-                pb = g;
-            }
+            const int ga = __ldca(lab + pa), gb = __ldca(lab + pb);
+            if (ga != pa) lab[a] = ga;
+            if (gb != pb) lab[b] = gb;
+            a = pa;
+            pa = ga;
+            b = pb;
+            pb = gb;
         }
         if (a == b) return true;
-        if (a > b) {
-            const int t = a;
-            a = b;
-            b = t;
-        }
-        const int old = atomicMin(&lab[b], a);
-        if (old == b) return true;
-        // b had been linked meanwhile: unite a with its new parent
+        const int lo = min(a, b), hi = max(a, b);
+        const int old = atomicMin(&lab[hi], lo);
+        if (old == hi) return true;
+        // hi had been linked meanwhile: unite lo with its new parent
+        a = lo;
         b = old;
-        pa = vl[a];
-        pb = vl[b];
+        pa = __ldca(lab + a);
+        pb = __ldca(lab + b);
     }
     return false;
 }
@@ -153,6 +149,7 @@ __global__ void __launch_bounds__(GB_THREADS) graph_init_kernel(const __grid_con
 template <int NC, typename T>
 __global__ void __launch_bounds__(GB_THREADS) graph_proj_kernel(const __grid_constant__ GraphDev G)
 {
+    overlap_begin();
     __shared__ double rs[3];
     if (threadIdx.x == 0) {
         unit_vector_dev<NC>(G.seed, (uint32_t)G.st->sweep, TAG_AXIS, 0, rs);
@@ -170,70 +167,148 @@ __global__ void __launch_bounds__(GB_THREADS) graph_proj_kernel(const __grid_con
 // Thread c takes the 16 bonds 16 c .. 16 c + 15 (one BOND call) and draws
 // the FLIP call c.  (One bond per lane with the words passed by shuffles was
 // measured slower: a warp's lanes then unite the bonds of the same few sites
-// at once.)
+// at once.)  The bonds are decided first, all sites and spins loaded together
+// (bond after bond, each waited for its own sites, spins and unions), then the
+// active ones are united in a loop of their own.
 template <int NC, typename T>
 __global__ void __launch_bounds__(GB_THREADS) graph_bond_kernel(const __grid_constant__ GraphDev G)
 {
+    overlap_begin();
     const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const uint32_t sweep = (uint32_t)G.st->sweep;
     if (128 * c < G.N) reinterpret_cast<uint4 *>(G.fb)[c] = philox_call(G.seed, sweep, TAG_FLIP, (uint64_t)c);
     const int64_t e0 = 16 * c;
     if (e0 >= G.NB) return;
     const uint4 w = philox_call(G.seed, sweep, TAG_BOND, (uint64_t)c);
+    const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
     const int nq = (int)(G.NB - e0 < 16 ? G.NB - e0 : 16);
-    uint32_t pres = 0xFFFFu;
-    if (G.present) pres = (G.present[e0 >> 5] >> (e0 & 31)) & 0xFFFFu;
-    bool ok = true;
-    // simple cubic: bond 3 s + d, walked incrementally from the chunk's first
-    int s = 0, d = 0, x = 0, y = 0, z = 0;
+    uint32_t pres = 0xFFFFu >> (16 - nq);
+    if (G.present) pres &= G.present[e0 >> 5] >> (e0 & 31);
+    // simple cubic: bond 3 s + d, from the chunk's first
+    int s0 = 0, d0 = 0, x0 = 0, y0 = 0, z0 = 0;
     if (G.L) {
-        const uint64_t s0 = (uint64_t)e0 / 3u;
-        s = (int)s0;
-        d = (int)((uint64_t)e0 - 3u * s0);
-        sc_coords(G.L, s, x, y, z);
+        const uint64_t s = (uint64_t)e0 / 3u;
+        s0 = (int)s;
+        d0 = (int)((uint64_t)e0 - 3u * s);
+        sc_coords(G.L, s0, x0, y0, z0);
     }
-#pragma unroll 1
-    for (int q = 0; q < nq; ++q) {
-        if (G.L && q > 0 && ++d == 3) {
-            d = 0;
-            ++s;
-            if (++x == G.L) {
-                x = 0;
+    const auto ends = [&](int q, int &i, int &j) {  // of bond e0 + q, q < nq
+        if (G.L) {
+            int x = x0, y = y0, z = z0, ds = (d0 + q) / 3;
+            const int d = d0 + q - 3 * ds;
+            i = s0 + ds;
+            for (x += ds; x >= G.L; x -= G.L)
                 if (++y == G.L) {
                     y = 0;
                     ++z;
                 }
+            j = sc_next(G.L, i, x, y, z, d);
+        } else {
+            i = G.bi[e0 + q];
+            j = G.bj[e0 + q];
+        }
+    };
+    uint32_t act = 0, tie = 0;
+    if (NC == 1) {
+        // bonds whose top byte is below (equals) the threshold's, then those
+        // between equal spins
+        const ByteCompare bc(G.thr);
+        if (bc.all) {
+            act = 0xFFFFu;
+        } else if (!bc.none) {
+            const uint32_t t4 = bc.t8 * 0x01010101u;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                act |= byte_flags_to_nibble(bytes_lt(ww[k], t4)) << (4 * k);
+                tie |= byte_flags_to_nibble(bytes_eq(ww[k], t4)) << (4 * k);
             }
         }
-        if (!((pres >> q) & 1u)) continue;
-        const int64_t e = e0 + q;
+        const uint32_t cand = (act | tie) & pres;
+        const int8_t *sp = static_cast<const int8_t *>(G.spins);
+        int si[16], sj[16];
+        if (!G.L && nq == 16) {  // the list in 16-byte loads
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int4 i = __ldg(reinterpret_cast<const int4 *>(G.bi + e0) + k);
+                const int4 j = __ldg(reinterpret_cast<const int4 *>(G.bj + e0) + k);
+                si[4 * k] = i.x;
+                si[4 * k + 1] = i.y;
+                si[4 * k + 2] = i.z;
+                si[4 * k + 3] = i.w;
+                sj[4 * k] = j.x;
+                sj[4 * k + 1] = j.y;
+                sj[4 * k + 2] = j.z;
+                sj[4 * k + 3] = j.w;
+            }
+        } else {
+#pragma unroll
+            for (int q = 0; q < 16; ++q) {
+                si[q] = sj[q] = 0;
+                if ((cand >> q) & 1u) ends(q, si[q], sj[q]);
+            }
+        }
+        uint32_t same = 0;
+#pragma unroll
+        for (int q = 0; q < 16; ++q) {
+            if (!((cand >> q) & 1u)) continue;
+            si[q] = sp[si[q]];
+            sj[q] = sp[sj[q]];
+        }  // (a bond that is no candidate is masked out below)
+#pragma unroll
+        for (int q = 0; q < 16; ++q) same |= (si[q] == sj[q] ? 1u : 0u) << q;
+        act &= same & pres;
+        tie &= same & pres;
+        for (uint32_t k = tie; k; k &= k - 1) {
+            const int q = __ffs(k) - 1;
+            const uint4 t = philox_call(G.seed, sweep, TAG_TIE, (uint64_t)(e0 + q) >> 2);
+            if ((word_of(t, q & 3) & 0xFFFFFFu) < bc.t24) act |= 1u << q;
+        }
+    } else {
+        const T *p = static_cast<const T *>(G.proj);
+        T xp[16];
+#pragma unroll
+        for (int h = 0; h < 16; h += 8) {
+            int si[8], sj[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                si[q] = sj[q] = -1;
+                if ((pres >> (h + q)) & 1u) ends(h + q, si[q], sj[q]);
+            }
+#pragma unroll
+            for (int q = 0; q < 8; ++q) xp[h + q] = si[q] >= 0 ? Ar<T>::mul(p[si[q]], p[sj[q]]) : (T)0;
+        }
+        // the pyrochlore kernel's shortcut: 256 p - b from one fast exponential
+        // decides all bonds but those within the margin of [0, 1]
+        const float K2l = (float)G.K2 * 1.44269504f;
+#pragma unroll
+        for (int q = 0; q < 16; ++q) {
+            if (!(xp[q] > (T)0)) continue;
+            const float nq2 = exp2_approx(fmaf(-K2l, (float)xp[q], 8.0f)) -
+                              (8388864.0f - __uint_as_float(__byte_perm(ww[q >> 2], 0x4B000000u, 0x7440u | (q & 3))));
+            if (nq2 < -1.0f - SHORTCUT_MARGIN) act |= 1u << q;
+            else if (!(nq2 > SHORTCUT_MARGIN)) tie |= 1u << q;
+        }
+        if (!(G.K2 > 0.0)) act = tie = 0;
+        for (uint32_t k = tie; k; k &= k - 1) {
+            const int q = __ffs(k) - 1;
+            int i, j;
+            ends(q, i, j);
+            const ByteCompare bc(prob_threshold(Ar<T>::bond_p((T)G.K2, Ar<T>::mul(p[i], p[j]))));
+            const uint32_t byte = (word_of(w, q >> 2) >> (8 * (q & 3))) & 0xFFu;
+            bool on = bc.all || byte < bc.t8;
+            if (!on && byte == bc.t8) {
+                const uint4 t = philox_call(G.seed, sweep, TAG_TIE, (uint64_t)(e0 + q) >> 2);
+                on = (word_of(t, q & 3) & 0xFFFFFFu) < bc.t24;
+            }
+            if (on && !bc.none) act |= 1u << q;
+        }
+    }
+    bool ok = true;
+#pragma unroll 1
+    for (; act; act &= act - 1) {
         int i, j;
-        if (G.L) {
-            i = s;
-            j = sc_next(G.L, s, x, y, z, d);
-        } else {
-            i = G.bi[e];
-            j = G.bj[e];
-        }
-        uint64_t thr;
-        if (NC == 1) {
-            const int8_t *sp = static_cast<const int8_t *>(G.spins);
-            if (sp[i] != sp[j]) continue;
-            thr = G.thr;
-        } else {
-            const T *p = static_cast<const T *>(G.proj);
-            const T xp = Ar<T>::mul(p[i], p[j]);
-            if (!(xp > (T)0)) continue;
-            thr = prob_threshold(Ar<T>::bond_p((T)G.K2, xp));
-        }
-        const uint64_t byte = (word_of(w, q >> 2) >> (8 * (q & 3))) & 0xFFu;
-        const uint64_t hi = thr >> 24;
-        bool act = byte < hi;
-        if (byte == hi) {
-            const uint4 t = philox_call(G.seed, sweep, TAG_TIE, (uint64_t)e >> 2);
-            act = (word_of(t, (int)(e & 3)) & 0xFFFFFFu) < (uint32_t)(thr & 0xFFFFFFu);
-        }
-        if (act && !gunite(G.lab, i, j)) ok = false;
+        ends(__ffs(act) - 1, i, j);
+        ok &= gunite(G.lab, i, j);
     }
     if (!ok) atomicOr(&G.st->status, ST_NOCONVERGE);
 }
@@ -241,15 +316,15 @@ __global__ void __launch_bounds__(GB_THREADS) graph_bond_kernel(const __grid_con
 template <int NC, typename T>
 __global__ void __launch_bounds__(GB_THREADS) graph_flip_kernel(const __grid_constant__ GraphDev G)
 {
+    overlap_begin();
     using A = Ar<T>;
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= G.N) return;
-    const volatile int32_t *vl = G.lab;
-    int r = vl[i];
+    int r = __ldca(G.lab + i);  // (stale entries are ancestors)
     int steps = 0;
 #pragma unroll 1
     for (;;) {
-        const int p = vl[r];
+        const int p = __ldca(G.lab + r);
         if (p == r) break;
         r = p;
         if (++steps > UF_MAX_ITERS) {
@@ -286,15 +361,18 @@ __global__ void __launch_bounds__(GB_THREADS) graph_flip_kernel(const __grid_con
 template <int NC, typename T>
 __global__ void __launch_bounds__(GB_THREADS) graph_measure_kernel(const __grid_constant__ GraphDev G)
 {
+    overlap_begin();
     const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     double v[4] = {0.0, 0.0, 0.0, 0.0};
     if (NC == 1) {
         const int8_t *s = static_cast<const int8_t *>(G.spins);
         long long e = 0, m = 0;
+#pragma unroll 4
         for (int64_t i = t0; i < G.N; i += stride)
             if (!G.occ || bit_of(G.occ, i)) m += s[i];
         if (G.L) {
+#pragma unroll 4
             for (int64_t i = t0; i < G.N; i += stride) {
                 int x, y, z;
                 sc_coords(G.L, (int)i, x, y, z);
@@ -305,10 +383,18 @@ __global__ void __launch_bounds__(GB_THREADS) graph_measure_kernel(const __grid_
                 }
             }
         } else {
-            for (int64_t b = t0; b < G.NB; b += stride) {
-                if (G.present && !bit_of(G.present, b)) continue;
-                e += s[G.bi[b]] == s[G.bj[b]] ? 1 : -1;
+            // four bonds per thread in 16-byte loads, two fours in flight
+            const int4 *bi = reinterpret_cast<const int4 *>(G.bi), *bj = reinterpret_cast<const int4 *>(G.bj);
+#pragma unroll 2
+            for (int64_t b = t0; b < G.NB >> 2; b += stride) {
+                const int4 i = __ldg(bi + b), j = __ldg(bj + b);
+                const uint32_t pres = G.present ? (G.present[b >> 3] >> (4 * (b & 7))) & 0xFu : 0xFu;
+                const uint32_t diff = (s[i.x] != s[j.x] ? 1u : 0u) | (s[i.y] != s[j.y] ? 2u : 0u) |
+                                      (s[i.z] != s[j.z] ? 4u : 0u) | (s[i.w] != s[j.w] ? 8u : 0u);
+                e += __popc(pres) - 2 * __popc(pres & diff);
             }
+            const int64_t b = (G.NB & ~(int64_t)3) + t0;
+            if (b < G.NB && (!G.present || bit_of(G.present, b))) e += s[G.bi[b]] == s[G.bj[b]] ? 1 : -1;
         }
         v[0] = (double)e;
         v[1] = (double)m;
@@ -328,28 +414,34 @@ __global__ void __launch_bounds__(GB_THREADS) graph_measure_kernel(const __grid_
             v[0] = __dadd_rn(v[0], d);
         }
     }
+    __shared__ double red[4][GB_THREADS];
+    block_sums<double, 4, GB_THREADS>(v, red);
+    if (threadIdx.x == 0)
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const double tot = block_sum_f64(v[q]);
-        if (threadIdx.x == 0) G.partials[4 * blockIdx.x + q] = tot;
-    }
+        for (int q = 0; q < 4; ++q) G.partials[4 * blockIdx.x + q] = v[q];
 }
 
 // One block: the partials in a fixed order, E = -J sum s_i . s_j,
 // m = |M| / N_occ, m^2, m^4; mode 1 adds them to the Neumaier sums and
 // advances the sweep counter, mode 2 only records them.
-__global__ void __launch_bounds__(1024) graph_accumulate_kernel(const __grid_constant__ GraphDev G, int nblocks,
-                                                                int mode)
+__global__ void __launch_bounds__(ACC_THREADS) graph_accumulate_kernel(const __grid_constant__ GraphDev G, int nblocks,
+                                                                       int mode)
 {
-    double v[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int b = threadIdx.x; b < nblocks; b += blockDim.x)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) v[q] = __dadd_rn(v[q], G.partials[4 * b + q]);
-    double tot[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) tot[q] = block_sum_f64(v[q]);
-    if (threadIdx.x != 0) return;
+    overlap_begin();
+    const int t = threadIdx.x;
     DevStats *st = G.st;
+    // the record's fields, read ahead of the sums they are needed after
+    const unsigned long long sweep = st->sweep, count = st->count;
+    double acc_s = t < 5 ? st->acc_s[t] : 0.0, acc_c = t < 5 ? st->acc_c[t] : 0.0;
+    __shared__ double red[4][ACC_THREADS];
+    double tot[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 4
+    for (int b = t; b < nblocks; b += ACC_THREADS)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) tot[q] += G.partials[4 * b + q];
+    block_sums<double, 4, ACC_THREADS>(tot, red);
+    if (t >= 32) return;
+    // every lane of the first warp forms the observables; lane k < 5 keeps sum k
     const double E = __dmul_rn(-G.J, tot[0]);
     double m = 0.0;
     if (G.nocc > 0) {
@@ -363,18 +455,23 @@ __global__ void __launch_bounds__(1024) graph_accumulate_kernel(const __grid_con
     }
     const double m2 = __dmul_rn(m, m);
     const double m4 = __dmul_rn(m2, m2);
-    st->last[0] = E;
-    st->last[1] = m2;
-    st->last[2] = m4;
-    st->last[3] = tot[1];
+    if (t == 0) {
+        st->last[0] = E;
+        st->last[1] = m2;
+        st->last[2] = m4;
+        st->last[3] = tot[1];
+    }
     if (mode != 1) return;
-    nsum_add(st->acc_s[0], st->acc_c[0], E);
-    nsum_add(st->acc_s[1], st->acc_c[1], __dmul_rn(E, E));
-    nsum_add(st->acc_s[2], st->acc_c[2], m2);
-    nsum_add(st->acc_s[3], st->acc_c[3], m4);
-    nsum_add(st->acc_s[4], st->acc_c[4], __dsqrt_rn(m2));
-    st->count += 1;
-    st->sweep += 1;
+    if (t < 5) {
+        const double x = t == 0 ? E : t == 1 ? __dmul_rn(E, E) : t == 2 ? m2 : t == 3 ? m4 : __dsqrt_rn(m2);
+        nsum_add(acc_s, acc_c, x);
+        st->acc_s[t] = acc_s;
+        st->acc_c[t] = acc_c;
+    }
+    if (t == 0) {
+        st->count = count + 1;
+        st->sweep = sweep + 1;
+    }
 }
 
 __global__ void graph_set_sweep_kernel(DevStats *st, unsigned long long s) { st->sweep = s; }
@@ -400,14 +497,14 @@ struct GraphOps {
     static void sweep(const GraphDev &G, cudaStream_t s, unsigned nproj, unsigned nbond, unsigned nsite,
                       unsigned nmeas)
     {
-        if (NC > 1) graph_proj_kernel<NC, T><<<nproj, GB_THREADS, 0, s>>>(G);
-        graph_bond_kernel<NC, T><<<nbond, GB_THREADS, 0, s>>>(G);
-        graph_flip_kernel<NC, T><<<nsite, GB_THREADS, 0, s>>>(G);
-        graph_measure_kernel<NC, T><<<nmeas, GB_THREADS, 0, s>>>(G);
+        if (NC > 1) launch_overlapped(graph_proj_kernel<NC, T>, nproj, GB_THREADS, 0, s, G);
+        launch_overlapped(graph_bond_kernel<NC, T>, nbond, GB_THREADS, 0, s, G);
+        launch_overlapped(graph_flip_kernel<NC, T>, nsite, GB_THREADS, 0, s, G);
+        launch_overlapped(graph_measure_kernel<NC, T>, nmeas, GB_THREADS, 0, s, G);
     }
     static void measure(const GraphDev &G, cudaStream_t s, unsigned nmeas)
     {
-        graph_measure_kernel<NC, T><<<nmeas, GB_THREADS, 0, s>>>(G);
+        launch_overlapped(graph_measure_kernel<NC, T>, nmeas, GB_THREADS, 0, s, G);
     }
 };
 
@@ -545,7 +642,7 @@ struct GraphEngine {
     {
         for (int64_t s = 0; s < n; ++s) {
             k.sweep(G, stream, nproj, nbond, nsite, nmeas);
-            graph_accumulate_kernel<<<1, 1024, 0, stream>>>(G, (int)nmeas, 1);
+            launch_overlapped(graph_accumulate_kernel, 1, ACC_THREADS, 0, stream, G, (int)nmeas, 1);
             launches += model == PYRO_ISING ? 4 : 5;
             lab_last = G.lab;
             std::swap(G.lab, G.lab_next);
@@ -556,7 +653,7 @@ struct GraphEngine {
     cudaError_t measure()
     {
         k.measure(G, stream, nmeas);
-        graph_accumulate_kernel<<<1, 1024, 0, stream>>>(G, (int)nmeas, 2);
+        launch_overlapped(graph_accumulate_kernel, 1, ACC_THREADS, 0, stream, G, (int)nmeas, 2);
         launches += 2;
         return cudaGetLastError();
     }

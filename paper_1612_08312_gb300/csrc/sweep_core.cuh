@@ -15,6 +15,7 @@
 // byte of its uniform from byte (b & 15) of BOND call b >> 4 = 3 c + g.
 #pragma once
 
+#include "bonds.cuh"
 #include "ccl.cuh"
 #include "launch.cuh"
 
@@ -193,40 +194,6 @@ __device__ __forceinline__ void antiparallel_groups(uint32_t U, uint32_t D, uint
     A = (u1 & 0x7777u) | ((u3 & 0x1111u) << 3);
     Bg = (u2 & 0x3333u) | ((d2 & 0x3333u) << 2);
     C = (d1 & 0x7777u) | ((d3 & 0x1111u) << 3);
-}
-
-// Bytewise unsigned a < b: bit 7 of each byte of the result.
-__device__ __forceinline__ uint32_t bytes_lt(uint32_t a, uint32_t b)
-{
-    const uint32_t d = (a | 0x80808080u) - (b & 0x7F7F7F7Fu);  // bit 7: low 7 bits of a >= those of b
-    return ((~(a ^ b) & ~d) | (~a & b)) & 0x80808080u;
-}
-
-// Bytewise a == b: bit 7 of each byte.
-__device__ __forceinline__ uint32_t bytes_eq(uint32_t a, uint32_t b)
-{
-    const uint32_t t = a ^ b;
-    return ~(((t & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | t) & 0x80808080u;
-}
-
-// Bit 7 of the four bytes -> four low bits.
-__device__ __forceinline__ uint32_t byte_flags_to_nibble(uint32_t f) { return (((f >> 7) * 0x204081u) >> 21) & 0xFu; }
-
-// Threshold of a bond: active iff its 32-bit uniform w < thr (thr <= 2^32).
-// w's top byte comes from the BOND stream, its low 24 bits (only needed on
-// a tie of the top bytes) from the TIE stream.
-struct ByteCompare {
-    uint32_t t8, t24;
-    bool all, none;
-    __device__ __forceinline__ explicit ByteCompare(uint64_t thr)
-        : t8((uint32_t)(thr >> 24)), t24((uint32_t)(thr & 0xFFFFFFu)), all(thr >= (1ull << 32)), none(thr == 0) {}
-};
-
-// Low 24 bits of the TIE-stream word of bond id 48 c + 16 g + 4 f + q.
-__device__ __forceinline__ uint32_t tie_bits(uint64_t seed, uint32_t sweep, int64_t cell, int g, int f, int q)
-{
-    const uint4 w = philox_call(seed, sweep, TAG_TIE, 12 * (uint64_t)cell + 4 * g + f);
-    return word_of(w, q) & 0xFFFFFFu;
 }
 
 // Flip bits of the tile's sites: bits 16 c .. 16 c + 15 of the FLIP stream

@@ -52,14 +52,6 @@ __host__ __device__ constexpr bool vec_stage_shared(int TX, int TY, int TZ)
     return vec_stage_bytes(TX, TY, TZ) <= (size_t)core_shared_words(TX * TY * TZ) * 4;
 }
 
-// 2^x, relative error at most 2^-22 (PTX ISA, ex2.approx.ftz.f32).
-__device__ __forceinline__ float exp2_approx(float x)
-{
-    float r;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-
 // Margin of the bond shortcut below, in units of 1/256 of probability.  The
 // evaluation errs by at most 2e-4 there: 2^-22 of ex2, 2^-22 in its argument
 // y log2 e (which moves exp(-y) by y exp(-y) 2^-22), and the rounding of q.
@@ -69,7 +61,7 @@ __device__ __forceinline__ float exp2_approx(float x)
 template <typename T>
 __device__ __forceinline__ float shortcut_margin(double K2)
 {
-    return sizeof(T) == 4 ? 1e-3f : 1e-3f + 4e-4f * (float)K2;
+    return sizeof(T) == 4 ? SHORTCUT_MARGIN : SHORTCUT_MARGIN + 4e-4f * (float)K2;
 }
 
 // Registers: two 512-thread blocks' worth of warps per SM.
