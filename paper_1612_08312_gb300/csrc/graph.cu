@@ -169,9 +169,11 @@ __global__ void __launch_bounds__(GB_THREADS) graph_proj_kernel(const __grid_con
 // measured slower: a warp's lanes then unite the bonds of the same few sites
 // at once.)  The bonds are decided first, all sites and spins loaded together
 // (bond after bond, each waited for its own sites, spins and unions), then the
-// active ones are united in a loop of their own.
+// active ones are united in a loop of their own: chains of dependent reads,
+// for which every warp the SM holds counts (simple cubic L = 256, a sweep with
+// 48, 40 and 32 registers: 697, 636 and 568 us).
 template <int NC, typename T>
-__global__ void __launch_bounds__(GB_THREADS) graph_bond_kernel(const __grid_constant__ GraphDev G)
+__global__ void __launch_bounds__(GB_THREADS, NC == 1 ? 8 : 4) graph_bond_kernel(const __grid_constant__ GraphDev G)
 {
     overlap_begin();
     const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -225,37 +227,40 @@ __global__ void __launch_bounds__(GB_THREADS) graph_bond_kernel(const __grid_con
         }
         const uint32_t cand = (act | tie) & pres;
         const int8_t *sp = static_cast<const int8_t *>(G.spins);
-        int si[16], sj[16];
-        if (!G.L && nq == 16) {  // the list in 16-byte loads
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int4 i = __ldg(reinterpret_cast<const int4 *>(G.bi + e0) + k);
-                const int4 j = __ldg(reinterpret_cast<const int4 *>(G.bj + e0) + k);
-                si[4 * k] = i.x;
-                si[4 * k + 1] = i.y;
-                si[4 * k + 2] = i.z;
-                si[4 * k + 3] = i.w;
-                sj[4 * k] = j.x;
-                sj[4 * k + 1] = j.y;
-                sj[4 * k + 2] = j.z;
-                sj[4 * k + 3] = j.w;
-            }
-        } else {
-#pragma unroll
-            for (int q = 0; q < 16; ++q) {
-                si[q] = sj[q] = 0;
-                if ((cand >> q) & 1u) ends(q, si[q], sj[q]);
-            }
-        }
         uint32_t same = 0;
 #pragma unroll
-        for (int q = 0; q < 16; ++q) {
-            if (!((cand >> q) & 1u)) continue;
-            si[q] = sp[si[q]];
-            sj[q] = sp[sj[q]];
-        }  // (a bond that is no candidate is masked out below)
+        for (int h = 0; h < 16; h += 8) {
+            int si[8], sj[8];
+            if (!G.L && nq == 16) {  // the list in 16-byte loads
 #pragma unroll
-        for (int q = 0; q < 16; ++q) same |= (si[q] == sj[q] ? 1u : 0u) << q;
+                for (int k = 0; k < 2; ++k) {
+                    const int4 i = __ldg(reinterpret_cast<const int4 *>(G.bi + e0 + h) + k);
+                    const int4 j = __ldg(reinterpret_cast<const int4 *>(G.bj + e0 + h) + k);
+                    si[4 * k] = i.x;
+                    si[4 * k + 1] = i.y;
+                    si[4 * k + 2] = i.z;
+                    si[4 * k + 3] = i.w;
+                    sj[4 * k] = j.x;
+                    sj[4 * k + 1] = j.y;
+                    sj[4 * k + 2] = j.z;
+                    sj[4 * k + 3] = j.w;
+                }
+            } else {
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    si[q] = sj[q] = 0;
+                    if ((cand >> (h + q)) & 1u) ends(h + q, si[q], sj[q]);
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                if (!((cand >> (h + q)) & 1u)) continue;
+                si[q] = sp[si[q]];
+                sj[q] = sp[sj[q]];
+            }  // (a bond that is no candidate is masked out below)
+#pragma unroll
+            for (int q = 0; q < 8; ++q) same |= (si[q] == sj[q] ? 1u : 0u) << (h + q);
+        }
         act &= same & pres;
         tie &= same & pres;
         for (uint32_t k = tie; k; k &= k - 1) {
@@ -574,7 +579,7 @@ struct GraphEngine {
         nbond = (unsigned)std::max<int64_t>(1, cdiv(nchunk, GB_THREADS));
         nsite = (unsigned)cdiv(N, GB_THREADS);
         nproj = (unsigned)std::min<int64_t>(cdiv(N, GB_THREADS), 152 * 8);
-        nmeas = (unsigned)std::min<int64_t>(cdiv(std::max(N, NB), GB_THREADS), 152 * 8);
+        nmeas = (unsigned)std::min<int64_t>(cdiv(std::max(N, NB), GB_THREADS), model == PYRO_ISING ? 152 * 4 : 152 * 8);
         struct {
             void **p;
             size_t bytes;
