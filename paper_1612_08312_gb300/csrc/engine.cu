@@ -256,7 +256,17 @@ static int64_t tiles_of(int L, const TileShape &t)
 TileShape default_tile(const int *Ls, int R, int model)
 {
     int64_t cells = 0;
-    for (int r = 0; r < R; ++r) cells += (int64_t)Ls[r] * Ls[r] * Ls[r];
+    int size[MAX_REPS], times[MAX_REPS], n = 0;  // the distinct sizes
+    for (int r = 0; r < R; ++r) {
+        cells += (int64_t)Ls[r] * Ls[r] * Ls[r];
+        int k = 0;
+        while (k < n && size[k] != Ls[r]) ++k;
+        if (k == n) {
+            size[n] = Ls[r];
+            times[n++] = 0;
+        }
+        ++times[k];
+    }
     const int cap = cells > 512 && cells <= 65536 ? 64 : (model == PYRO_ISING ? 256 : 128);
     const double w = model == PYRO_ISING ? 1.2 : 0.55;
     TileShape best{1, 1, 1};
@@ -267,12 +277,12 @@ TileShape default_tile(const int *Ls, int R, int model)
                 const int nt = tx * ty * tz;
                 if (nt > cap) continue;
                 double cost = 0.0;
-                for (int r = 0; r < R; ++r) {
+                for (int k = 0; k < n; ++k) {
                     double f = 1.0;
-                    if (tx < Ls[r]) f += w / tx;
-                    if (ty < Ls[r]) f += w / ty;
-                    if (tz < Ls[r]) f += w / tz;
-                    cost += f * (double)tiles_of(Ls[r], TileShape{tx, ty, tz}) * std::max(nt, 32);
+                    if (tx < size[k]) f += w / tx;
+                    if (ty < size[k]) f += w / ty;
+                    if (tz < size[k]) f += w / tz;
+                    cost += f * times[k] * (double)tiles_of(size[k], TileShape{tx, ty, tz}) * std::max(nt, 32);
                 }
                 // equal costs: fewer threads, then the longer x edge
                 if (best_cost < 0.0 || cost < best_cost * (1.0 - 1e-9) ||
