@@ -55,38 +55,39 @@ __device__ __forceinline__ int label_link_if(bool on, int hi, int lo)
                  : "memory");
     return old;
 }
-// Cell of a name less the base, and its site index 16 t + s (exact for up to
-// 512 cells).
-__device__ __forceinline__ int name_cell(int off) { return ((off >> 2) * 61681) >> 20; }
-__device__ __forceinline__ int name_site(int off) { return (off >> 2) - name_cell(off); }
+// Cell t of a label's word 17 t + s (exact for up to 512 cells).
+__device__ __forceinline__ int word_cell(int word) { return (word * 61681) >> 20; }
 
 // Iteration bound of one union (4096).  A test can lower it (to 0) through
 // pyro_debug_set to exercise the bound-exceeded status path.
 static __constant__ int c_unite_bound = 4096;
 
-// Union of the clusters of a and b in shared memory.  Both finds walk in
-// lockstep, one step of each per iteration without a branch (the label of a
+// Unions of the clusters of a0 and b0 and of a1 and b1 in shared memory.  All
+// four finds walk in lockstep, one step of each per iteration (the label of a
 // root is its own name, so a find that has arrived stays); they write nothing
 // on the way.  Returns false if the iteration bound was hit.
-__device__ __forceinline__ bool sunite(int a, int b)
+__device__ __forceinline__ bool sunite2(int a0, int b0, int a1, int b1)
 {
-    const int bound = c_unite_bound;
+    int a[2] = {a0, a1}, b[2] = {b0, b1};
+    const int bound = c_unite_bound * 16;
 #pragma unroll 1
     for (int it = 0; it < bound; ++it) {
-#pragma unroll 1
-        for (int st = 0; st < 65536; ++st) {
-            const int ga = label_get(a), gb = label_get(b);
-            if (ga == a && gb == b) break;
-            a = ga;
-            b = gb;
+        int ga[2], gb[2];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            ga[k] = label_get(a[k]);
+            gb[k] = label_get(b[k]);
         }
-        if (a == b) return true;
-        const int lo = min(a, b), hi = max(a, b);
-        const int old = label_link(hi, lo);
-        if (old == hi) return true;
-        // hi had been linked meanwhile: unite lo with its new parent
-        a = lo;
-        b = old;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const bool arrived = ga[k] == a[k] && gb[k] == b[k];
+            const int lo = min(ga[k], gb[k]), hi = max(ga[k], gb[k]);
+            // (not a root any more: its new parent)
+            const int old = label_link_if(arrived && lo != hi, hi, lo);
+            a[k] = lo;
+            b[k] = old == hi && arrived ? lo : old;  // united: the same twice
+        }
+        if (a[0] == b[0] && a[1] == b[1]) return true;
     }
     return false;
 }

@@ -256,13 +256,10 @@ constexpr PairTable make_pair_table()
 }
 static __device__ const PairTable pair_table = make_pair_table();
 
-// Vertices v of the down tetrahedron of f whose cell is a backward step along
-// axis d (bit v).
-__host__ __device__ constexpr uint32_t vertex_axis_mask(int f, int d)
+// The same of all four tetrahedra (bit 6 f + k).
+__host__ __device__ constexpr uint32_t leaving_pairs(int d)
 {
-    uint32_t m = 0;
-    for (int v = 0; v < 4; ++v) m |= (uint32_t)((down_mask(f, v) >> d) & 1) << v;
-    return m;
+    return pair_axis_mask(0, d) | (pair_axis_mask(1, d) << 6) | (pair_axis_mask(2, d) << 12) | (pair_axis_mask(3, d) << 18);
 }
 
 // Sites (bit 4 g + v) of a cell that belong to down tetrahedra reaching across
@@ -324,6 +321,11 @@ __device__ __forceinline__ void core_prologue(const CoreSmem &s)
     for (int i = threadIdx.x; i < 64; i += blockDim.x) s.lut[i] = tet_table.e[i];
 }
 
+// The code of a tile-local root without a slot is its label's word, 17 t + s; the
+// codes of the slots follow from the next multiple of 32.
+__host__ __device__ constexpr int slot_code(int nt) { return (17 * nt + 31) & ~31; }
+static_assert(slot_code(512) + 16 * 512 < 65536, "codes are 16-bit");
+
 // Entries at or above this are codes, not names.
 constexpr int IS_CODE = 1 << 20;
 // Synchronous rounds of the resolution before the walks.
@@ -360,17 +362,13 @@ __device__ __forceinline__ void local_core(const TileCtx &c, const Rep &R, const
     // the down tetrahedra join every vertex v to the smallest vertex connected
     // to it: pairs with a vertex across a backward tile face are left to the
     // crossing unions, the others are united here
-    uint32_t dntab[4];
-    uint32_t cross = 0, inside[4];
+    uint32_t span = 0, leave = 0;  // bit 6 f + k: pair k of tetrahedron f
 #pragma unroll
-    for (int f = 0; f < 4; ++f) {
-        dntab[f] = s.lut[down_tet_index(C, Bg, f)];
-        const uint32_t leave = ((out & 1u) ? pair_axis_mask(f, 0) : 0u) | ((out & 2u) ? pair_axis_mask(f, 1) : 0u) |
-                               ((out & 4u) ? pair_axis_mask(f, 2) : 0u);
-        cross |= ((dntab[f] >> 16) & leave & 0x3Fu) << (6 * f);
-        inside[f] = ~(((out & 1u) ? vertex_axis_mask(f, 0) : 0u) | ((out & 2u) ? vertex_axis_mask(f, 1) : 0u) |
-                      ((out & 4u) ? vertex_axis_mask(f, 2) : 0u));
-    }
+    for (int f = 0; f < 4; ++f) span |= ((s.lut[down_tet_index(C, Bg, f)] >> 16) & 0x3Fu) << (6 * f);
+    if (out & 1u) leave |= leaving_pairs(0);
+    if (out & 2u) leave |= leaving_pairs(1);
+    if (out & 4u) leave |= leaving_pairs(2);
+    const uint32_t in = span & ~leave, cross = span & leave;
     __syncthreads();  // labels initialised
     // First pass over all pairs, without finds: each links the larger of its
     // ends' parents under the other if that is a root still (seven pairs of
@@ -389,11 +387,16 @@ __device__ __forceinline__ void local_core(const TileCtx &c, const Rep &R, const
         int a[3], b[3];
 #pragma unroll
         for (int v = 1; v < 4; ++v) {
-            const uint32_t rv = (dntab[f] >> (2 * v)) & 3u;
-            const bool on = rv != (uint32_t)v && ((inside[f] >> v) & (inside[f] >> rv) & 1u);
-            // (no pair: the same label twice)
-            a[v - 1] = label_get(!on ? me : rv == 0 ? name[0] : rv == 1 ? name[1] : name[2]);
-            b[v - 1] = label_get(!on ? me : name[v]);
+            // at most one pair (u, v), u < v, spans; none: the same label twice
+            int ea = me, eb = me;
+#pragma unroll
+            for (int u = 0; u < v; ++u)
+                if ((in >> (6 * f + pair_index(u, v))) & 1u) {
+                    ea = name[u];
+                    eb = name[v];
+                }
+            a[v - 1] = label_get(ea);
+            b[v - 1] = label_get(eb);
         }
 #pragma unroll
         for (int v = 0; v < 3; ++v) {
@@ -414,9 +417,9 @@ __device__ __forceinline__ void local_core(const TileCtx &c, const Rep &R, const
     __syncthreads();  // pairs listed
     bool ok = true;
     const int np = s.pcount[0];
-    for (int e = threadIdx.x; e < np; e += nt) {
-        const uint32_t pr = s.plist[e];
-        ok &= sunite((int)(pr & 0xFFFFu), (int)(pr >> 16));
+    for (int e = threadIdx.x; e < np; e += 2 * nt) {
+        const uint32_t p0 = s.plist[e], p1 = e + nt < np ? s.plist[e + nt] : p0;
+        ok &= sunite2((int)(p0 & 0xFFFFu), (int)(p0 >> 16), (int)(p1 & 0xFFFFu), (int)(p1 >> 16));
     }
     __syncthreads();  // all unions done
     if (!ok) atomicOr(&R.st->status, ST_NOCONVERGE);
@@ -507,7 +510,7 @@ __device__ __forceinline__ void local_core(const TileCtx &c, const Rep &R, const
             const int q = __ffs(marked) - 1;
             marked &= marked - 1;
             P[slot] = (int32_t)(16 * c.cell) + q;
-            label_set(me + 4 * q, IS_CODE + 16 * nt + slot);
+            label_set(me + 4 * q, IS_CODE + slot_code(nt) + slot);
             ++slot;
         }
     }
@@ -526,7 +529,7 @@ __device__ __forceinline__ void local_core(const TileCtx &c, const Rep &R, const
         for (int v = 0; v < 4; ++v) {
             const uint32_t rv = (uptab[f] >> (2 * v)) & 3u;
             const int e = ent[4 * f + v];
-            uint32_t r = e < IS_CODE ? (uint32_t)name_site(e - s.lab) : (uint32_t)(e - IS_CODE);
+            uint32_t r = e < IS_CODE ? (uint32_t)(e - s.lab) >> 2 : (uint32_t)(e - IS_CODE);
 #pragma unroll
             for (int u = 0; u < v; ++u)
                 if (rv == (uint32_t)u) r = code[u];
@@ -610,13 +613,13 @@ __device__ __forceinline__ uint32_t tile_of(const Rep &R, const Batch &B, int x,
 // Slot of site s of cell (x, y, z), an end of a crossing bond.
 __device__ __forceinline__ uint32_t crossing_slot(const Rep &R, const Batch &B, int x, int y, int z, int s)
 {
-    const uint32_t L = (uint32_t)R.L, ns = 16u * B.TX * B.TY * B.TZ;  // (N < 2^31)
+    const uint32_t L = (uint32_t)R.L, nt = (uint32_t)(B.TX * B.TY * B.TZ);  // (N < 2^31)
     const uint32_t code = R.L16[16 * ((uint32_t)x + L * ((uint32_t)y + L * (uint32_t)z)) + (uint32_t)s];
-    return tile_of(R, B, x, y, z) * ns + (code - ns);
+    return tile_of(R, B, x, y, z) * (16 * nt) + (code - (uint32_t)slot_code((int)nt));
 }
 
-// Shared-memory bytes of the flip stage: the cells' flip words and the slots'.
-__host__ __device__ constexpr size_t resolve_smem_bytes(int nt) { return (size_t)nt * 4 + 16; }
+// Shared-memory bytes of the flip stage: a bit per code.
+__host__ __device__ constexpr size_t resolve_smem_bytes(int nt) { return (size_t)slot_code(nt) / 8 + (size_t)nt * 2 + 16; }
 
 // Global index of the cluster root of every site of the calling thread's
 // (valid) cell.
@@ -626,41 +629,47 @@ __device__ __forceinline__ void resolve_cell(const TileCtx &c, const Rep &R, int
     const uint4 a0 = src[0], a1 = src[1];
     const uint32_t w[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
     const uint32_t *P = reinterpret_cast<const uint32_t *>(R.P);
-    const int ns = 16 * c.nt;
+    const int base = slot_code(c.nt);
 #pragma unroll
     for (int s = 0; s < 16; ++s) {
         const int code = (int)((w[s >> 1] >> (16 * (s & 1))) & 0xFFFFu);
-        if (code >= ns) {
-            root[s] = (int)slot_root(P, P[(int64_t)tile * ns + (code - ns)]);
+        if (code >= base) {
+            root[s] = (int)slot_root(P, P[(int64_t)tile * (16 * c.nt) + (code - base)]);
         } else {
-            const int lc = code >> 4;
+            const int lc = word_cell(code);
             const int rx = c.ox + (lc & (c.TX - 1));
             const int ry = c.oy + ((lc >> c.lTX) & (c.TY - 1));
             const int rz = c.oz + (lc >> (c.lTX + c.lTY));
-            root[s] = 16 * (rx + c.L * (ry + c.L * rz)) + (code & 15);
+            root[s] = 16 * (rx + c.L * (ry + c.L * rz)) + (code - 17 * lc);
         }
     }
 }
 
 // Flip mask of the calling thread's cell (bit s = site 16 c + s flips): each
-// site's code indexes the flip bits of the tile's sites, followed by those of
-// its slots' clusters, which the block shares.  Called by every thread of the
-// block.
+// site's code indexes a bit array the block shares, the flip bits of the
+// tile's sites (17 bits a cell), then those of its slots' clusters.  Called by
+// every thread of the block.
 __device__ __forceinline__ uint32_t cell_flip_mask(const TileCtx &c, const Rep &R, int tile, int *smem)
 {
-    uint16_t *fx = reinterpret_cast<uint16_t *>(smem);
+    uint32_t *fx = reinterpret_cast<uint32_t *>(smem);
+    const int words = slot_code(c.nt) >> 5;
+    for (int i = c.t; i < words; i += c.nt) fx[i] = 0;
     const uint4 *src = reinterpret_cast<const uint4 *>(R.L16 + 16 * c.cell);
     const uint4 a0 = src[0], a1 = src[1];
     const uint32_t w[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-    fx[c.t] = R.F[c.cell];
+    const uint32_t f = R.F[c.cell];
     const uint16_t *sf = reinterpret_cast<const uint16_t *>(R.sflip) + (int64_t)tile * c.nt;
-    if (16 * c.t < R.nslots[tile]) fx[c.nt + c.t] = sf[c.t];
+    if (16 * c.t < R.nslots[tile]) reinterpret_cast<uint16_t *>(fx + words)[c.t] = sf[c.t];
+    __syncthreads();
+    const int bit = 17 * c.t;
+    atomicOr(fx + (bit >> 5), f << (bit & 31));
+    if ((bit & 31) > 16) atomicOr(fx + (bit >> 5) + 1, f >> (32 - (bit & 31)));
     __syncthreads();
     uint32_t flip = 0;
 #pragma unroll
     for (int s = 0; s < 16; ++s) {
         const int code = (int)((w[s >> 1] >> (16 * (s & 1))) & 0xFFFFu);
-        flip |= ((fx[code >> 4] >> (code & 15)) & 1u) << s;
+        flip |= ((fx[code >> 5] >> (code & 31)) & 1u) << s;
     }
     return flip;
 }
