@@ -239,20 +239,22 @@ static int64_t tiles_of(int L, const TileShape &t)
 }
 
 // The tile whose modelled sweep is cheapest over the set of lattices, among
-// the power-of-two tiles of at most 256 cells (Ising) or 128 (n-vector).  The
-// edges need not divide L.  Model: every tile costs its cells, padded to the
-// lattice's edge and to a warp, times 1 + w (1/TX + 1/TY + 1/TZ) over the axes
-// it does not cover, for the crossing unions of its faces; w is the measured
-// cost of the crossing phase per face cell over the local phase's per cell
-// (L = 128, Ising: 186 us over 0.5 face cells per cell against 240 us; n = 3:
-// 183 over 0.625 against 534).  Before, the edges were the largest powers of
-// two dividing L: one-cell tiles of one thread for odd L (Ising L = 45: 951 us
-// a sweep, now 99; Heisenberg FP64 L = 50, tile 2 x 2 x 2: 2,521 us, now 814).
-// Sets of at most 65,536 cells do not fill the GPU and are bound by a block's
-// latency, which grows with its threads: at most 64 cells there (Ising
-// L = 16: 76 us a sweep with 4 x 4 x 4, 84 with 16 x 4 x 4 or 8 x 8 x 4; L = 32:
-// 80 and 92), except where one lattice is hardly more than one tile (L = 8:
-// 71 us with 4 x 4 x 4, 65 with 8 x 8 x 4).
+// the power-of-two tiles of at most `cap` cells.  The edges need not divide L.
+// Model: every tile costs its cells, padded to the lattice's edge and to a
+// warp, times 1 + w (1/TX + 1/TY + 1/TZ) over the axes it does not cover, for the
+// crossing unions of its faces; w is the measured cost of the crossing phase
+// per face cell over the local phase's per cell (Ising L = 256: 640 us over 0.5
+// face cells per cell against 1,449; n = 3, L = 128: 91 over 0.5 against 268).
+// Before, the edges were the largest powers of two dividing L: one-cell tiles
+// of one thread for odd L (Ising L = 45: 951 us a sweep then, 99 with this).
+//
+// cap.  Sets that do not fill the GPU are bound by a block's latency, which
+// grows with its threads; sets that do, by the crossing work, which falls with
+// the tile.  A sweep in us at 64 / 128 / 256 cells: Ising L = 32 39.5 / 39.2 / 40.2,
+// L = 64 78.9 / 72.4 / 74.5, L = 128 (phases) - / 364 / 352 and 367 at 512; n = 3
+// L = 32 50.0 / 52.2 / 55.4, L = 64 112.8 / 109.4 / 108.7, L = 128 (phases)
+// 715 / 652 / 621.  One lattice that a block of 512 cells covers has no crossing
+// work at all: L = 8 25.4, and 27.9 with two tiles of 256.
 TileShape default_tile(const int *Ls, int R, int model)
 {
     int64_t cells = 0;
@@ -267,8 +269,9 @@ TileShape default_tile(const int *Ls, int R, int model)
         }
         ++times[k];
     }
-    const int cap = cells > 512 && cells <= 65536 ? 64 : (model == PYRO_ISING ? 256 : 128);
-    const double w = model == PYRO_ISING ? 1.2 : 0.55;
+    const int cap = model == PYRO_ISING ? (cells <= 512 ? 512 : cells <= 300000 ? 128 : 256)
+                                        : (cells <= 512 ? 256 : cells <= 65536 ? 64 : 256);
+    const double w = model == PYRO_ISING ? 0.9 : 0.66;
     TileShape best{1, 1, 1};
     double best_cost = -1.0;
     for (int tx = 32; tx >= 1; tx /= 2)
