@@ -402,8 +402,10 @@ int64_t pyro_graph_num_bonds(pyro_graph g);
 /* Wait for the handle's work; PYRO_E_NOCONVERGE if a union hit its bound. */
 int pyro_graph_sync(pyro_graph g);
 void *pyro_graph_get_stream(pyro_graph g);
-/* Kernel launches issued so far (four per Ising sweep, five for n > 1,
- * two per pyro_graph_measure, one at creation). */
+/* Kernel launches issued so far (four per Ising sweep of a bond list, six on
+ * the simple-cubic lattice, five for n > 1, two per pyro_graph_measure, one at
+ * creation; one per call that copies the spins or the labels of the simple-
+ * cubic Ising lattice, whose device layout is packed). */
 uint64_t pyro_graph_launch_count(pyro_graph g);
 /* Free the lattice's device memory (after its stream's work) and the handle. */
 void pyro_graph_destroy(pyro_graph g);

@@ -3,7 +3,8 @@
 // neighbour table), the simple-cubic lattice with implicit bonds (Sec. 3.4,
 // the comparison lattice of Eq. 5-6), either one optionally diluted by a
 // site mask and a bond mask (Sec. 4).  Ising (n = 1) and the embedded-
-// cluster n-vector models (n = 2, 3), conventions as in include/pyro.h.
+// cluster n-vector models (n = 2, 3), conventions as in include/pyro.h.  The
+// Ising model on the simple-cubic lattice has a sweep of its own (sc.cuh).
 //
 // A sweep is four launches (five for n > 1):
 //   graph_proj   (n > 1) the sweep's axis r and every projection s_i . r;
@@ -33,12 +34,13 @@
 #include "engine.h"
 #include "launch.cuh"
 #include "nvec.cuh"
+#include "sc.cuh"
 
 namespace pyro {
 
 struct GraphDev {
     int64_t N, NB, nocc;
-    int L;     // simple-cubic edge; 0 = explicit bond list
+    int L;     // simple-cubic edge (n > 1; Ising: sc.cuh); 0 = explicit bond list
     int nc;    // spin components
     const int32_t *bi, *bj;
     const uint32_t *present;  // bond bit set (bond mask and both ends occupied), or null
@@ -188,14 +190,14 @@ __global__ void __launch_bounds__(GB_THREADS, NC == 1 ? 8 : 4) graph_bond_kernel
     if (G.present) pres &= G.present[e0 >> 5] >> (e0 & 31);
     // simple cubic: bond 3 s + d, from the chunk's first
     int s0 = 0, d0 = 0, x0 = 0, y0 = 0, z0 = 0;
-    if (G.L) {
+    if (NC > 1 && G.L) {
         const uint64_t s = (uint64_t)e0 / 3u;
         s0 = (int)s;
         d0 = (int)((uint64_t)e0 - 3u * s);
         sc_coords(G.L, s0, x0, y0, z0);
     }
     const auto ends = [&](int q, int &i, int &j) {  // of bond e0 + q, q < nq
-        if (G.L) {
+        if (NC > 1 && G.L) {
             int x = x0, y = y0, z = z0, ds = (d0 + q) / 3;
             const int d = d0 + q - 3 * ds;
             i = s0 + ds;
@@ -231,7 +233,7 @@ __global__ void __launch_bounds__(GB_THREADS, NC == 1 ? 8 : 4) graph_bond_kernel
 #pragma unroll
         for (int h = 0; h < 16; h += 8) {
             int si[8], sj[8];
-            if (!G.L && nq == 16) {  // the list in 16-byte loads
+            if (nq == 16) {  // the list in 16-byte loads
 #pragma unroll
                 for (int k = 0; k < 2; ++k) {
                     const int4 i = __ldg(reinterpret_cast<const int4 *>(G.bi + e0 + h) + k);
@@ -376,31 +378,18 @@ __global__ void __launch_bounds__(GB_THREADS) graph_measure_kernel(const __grid_
 #pragma unroll 4
         for (int64_t i = t0; i < G.N; i += stride)
             if (!G.occ || bit_of(G.occ, i)) m += s[i];
-        if (G.L) {
-#pragma unroll 4
-            for (int64_t i = t0; i < G.N; i += stride) {
-                int x, y, z;
-                sc_coords(G.L, (int)i, x, y, z);
-#pragma unroll
-                for (int d = 0; d < 3; ++d) {
-                    if (G.present && !bit_of(G.present, 3 * i + d)) continue;
-                    e += s[i] == s[sc_next(G.L, (int)i, x, y, z, d)] ? 1 : -1;
-                }
-            }
-        } else {
-            // four bonds per thread in 16-byte loads, two fours in flight
-            const int4 *bi = reinterpret_cast<const int4 *>(G.bi), *bj = reinterpret_cast<const int4 *>(G.bj);
+        // four bonds per thread in 16-byte loads, two fours in flight
+        const int4 *bi = reinterpret_cast<const int4 *>(G.bi), *bj = reinterpret_cast<const int4 *>(G.bj);
 #pragma unroll 2
-            for (int64_t b = t0; b < G.NB >> 2; b += stride) {
-                const int4 i = __ldg(bi + b), j = __ldg(bj + b);
-                const uint32_t pres = G.present ? (G.present[b >> 3] >> (4 * (b & 7))) & 0xFu : 0xFu;
-                const uint32_t diff = (s[i.x] != s[j.x] ? 1u : 0u) | (s[i.y] != s[j.y] ? 2u : 0u) |
-                                      (s[i.z] != s[j.z] ? 4u : 0u) | (s[i.w] != s[j.w] ? 8u : 0u);
-                e += __popc(pres) - 2 * __popc(pres & diff);
-            }
-            const int64_t b = (G.NB & ~(int64_t)3) + t0;
-            if (b < G.NB && (!G.present || bit_of(G.present, b))) e += s[G.bi[b]] == s[G.bj[b]] ? 1 : -1;
+        for (int64_t b = t0; b < G.NB >> 2; b += stride) {
+            const int4 i = __ldg(bi + b), j = __ldg(bj + b);
+            const uint32_t pres = G.present ? (G.present[b >> 3] >> (4 * (b & 7))) & 0xFu : 0xFu;
+            const uint32_t diff = (s[i.x] != s[j.x] ? 1u : 0u) | (s[i.y] != s[j.y] ? 2u : 0u) |
+                                  (s[i.z] != s[j.z] ? 4u : 0u) | (s[i.w] != s[j.w] ? 8u : 0u);
+            e += __popc(pres) - 2 * __popc(pres & diff);
         }
+        const int64_t b = (G.NB & ~(int64_t)3) + t0;
+        if (b < G.NB && (!G.present || bit_of(G.present, b))) e += s[G.bi[b]] == s[G.bj[b]] ? 1 : -1;
         v[0] = (double)e;
         v[1] = (double)m;
     } else {
@@ -535,6 +524,9 @@ struct GraphEngine {
     double beta = -1.0;
     unsigned nproj = 1, nbond = 1, nsite = 1, nmeas = 1;
     GraphKernels k{};
+    ScDev sc{};               // Ising on the simple-cubic lattice
+    unsigned sc_tiles = 0;    // its tiles; 0 = the generic kernels
+    bool swept = false;
 
     cudaError_t alloc(void **p, size_t bytes)
     {
@@ -568,6 +560,7 @@ struct GraphEngine {
             if (e != cudaSuccess) return err = "stream creation", e;
             own_stream = true;
         }
+        if (c.sc_L && model == PYRO_ISING) return sc_setup(c, N, present, occ, nocc, err);
         G.N = N;
         G.NB = NB;
         G.nocc = nocc;
@@ -638,13 +631,168 @@ struct GraphEngine {
     {
         if (b == beta) return cudaSuccess;
         beta = b;
-        G.thr = ising_threshold(b, G.J);
+        G.thr = sc.thr = ising_threshold(b, G.J);
         G.K2 = 2.0 * b * G.J;
         return cudaSuccess;
     }
 
+    // Tile of the simple-cubic sweep: the power-of-two tile of at most `cap`
+    // segments whose padded cost is least, each axis it does not cover adding its
+    // crossing faces (as default_tile in engine.cu).
+    void sc_tile()
+    {
+        const int64_t segs = (int64_t)sc.SX * sc.L * sc.L;
+        const int cap = segs > 256 && segs <= 16384 ? 64 : 256;
+        const auto along = [](int n, int t) { return (n + t - 1) / t; };
+        double best = -1.0;
+        for (int tx = 1; tx <= 8; tx *= 2)
+            for (int ty = 32; ty >= 1; ty /= 2)
+                for (int tz = 32; tz >= 1; tz /= 2) {
+                    const int nt = tx * ty * tz;
+                    if (nt > cap) continue;
+                    const int ax = along(sc.SX, tx), ay = along(sc.L, ty), az = along(sc.L, tz);
+                    double f = 1.0;
+                    if (ax > 1) f += 1.0 / (16.0 * tx);
+                    if (ay > 1) f += 1.0 / ty;
+                    if (az > 1) f += 1.0 / tz;
+                    const double cost = f * (double)ax * ay * az * std::max(nt, 32);
+                    if (best >= 0.0 && cost >= best * (1.0 - 1e-9)) continue;
+                    best = cost;
+                    sc.TX = tx;
+                    sc.TY = ty;
+                    sc.TZ = tz;
+                    sc.ntx = ax;
+                    sc.nty = ay;
+                    sc.ntz = az;
+                }
+        for (sc.lTX = 0; (1 << sc.lTX) < sc.TX;) ++sc.lTX;
+        for (sc.lTY = 0; (1 << sc.lTY) < sc.TY;) ++sc.lTY;
+        for (sc.lTZ = 0; (1 << sc.lTZ) < sc.TZ;) ++sc.lTZ;
+        // slots: every site of the segments on y and z faces, two of the others
+        const int face = sc.TX * (sc.TY * sc.TZ - std::max(0, sc.TY - 2) * std::max(0, sc.TZ - 2));
+        sc.nslot = (16 * face + 2 * (sc.TX * sc.TY * sc.TZ - face) + 31) & ~31;
+    }
+
+    size_t sc_flip_smem() const { return (size_t)slot_code(sc.TX * sc.TY * sc.TZ) / 8 + (size_t)sc.nslot / 8; }
+    unsigned sc_seg_blocks() const { return (unsigned)cdiv(sc.nsegs, 256); }
+
+    cudaError_t sc_setup(const pyro_graph_config &c, int64_t N, const std::vector<uint32_t> &present,
+                         const std::vector<uint32_t> &occ, int64_t nocc, std::string &err)
+    {
+        G.N = sc.N = N;
+        G.NB = 3 * N;
+        G.nocc = nocc;
+        G.nc = 1;
+        G.J = c.J;
+        sc.L = c.sc_L;
+        sc.SX = (sc.L + 15) / 16;
+        sc.nsegs = (int64_t)sc.SX * sc.L * sc.L;
+        sc.seed = c.seed;
+        sc_tile();
+        const int nt = sc.TX * sc.TY * sc.TZ;
+        sc_tiles = (unsigned)sc.ntx * (unsigned)sc.nty * (unsigned)sc.ntz;
+        nmeas = (unsigned)std::min<int64_t>(cdiv((int64_t)sc_tiles * nt, 256), 152 * 4);
+        const size_t segs = (size_t)sc.nsegs, mask = present.empty() ? 0 : segs * 2;
+        struct {
+            void **p;
+            size_t bytes;
+        } al[] = {{(void **)&sc.spins, segs * 2},
+                  {(void **)&sc.code, segs * 32},
+                  {(void **)&sc.P, (size_t)sc_tiles * sc.nslot * 4},
+                  {(void **)&sc.nslots, (size_t)sc_tiles * 4},
+                  {(void **)&sc.sflip, (size_t)sc_tiles * (sc.nslot / 8)},
+                  {(void **)&sc.cross, segs * 8},
+                  {(void **)&sc.fb, (size_t)cdiv(N, 128) * 16 + 16},
+                  {(void **)&sc.px, mask},
+                  {(void **)&sc.py, mask},
+                  {(void **)&sc.pz, mask},
+                  {(void **)&sc.occ, occ.empty() ? 0 : segs * 2},
+                  {(void **)&sc.bytes, (size_t)N},
+                  {(void **)&G.partials, (size_t)nmeas * 4 * sizeof(double)},
+                  {(void **)&G.st, sizeof(DevStats)}};
+        cudaError_t e;
+        for (auto &a : al) {
+            if (!a.bytes) continue;
+            e = alloc(a.p, a.bytes);
+            if (e != cudaSuccess) return err = "device allocation failed", e;
+        }
+        sc.partials = G.partials;
+        sc.st = G.st;
+        // the masks per segment
+        if (mask || !occ.empty()) {
+            std::vector<uint16_t> w[4];
+            for (auto &v : w) v.assign(segs, 0);
+            for (int64_t i = 0; i < N; ++i) {
+                const int64_t x = i % sc.L, seg = x / 16 + sc.SX * (i / sc.L);
+                const uint16_t b = (uint16_t)(1u << (x % 16));
+                for (int d = 0; d < 3 && mask; ++d)
+                    if ((present[(size_t)((3 * i + d) >> 5)] >> ((3 * i + d) & 31)) & 1u) w[d][(size_t)seg] |= b;
+                if (!occ.empty() && ((occ[(size_t)(i >> 5)] >> (i & 31)) & 1u)) w[3][(size_t)seg] |= b;
+            }
+            const uint16_t *dst[4] = {sc.px, sc.py, sc.pz, sc.occ};
+            for (int d = 0; d < 4; ++d) {
+                if (!dst[d]) continue;
+                e = cudaMemcpyAsync(const_cast<uint16_t *>(dst[d]), w[d].data(), segs * 2, cudaMemcpyHostToDevice, stream);
+                if (e == cudaSuccess) e = cudaStreamSynchronize(stream);  // (pageable source)
+                if (e != cudaSuccess) return err = "mask copy", e;
+            }
+        }
+        e = cudaMemsetAsync(G.st, 0, sizeof(DevStats), stream);
+        if (e != cudaSuccess) return err = "stats reset", e;
+        sc_init_kernel<<<sc_seg_blocks(), 256, 0, stream>>>(sc, c.start == PYRO_START_RANDOM);
+        ++launches;
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return err = "init launch", e;
+        e = cudaStreamSynchronize(stream);
+        if (e != cudaSuccess) return err = "set-up", e;
+        return cudaSuccess;
+    }
+
+    cudaError_t sc_sweeps(int64_t n)
+    {
+        const unsigned nt = (unsigned)(sc.TX * sc.TY * sc.TZ);
+        for (int64_t s = 0; s < n; ++s) {
+            launch_overlapped(sc_local_kernel, sc_tiles, nt, core_smem_bytes((int)nt), stream, sc);
+            launch_overlapped(sc_unite_kernel, sc_tiles, nt, (size_t)nt * 33 * 2, stream, sc);
+            launch_overlapped(sc_slot_flip_kernel, sc_tiles, SLOT_BLOCK, 0, stream, sc);
+            launch_overlapped(sc_flip_kernel, sc_tiles, nt, sc_flip_smem(), stream, sc);
+            launch_overlapped(sc_measure_kernel, nmeas, 256, 0, stream, sc, (int)sc_tiles);
+            launch_overlapped(graph_accumulate_kernel, 1, ACC_THREADS, 0, stream, G, (int)nmeas, 1);
+            launches += 6;
+            swept = true;
+        }
+        return cudaGetLastError();
+    }
+
+    // The spins as N bytes of +-1 in sc.bytes.
+    cudaError_t sc_unpack()
+    {
+        sc_unpack_kernel<<<sc_seg_blocks(), 256, 0, stream>>>(sc);
+        ++launches;
+        return cudaGetLastError();
+    }
+    cudaError_t sc_pack()
+    {
+        sc_pack_kernel<<<sc_seg_blocks(), 256, 0, stream>>>(sc);
+        ++launches;
+        return cudaGetLastError();
+    }
+
+    cudaError_t sc_labels()
+    {
+        if (!sc.labels) {
+            const cudaError_t e = alloc((void **)&sc.labels, (size_t)sc.N * 4);
+            if (e != cudaSuccess) return e;
+        }
+        sc_labels_kernel<<<sc_tiles, sc.TX * sc.TY * sc.TZ, 0, stream>>>(sc, swept);
+        ++launches;
+        lab_last = sc.labels;
+        return cudaGetLastError();
+    }
+
     cudaError_t sweeps(int64_t n)
     {
+        if (sc_tiles) return sc_sweeps(n);
         for (int64_t s = 0; s < n; ++s) {
             k.sweep(G, stream, nproj, nbond, nsite, nmeas);
             launch_overlapped(graph_accumulate_kernel, 1, ACC_THREADS, 0, stream, G, (int)nmeas, 1);
@@ -657,7 +805,8 @@ struct GraphEngine {
 
     cudaError_t measure()
     {
-        k.measure(G, stream, nmeas);
+        if (sc_tiles) launch_overlapped(sc_measure_kernel, nmeas, 256, 0, stream, sc, (int)sc_tiles);
+        else k.measure(G, stream, nmeas);
         launch_overlapped(graph_accumulate_kernel, 1, ACC_THREADS, 0, stream, G, (int)nmeas, 2);
         launches += 2;
         return cudaGetLastError();
@@ -896,7 +1045,9 @@ int pyro_graph_get_spins(pyro_graph g, void *host, size_t bytes)
     const int64_t N = e.G.N;
     if (e.model == PYRO_ISING) {
         if (bytes != (size_t)N) return gfail(PYRO_E_INVAL, "Ising spins need N bytes");
-        GRAPH_CUDA(cudaMemcpyAsync(host, e.G.spins, (size_t)N, cudaMemcpyDeviceToHost, e.stream), "spins copy");
+        if (e.sc_tiles) GRAPH_CUDA(e.sc_unpack(), "spins unpacking");
+        GRAPH_CUDA(cudaMemcpyAsync(host, e.sc_tiles ? e.sc.bytes : e.G.spins, (size_t)N, cudaMemcpyDeviceToHost, e.stream),
+                   "spins copy");
         return gfinish(e);
     }
     const int n = e.model;
@@ -924,7 +1075,9 @@ int pyro_graph_set_spins(pyro_graph g, const void *host, size_t bytes)
         unsigned bad = 0;  // branch-free, so that the check vectorises
         for (int64_t i = 0; i < N; ++i) bad |= (unsigned)((uint8_t)(s[i] + 1) & 0xFDu);  // 0 for -1 and +1 only
         if (bad) return gfail(PYRO_E_INVAL, "Ising spins must be +1 or -1");
-        GRAPH_CUDA(cudaMemcpyAsync(e.G.spins, host, (size_t)N, cudaMemcpyHostToDevice, e.stream), "spins copy");
+        GRAPH_CUDA(cudaMemcpyAsync(e.sc_tiles ? e.sc.bytes : e.G.spins, host, (size_t)N, cudaMemcpyHostToDevice, e.stream),
+                   "spins copy");
+        if (e.sc_tiles) GRAPH_CUDA(e.sc_pack(), "spins packing");
         GRAPH_CUDA(cudaStreamSynchronize(e.stream), "stream synchronize");
         return PYRO_OK;
     }
@@ -946,6 +1099,7 @@ int pyro_graph_get_labels(pyro_graph g, int32_t *host, int64_t n)
 {
     if (!g || !host) return gfail(PYRO_E_INVAL, "NULL argument");
     if (n != g->g.G.N) return gfail(PYRO_E_INVAL, "labels need N entries");
+    if (g->g.sc_tiles) GRAPH_CUDA(g->g.sc_labels(), "labels");
     GRAPH_CUDA(cudaMemcpyAsync(host, g->g.lab_last, (size_t)n * 4, cudaMemcpyDeviceToHost, g->g.stream), "labels copy");
     return gfinish(g->g);
 }

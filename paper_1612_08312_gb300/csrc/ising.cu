@@ -272,9 +272,6 @@ __global__ void __launch_bounds__(512, 4) boundary_unite_kernel(const __grid_con
     if (!ok) atomicOr(&R.st->status, ST_NOCONVERGE);
 }
 
-// Threads of a slot block.
-constexpr int SLOT_BLOCK = 128;
-
 // Phase 1, second launch: the flip bit of every slot's cluster (that of its
 // root site), 32 slots to a word.  All unions are done and this pass writes no
 // link, so the walks may take the cached read-only path.
@@ -290,30 +287,7 @@ __global__ void __launch_bounds__(SLOT_BLOCK) boundary_flip_kernel(const __grid_
     const uint32_t *own = P + tile * (16 * nt);
     // (a tile of one cell has half a word of slots)
     uint16_t *out = reinterpret_cast<uint16_t *>(R.sflip) + tile * nt;
-    // three slots per thread at a time, their walks in lockstep
-    const int lane = threadIdx.x & 31;
-    for (int k0 = threadIdx.x & ~31; k0 < n; k0 += 3 * SLOT_BLOCK) {
-        uint32_t v[3];
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            const int k = k0 + j * SLOT_BLOCK + lane;
-            v[j] = k < n ? __ldg(own + k) : 0u;
-        }
-#pragma unroll 1
-        for (int it = 0; it < (1 << 20) && ((v[0] | v[1] | v[2]) & SLOT_LINK); ++it)
-#pragma unroll
-            for (int j = 0; j < 3; ++j)
-                if (slot_linked(v[j])) v[j] = __ldg(P + (v[j] & ~SLOT_LINK));
-        uint32_t bit[3];
-#pragma unroll
-        for (int j = 0; j < 3; ++j) bit[j] = ((uint32_t)__ldg(R.F + (v[j] >> 4)) >> (v[j] & 15)) & 1u;
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            const int k = k0 + j * SLOT_BLOCK + lane;
-            const uint32_t word = __ballot_sync(0xffffffffu, bit[j]);
-            if ((lane & 15) == 0 && k < n) out[k >> 4] = (uint16_t)(word >> (lane & 16));
-        }
-    }
+    slot_flips(own, P, n, out, [&](uint32_t site) { return ((uint32_t)__ldg(R.F + (site >> 4)) >> (site & 15)) & 1u; });
 }
 
 // ------------------------------------------------------------ launchers --

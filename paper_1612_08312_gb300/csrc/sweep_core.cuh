@@ -331,6 +331,135 @@ constexpr int IS_CODE = 1 << 20;
 // Synchronous rounds of the resolution before the walks.
 constexpr int RESOLVE_ROUNDS = 1;
 
+// The second half of a tile's labelling, for a thread's 16 sites named me, me +
+// 4, ..: unites the listed pairs, resolves every representative (reps) to its
+// root, gives the roots of the sites in `ends` (which a crossing bond may end
+// on) a slot each in P (the root's site: site0 + q for the thread's q-th), and
+// returns in ent the codes of the representatives (entries below IS_CODE are
+// names of roots without a slot).  Called by every thread of the block.
+template <typename Ends>
+__device__ __forceinline__ void finish_labels(const CoreSmem &s, int nt, int me, uint32_t reps, const Ends &ends_of,
+                                              int32_t site0, int32_t *P, int32_t *nslots, int *status, int ent[16])
+{
+    __syncthreads();  // pairs listed
+    bool ok = true;
+    const int np = min(s.pcount[0], 15 * nt);
+    for (int e = threadIdx.x; e < np; e += 2 * nt) {
+        const uint32_t p0 = s.plist[e], p1 = e + nt < np ? s.plist[e + nt] : p0;
+        ok &= sunite2((int)(p0 & 0xFFFFu), (int)(p0 >> 16), (int)(p1 & 0xFFFFu), (int)(p1 >> 16));
+    }
+    __syncthreads();  // all unions done
+    if (!ok) atomicOr(status, ST_NOCONVERGE);
+    // Resolution: every representative's entry becomes its root's name.  No
+    // union changes the trees any more, and entries only move up them.
+    // RESOLVE_ROUNDS times all entries move to their grandparents together, a
+    // barrier after each; a representative whose parent is a root is done for
+    // good.  The few left on deeper chains are walked to their roots by their
+    // threads, three at a time, read-only (whatever the others write meanwhile,
+    // an entry is an ancestor).  The loads of a step are issued together: one
+    // representative after the other took 31 % of the kernel.  Ising local kernel
+    // at L = 256 with 0, 1, 2 rounds: 1,698, 1,595, 1,684 us (a round between the
+    // first pass and the listed pairs besides: 60 us slower than without).
+    uint32_t todo = reps;
+#pragma unroll 1
+    for (int it = 0; it < RESOLVE_ROUNDS; ++it) {
+        int p[16];
+#pragma unroll
+        for (int q = 0; q < 16; ++q) p[q] = label_get(me + 4 * q);
+        todo = 0;
+#pragma unroll
+        for (int q = 0; q < 16; ++q) {
+            const int gp = label_get(p[q]);
+            const bool move = ((reps >> q) & 1u) && gp != p[q];
+            label_set_if(move, me + 4 * q, gp);
+            todo |= (move ? 1u : 0u) << q;
+        }
+        __syncthreads();
+    }
+    bool walked = true;
+#pragma unroll 1
+    while (todo) {
+        int x[3], r[3];
+        const int q0 = __ffs(todo) - 1;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            x[k] = me + 4 * (todo ? __ffs(todo) - 1 : q0);
+            todo &= todo - 1;
+            r[k] = label_get(x[k]);
+        }
+#pragma unroll 1
+        for (int st = 0;; ++st) {
+            int p[3];
+            bool there = true;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                p[k] = label_get(r[k]);
+                there &= p[k] == r[k];
+            }
+            if (there) break;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) r[k] = p[k];
+            if (st == 16 * nt) {
+                walked = false;
+                break;
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) label_set(x[k], r[k]);
+    }
+    if (!walked) atomicOr(status, ST_NOCONVERGE);
+    __syncthreads();
+    // Mark the roots of the sites a crossing bond may end on: the root's own
+    // entry, its name, gets bit 0 set (every marker stores the same value).
+    // A site's entry is its root's name or its representative's, so two loads
+    // lead to the root whatever is marked meanwhile.
+    const uint32_t ends = ends_of();
+#pragma unroll
+    for (int q = 0; q < 16; ++q) ent[q] = label_get(me + 4 * q) & ~1;
+    if (ends) {
+#pragma unroll
+        for (int q = 0; q < 16; ++q) {
+            const bool end = (ends >> q) & 1u;
+            const int r = label_get(end ? ent[q] : me) & ~1;
+            label_set_if(end, r, r | 1);
+        }
+    }
+    __syncthreads();
+    // number the marked roots; a marked root's own entry becomes its code
+    {
+        uint32_t marked = 0;
+#pragma unroll
+        for (int q = 0; q < 16; ++q) marked |= (uint32_t)(label_get(me + 4 * q) & 1) << q;
+        const unsigned lanes = lanes_mask(nt);
+        const int lane = threadIdx.x & 31, last = 31 - __clz(lanes);
+        const int n = __popc(marked);
+        int incl = n;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(lanes, incl, o);
+            if (lane >= o) incl += v;
+        }
+        int base = 0;
+        if (lane == last && incl) base = atomicAdd(s.pcount + 1, incl);
+        int slot = __shfl_sync(lanes, base, last) + incl - n;
+#pragma unroll 1
+        while (marked) {
+            const int q = __ffs(marked) - 1;
+            marked &= marked - 1;
+            P[slot] = site0 + q;
+            label_set(me + 4 * q, IS_CODE + slot_code(nt) + slot);
+            ++slot;
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) *nslots = s.pcount[1];
+    // every site takes the code of its component's representative: the entry
+    // of its root (a code, or the name of a root without a slot)
+#pragma unroll
+    for (int q = 0; q < 16; ++q)
+        ent[q] = label_get(ent[q]);
+}
+
 // Tile-local labelling of one cell's sites from its active-bond groups.
 // Writes L16 (the code of each site), F (flip bits), the tile's slots and, for
 // face cells, dmask (the union pairs that leave the tile: bit 6 f + k, k the
@@ -414,125 +543,9 @@ __device__ __forceinline__ void local_core(const TileCtx &c, const Rep &R, const
         for (int k = 0; k < 12; ++k)
             if (rest[k]) s.plist[pos++] = rest[k];
     }
-    __syncthreads();  // pairs listed
-    bool ok = true;
-    const int np = s.pcount[0];
-    for (int e = threadIdx.x; e < np; e += 2 * nt) {
-        const uint32_t p0 = s.plist[e], p1 = e + nt < np ? s.plist[e + nt] : p0;
-        ok &= sunite2((int)(p0 & 0xFFFFu), (int)(p0 >> 16), (int)(p1 & 0xFFFFu), (int)(p1 >> 16));
-    }
-    __syncthreads();  // all unions done
-    if (!ok) atomicOr(&R.st->status, ST_NOCONVERGE);
-    // Resolution: every representative's entry becomes its root's name.  No
-    // union changes the trees any more, and entries only move up them.
-    // RESOLVE_ROUNDS times all entries move to their grandparents together, a
-    // barrier after each; a representative whose parent is a root is done for
-    // good.  The few left on deeper chains are walked to their roots by their
-    // threads, three at a time, read-only (whatever the others write meanwhile,
-    // an entry is an ancestor).  The loads of a step are issued together: one representative
-    // after the other took 31 % of the kernel.  Local kernel at L = 256 with
-    // 0, 1, 2 rounds: 1,698, 1,595, 1,684 us (a round between the first pass and
-    // the listed pairs besides: 60 us slower than without).
-    uint32_t todo = reps;
-#pragma unroll 1
-    for (int it = 0; it < RESOLVE_ROUNDS; ++it) {
-        int p[16];
-#pragma unroll
-        for (int q = 0; q < 16; ++q) p[q] = label_get(me + 4 * q);
-        todo = 0;
-#pragma unroll
-        for (int q = 0; q < 16; ++q) {
-            const int gp = label_get(p[q]);
-            const bool move = ((reps >> q) & 1u) && gp != p[q];
-            label_set_if(move, me + 4 * q, gp);
-            todo |= (move ? 1u : 0u) << q;
-        }
-        __syncthreads();
-    }
-    bool walked = true;
-#pragma unroll 1
-    while (todo) {
-        int x[3], r[3];
-        const int q0 = __ffs(todo) - 1;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            x[k] = me + 4 * (todo ? __ffs(todo) - 1 : q0);
-            todo &= todo - 1;
-            r[k] = label_get(x[k]);
-        }
-#pragma unroll 1
-        for (int st = 0;; ++st) {
-            int p[3];
-            bool there = true;
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                p[k] = label_get(r[k]);
-                there &= p[k] == r[k];
-            }
-            if (there) break;
-#pragma unroll
-            for (int k = 0; k < 3; ++k) r[k] = p[k];
-            if (st == 16 * nt) {
-                walked = false;
-                break;
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < 3; ++k) label_set(x[k], r[k]);
-    }
-    if (!walked) atomicOr(&R.st->status, ST_NOCONVERGE);
-    __syncthreads();
-    // Mark the roots of the sites a crossing bond may end on: the root's own
-    // entry, its name, gets bit 0 set (every marker stores the same value).
-    // A site's entry is its root's name or its representative's, so two loads
-    // lead to the root whatever is marked meanwhile.
-    const uint32_t ends = crossing_sites(c);
     int ent[16];
-#pragma unroll
-    for (int q = 0; q < 16; ++q) ent[q] = label_get(me + 4 * q) & ~1;
-    if (ends) {
-#pragma unroll
-        for (int q = 0; q < 16; ++q) {
-            const bool end = (ends >> q) & 1u;
-            const int r = label_get(end ? ent[q] : me) & ~1;
-            label_set_if(end, r, r | 1);
-        }
-    }
-    __syncthreads();
-    // number the marked roots; a marked root's own entry becomes its code
-    {
-        uint32_t marked = 0;
-#pragma unroll
-        for (int q = 0; q < 16; ++q) marked |= (uint32_t)(label_get(me + 4 * q) & 1) << q;
-        const unsigned lanes = lanes_mask(nt);
-        const int lane = threadIdx.x & 31, last = 31 - __clz(lanes);
-        const int n = __popc(marked);
-        int incl = n;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int v = __shfl_up_sync(lanes, incl, o);
-            if (lane >= o) incl += v;
-        }
-        int base = 0;
-        if (lane == last && incl) base = atomicAdd(s.pcount + 1, incl);
-        int slot = __shfl_sync(lanes, base, last) + incl - n;
-        int32_t *P = R.P + (int64_t)tile * (16 * nt);
-#pragma unroll 1
-        while (marked) {
-            const int q = __ffs(marked) - 1;
-            marked &= marked - 1;
-            P[slot] = (int32_t)(16 * c.cell) + q;
-            label_set(me + 4 * q, IS_CODE + slot_code(nt) + slot);
-            ++slot;
-        }
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) R.nslots[tile] = s.pcount[1];
-    // every site takes the code of its component's representative: the entry
-    // of its root (a code, or the name of a root without a slot)
-#pragma unroll
-    for (int q = 0; q < 16; ++q)
-        ent[q] = label_get(ent[q]);
+    finish_labels(s, nt, me, reps, [&] { return crossing_sites(c); }, (int32_t)(16 * c.cell), R.P + (int64_t)tile * (16 * nt),
+                  R.nslots + tile, &R.st->status, ent);
     uint32_t packed[8];
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
@@ -614,6 +627,41 @@ __device__ __forceinline__ uint32_t slot_root(const uint32_t *P, uint32_t v)
 #pragma unroll 1
     for (int it = 0; it < (1 << 20) && slot_linked(v); ++it) v = __ldg(P + (v & ~SLOT_LINK));
     return v;
+}
+
+// Threads of a slot block.
+constexpr int SLOT_BLOCK = 128;
+
+// The flip bits of the clusters of a tile's n slots, 16 to a word: three slots
+// per thread at a time, their walks in lockstep.  All unions are done and
+// nothing here writes a link, so the walks may take the cached read-only path.
+template <typename FlipBit>
+__device__ __forceinline__ void slot_flips(const uint32_t *own, const uint32_t *P, int n, uint16_t *out,
+                                           const FlipBit &flip_bit)
+{
+    const int lane = threadIdx.x & 31;
+    for (int k0 = threadIdx.x & ~31; k0 < n; k0 += 3 * SLOT_BLOCK) {
+        uint32_t v[3];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const int k = k0 + j * SLOT_BLOCK + lane;
+            v[j] = k < n ? __ldg(own + k) : 0u;
+        }
+#pragma unroll 1
+        for (int it = 0; it < (1 << 20) && ((v[0] | v[1] | v[2]) & SLOT_LINK); ++it)
+#pragma unroll
+            for (int j = 0; j < 3; ++j)
+                if (slot_linked(v[j])) v[j] = __ldg(P + (v[j] & ~SLOT_LINK));
+        uint32_t bit[3];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) bit[j] = flip_bit(v[j]);
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const int k = k0 + j * SLOT_BLOCK + lane;
+            const uint32_t word = __ballot_sync(0xffffffffu, bit[j]);
+            if ((lane & 15) == 0 && k < n) out[k >> 4] = (uint16_t)(word >> (lane & 16));
+        }
+    }
 }
 
 // Index of the tile of cell (x, y, z) in its lattice.
