@@ -104,6 +104,13 @@ __device__ __forceinline__ void tile_sum4_f64(double v[4], int nt, double *scrat
     for (int q = 0; q < 4; ++q) v[q] = scratch[q * nt];
 }
 
+// Tile-local cell of a vertex whose cell is this cell stepped back along
+// the axes of mask m (only meaningful if the vertex is inside the tile).
+__device__ __forceinline__ int vertex_local_cell(const TileCtx &c, int m)
+{
+    return c.t + ((m & 1) ? c.dxm : 0) + ((m & 2) ? c.dym : 0) + ((m & 4) ? c.dzm : 0);
+}
+
 __device__ __forceinline__ int wrap_back(int v, int L) { return v == 0 ? L - 1 : v - 1; }
 
 // Cells of the backward halo staged by the tile kernels.
@@ -500,34 +507,33 @@ __device__ __forceinline__ void local_core(const TileCtx &c, const Rep &R, const
     uint32_t rest[12];
     uint32_t nrest = 0;
     const bool unite = c_unite_bound > 0;
-    // (a cell that a step would take out of the tile counts as this one: its
-    // label is read but not used)
-    const int sx = c.bx ? 0 : CELL_BYTES * c.dxm, sy = c.by ? 0 : CELL_BYTES * c.dym, sz = c.bz ? 0 : CELL_BYTES * c.dzm;
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
-        // labels of the vertices; vertex 0 is the cell's own site and its own
-        // representative (a link meanwhile is found by the compare-and-swap)
-        int l[4] = {me + 16 * f, 0, 0, 0};
+        int name[4];
+#pragma unroll
+        for (int v = 0; v < 4; ++v)
+            name[v] = s.lab + CELL_BYTES * vertex_local_cell(c, down_mask(f, v)) + 4 * down_bit(f, v);
+        int a[3], b[3];
 #pragma unroll
         for (int v = 1; v < 4; ++v) {
-            const int m = down_mask(f, v);
-            l[v] = label_get(me + ((m & 1) ? sx : 0) + ((m & 2) ? sy : 0) + ((m & 4) ? sz : 0) + 4 * down_bit(f, v));
+            // at most one pair (u, v), u < v, spans; none: the same label twice
+            int ea = me, eb = me;
+#pragma unroll
+            for (int u = 0; u < v; ++u)
+                if ((in >> (6 * f + pair_index(u, v))) & 1u) {
+                    ea = name[u];
+                    eb = name[v];
+                }
+            a[v - 1] = label_get(ea);
+            b[v - 1] = label_get(eb);
         }
 #pragma unroll
-        for (int v = 1; v < 4; ++v) {
-            // at most one pair (u, v), u < v, spans
-            uint32_t any = 0;
-            int u = l[0];
-#pragma unroll
-            for (int k = 0; k < v; ++k) {
-                any |= 1u << (6 * f + pair_index(k, v));
-                if (k > 0 && ((in >> (6 * f + pair_index(k, v))) & 1u)) u = l[k];
-            }
-            const int lo = min(u, l[v]), hi = max(u, l[v]);
-            int old = label_link_if(unite && (in & any) && lo != hi, hi, lo);
-            if (!unite && (in & any)) old = lo;
+        for (int v = 0; v < 3; ++v) {
+            const int lo = min(a[v], b[v]), hi = max(a[v], b[v]);
+            int old = label_link_if(unite && lo != hi, hi, lo);
+            if (!unite) old = lo;
             const uint32_t r = old != hi ? (uint32_t)lo | ((uint32_t)old << 16) : 0u;
-            rest[3 * f + v - 1] = r;
+            rest[3 * f + v] = r;
             nrest += r ? 1u : 0u;
         }
     }
