@@ -174,26 +174,29 @@ static __device__ const TetTable tet_table = make_tet_table();
 
 // The four spins of the down tetrahedron of each FCC point f of a cell,
 // gathered into one 16-bit word (bit 4 f + v = vertex v).  w[m] = spin word
-// of the cell stepped back along the axes of mask m.
+// of the cell stepped back along the axes of mask m.  ONE = 0x10001: two
+// cells at once, one in each half of the words.
+template <uint32_t ONE = 1u>
 __device__ __forceinline__ uint32_t down_word(const uint32_t w[7])
 {
     uint32_t D = 0;
 #pragma unroll
     for (int f = 0; f < 4; ++f)
 #pragma unroll
-        for (int v = 0; v < 4; ++v) D |= ((w[down_mask(f, v)] >> down_bit(f, v)) & 1u) << (4 * f + v);
+        for (int v = 0; v < 4; ++v) D |= ((w[down_mask(f, v)] >> down_bit(f, v)) & ONE) << (4 * f + v);
     return D;
 }
 
 // Antiparallel bits of the three bond groups from the up and down spin
-// words (shift-XOR within each nibble).
+// words (shift-XOR within each nibble, so halves of a word stay apart).
+template <uint32_t ONE = 1u>
 __device__ __forceinline__ void antiparallel_groups(uint32_t U, uint32_t D, uint32_t &A, uint32_t &Bg, uint32_t &C)
 {
     const uint32_t u1 = U ^ (U >> 1), u2 = U ^ (U >> 2), u3 = U ^ (U >> 3);
     const uint32_t d1 = D ^ (D >> 1), d2 = D ^ (D >> 2), d3 = D ^ (D >> 3);
-    A = (u1 & 0x7777u) | ((u3 & 0x1111u) << 3);
-    Bg = (u2 & 0x3333u) | ((d2 & 0x3333u) << 2);
-    C = (d1 & 0x7777u) | ((d3 & 0x1111u) << 3);
+    A = (u1 & (0x7777u * ONE)) | ((u3 & (0x1111u * ONE)) << 3);
+    Bg = (u2 & (0x3333u * ONE)) | ((d2 & (0x3333u * ONE)) << 2);
+    C = (d1 & (0x7777u * ONE)) | ((d3 & (0x1111u * ONE)) << 3);
 }
 
 // Flip bits of the tile's sites: bits 16 c .. 16 c + 15 of the FLIP stream
