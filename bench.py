@@ -51,8 +51,8 @@ SWEEP_BYTES_PER_SITE = SWEEP_BYTES[1][1]
 # move nothing the model counts.
 PHASE_BYTES_PER_SITE = {"local": 0.125 + 4.0, "boundary": 0.0, "flip": 4.0 + 0.125, "measure": 0.0,
                         "accumulate": 0.0}
-KERNEL_NAMES = {"local": "ising_local_kernel", "boundary": "boundary_kernel", "flip": "ising_flip_kernel",
-                "measure": "ising_measure_kernel", "accumulate": "accumulate_kernel"}
+KERNEL_NAMES = {"local": "ising_local_kernel", "boundary": "boundary_unite_kernel+boundary_flip_kernel",
+                "flip": "ising_flip_kernel", "measure": "ising_measure_kernel", "accumulate": "accumulate_kernel"}
 
 
 def peaks():
@@ -69,7 +69,7 @@ def peaks():
 
 
 # The sources the Ising sweep's kernels are compiled from.
-ISING_KERNEL_SOURCES = ("ccl.cuh", "ising.cu", "pyro_internal.cuh", "sweep_core.cuh")
+ISING_KERNEL_SOURCES = ("bonds.cuh", "ccl.cuh", "ising.cu", "launch.cuh", "pyro_internal.cuh", "sweep_core.cuh")
 
 
 def kernel_source_hash() -> str:

@@ -38,14 +38,8 @@ __device__ __forceinline__ void label_set_if(bool on, int name, int v)
                  "r"((int)on)
                  : "memory");
 }
-// Links root hi under lo; hi if it was a root still, else its entry.
-__device__ __forceinline__ int label_link(int hi, int lo)
-{
-    int old;
-    asm volatile("atom.shared.cas.b32 %0, [%1], %2, %3;" : "=r"(old) : "r"(hi), "r"(hi), "r"(lo) : "memory");
-    return old;
-}
-// The same if on, else hi.
+// If on, links root hi under lo; hi if it was a root still (or not on), else
+// its entry.
 __device__ __forceinline__ int label_link_if(bool on, int hi, int lo)
 {
     int old = hi;

@@ -13,9 +13,9 @@
 //   ising_flip      flips every site whose cluster's flip bit is set: the
 //                   bit of its tile-local root, or of its slot's cluster
 //                   where the cluster may cross a tile face.
-//   ising_measure   counts antiparallel bonds and -1 spins per tile, four
-//                   cells per thread (exact integers; energy of Eq. 1,
-//                   magnetisation of Eq. 2).
+//   ising_measure   counts antiparallel bonds and -1 spins per tile, a warp
+//                   per tile, four cells of a row at a time (exact integers;
+//                   energy of Eq. 1, magnetisation of Eq. 2).
 //   boundary_unite, boundary_flip  unite the clusters that cross tile faces and
 //                   find their flip bits (all models).
 //   labels_kernel   writes the canonical label of every site on demand.
@@ -25,7 +25,8 @@
 
 namespace pyro {
 
-// Threads of a measurement block (a tile of up to 512 cells, four per thread).
+// Threads of a measurement block: four tiles of up to 256 cells, a warp each,
+// or a tile of up to 512, four cells per thread.
 constexpr int MEASURE_BLOCK = 128;
 
 __global__ void __launch_bounds__(512) ising_local_kernel(const __grid_constant__ Batch B)

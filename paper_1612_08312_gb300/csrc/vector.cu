@@ -7,17 +7,17 @@
 //
 // Spins are stored as n component planes of N values of T (float or
 // double).  A bond with p_i p_j > 0 is active iff its 32-bit uniform
-// w < floor(p 2^32), w drawn like the Ising bonds' (sweep_core.cuh).  The FP64 path uses explicitly rounded IEEE operations in the
-// same order as the definition, so projections, reflections and the axis
-// are bit-identical to a straightforward FP64 evaluation without fused
-// multiply-add.  The FP32 path stores and updates spins in float; its
+// w < floor(p 2^32), w drawn like the Ising bonds' (sweep_core.cuh).  The FP64
+// path rounds every operation as IEEE does, in the order of the definition, so
+// projections, reflections and the axis are bit-identical to a straightforward
+// FP64 evaluation without fused multiply-add.  The FP32 path stores and updates spins in float; its
 // measurements are accumulated in FP64.
 //
 // Kernels (each over a Batch of lattices): vec_local (projections of the
 // tile + halo staged in shared memory, bond activation, tile-local
-// labelling), the global union of tile-crossing clusters (boundary_kernel,
-// shared with the Ising sweep), vec_flip (root, flip, reflection) and
-// vec_measure (E and M per block in FP64).
+// labelling), the global union of tile-crossing clusters (boundary_unite and
+// boundary_flip, shared with the Ising sweep), vec_flip (root, flip,
+// reflection) and vec_measure (E and M per block in FP64).
 #include <algorithm>
 
 #include "nvec.cuh"
@@ -52,9 +52,10 @@ __host__ __device__ constexpr bool vec_stage_shared(int TX, int TY, int TZ)
     return vec_stage_bytes(TX, TY, TZ) <= (size_t)core_shared_words(TX * TY * TZ) * 4;
 }
 
-// Margin of the bond shortcut below, in units of 1/256 of probability.  The
-// evaluation errs by at most 2e-4 there: 2^-22 of ex2, 2^-22 in its argument
-// y log2 e (which moves exp(-y) by y exp(-y) 2^-22), and the rounding of q.
+// Margin of the bond shortcut below, in units of 1/256 of probability.  With
+// 256 exp(-y) = 2^(8 - y log2 e) the evaluation errs by at most 2e-4 there:
+// 256 * 2^-22 of ex2, 2^-22 in its argument (256 ln 2 * 2^-22), four roundings
+// of y log2 e (256 y exp(-y) * 2^-22 <= 94 * 2^-22) and that of q.
 // FP64 projections are staged in FP32 as sums of rounded terms, 3e-7 off at
 // most (six roundings of 2^-24), so y = K2 p p' errs by 6e-7 K2 more and q by
 // 1.6e-4 K2.
