@@ -116,9 +116,10 @@ __global__ void __launch_bounds__(512) ising_flip_kernel(const __grid_constant__
     const Rep &R = B.reps[r];
     const int tile = (int)(blockIdx.x - B.tile_begin[r]);
     const TileCtx c = tile_ctx(B, R, tile);
-    const uint32_t flip = cell_flip_mask(c, R, tile, smem);
     uint16_t *spins = static_cast<uint16_t *>(R.spins);
-    if (c.valid) spins[c.cell] = (uint16_t)((uint32_t)spins[c.cell] ^ flip);
+    const uint32_t was = spins[c.cell];
+    const uint32_t flip = cell_flip_mask(c, R, tile, smem);
+    if (c.valid) spins[c.cell] = (uint16_t)(was ^ flip);
 }
 
 // Canonical label (global index of the cluster root) of every site.

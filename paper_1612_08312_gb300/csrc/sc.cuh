@@ -345,9 +345,9 @@ __global__ void __launch_bounds__(256) sc_flip_kernel(const __grid_constant__ Sc
 {
     extern __shared__ uint32_t bits[];
     const int nt = S.TX * S.TY * S.TZ, words = slot_code(nt) >> 5;
-    for (int i = threadIdx.x; i < words; i += nt) bits[i] = 0;
     overlap_begin();
     const ScCtx c = sc_ctx(S, blockIdx.x, threadIdx.x);
+    const uint32_t was = S.spins[c.seg];
     const uint4 *src = reinterpret_cast<const uint4 *>(S.code + 16 * c.seg);
     const uint4 a0 = src[0], a1 = src[1];
     const uint32_t w[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
@@ -355,10 +355,7 @@ __global__ void __launch_bounds__(256) sc_flip_kernel(const __grid_constant__ Sc
     const int n = (S.nslots[blockIdx.x] + 15) >> 4;
     const uint16_t *sf = S.sflip + (int64_t)blockIdx.x * (S.nslot / 16);
     for (int i = threadIdx.x; i < n; i += nt) reinterpret_cast<uint16_t *>(bits + words)[i] = sf[i];
-    __syncthreads();
-    const int bit = 17 * c.t;
-    atomicOr(bits + (bit >> 5), f << (bit & 31));
-    if ((bit & 31) > 16) atomicOr(bits + (bit >> 5) + 1, f >> (32 - (bit & 31)));
+    place_flip_bits(bits, f, c.t, nt);
     __syncthreads();
     if (!c.vm) return;
     uint32_t flip = 0;
@@ -368,7 +365,7 @@ __global__ void __launch_bounds__(256) sc_flip_kernel(const __grid_constant__ Sc
         if (q < c.nv) flip |= ((bits[code >> 5] >> (code & 31)) & 1u) << q;
     }
     if (S.occ) flip &= S.occ[c.seg];
-    S.spins[c.seg] = (uint16_t)((uint32_t)S.spins[c.seg] ^ (flip & c.vm));
+    S.spins[c.seg] = (uint16_t)(was ^ (flip & c.vm));
 }
 
 // Sum over present bonds of s_i s_j and magnetisation of the occupied sites,
