@@ -197,8 +197,9 @@ void *pyro_get_stream(pyro_handle h);
 /* Number of kernel launches this handle has issued (for accounting). */
 uint64_t pyro_launch_count(pyro_handle h);
 
-/* Whether multi-sweep calls replay captured CUDA graphs (default on; only
- * with a library-owned stream).  Off = one launch per phase per sweep. */
+/* Whether whole chunks of 32 sweeps and single sweeps replay captured CUDA
+ * graphs (default on; only with a library-owned stream).  Off = one launch per
+ * phase per sweep, as in between. */
 int pyro_set_graphs(pyro_handle h, int on);
 
 /* Autotuner: equilibrate a scratch lattice for 60 sweeps at beta, then
@@ -287,7 +288,7 @@ int pyro_ising_sweep_noalloc(const uint16_t *spins_in, uint16_t *spins_out, int3
 
 /* R independent lattices of sizes L[r] at inverse temperatures beta[r],
  * one model and precision, updated together: every phase of a sweep is one
- * launch over all replicas' tiles, and a multi-sweep call is a CUDA graph.
+ * launch over all replicas' tiles, and a chunk of 32 sweeps is a CUDA graph.
  * Replica r uses seed + r * 0x9E3779B97F4A7C15 (mod 2^64), so it is the
  * same chain as a single lattice created with that seed.  start as in
  * pyro_config.  Independent runs (Sec. 2: five independent runs). */
