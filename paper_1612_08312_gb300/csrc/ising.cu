@@ -248,6 +248,26 @@ __global__ void __launch_bounds__(CELL_BLOCK) ising_init_kernel(const __grid_con
     static_cast<uint16_t *>(R.spins)[cell] = (uint16_t)word;
 }
 
+// A listed crossing pair: its cell in the tile, nine bits a coordinate (a tile
+// has at most 512 cells, so an edge may have as many), and the pair 6 f + k.
+__host__ __device__ constexpr uint32_t cell_entry(int lx, int ly, int lz)
+{
+    return (uint32_t)lx | ((uint32_t)ly << 9) | ((uint32_t)lz << 18);
+}
+__host__ __device__ constexpr uint32_t pair_entry(uint32_t cell, int pair) { return cell | ((uint32_t)pair << 27); }
+__host__ __device__ constexpr int entry_x(uint32_t e) { return (int)(e & 511u); }
+__host__ __device__ constexpr int entry_y(uint32_t e) { return (int)((e >> 9) & 511u); }
+__host__ __device__ constexpr int entry_z(uint32_t e) { return (int)((e >> 18) & 511u); }
+__host__ __device__ constexpr int entry_pair(uint32_t e) { return (int)(e >> 27); }
+constexpr bool entry_holds(int lx, int ly, int lz, int pair)
+{
+    const uint32_t e = pair_entry(cell_entry(lx, ly, lz), pair);
+    return entry_x(e) == lx && entry_y(e) == ly && entry_z(e) == lz && entry_pair(e) == pair;
+}
+static_assert(entry_holds(511, 0, 0, 23) && entry_holds(0, 511, 0, 23) && entry_holds(0, 0, 511, 23) &&
+                  entry_holds(511, 511, 511, 0),
+              "a pair entry holds every cell of the longest tile");
+
 // Phase 1, first launch, over the face cells of every tile (one thread each):
 // unites the clusters joined by the union pairs that leave the tile.  Model-
 // independent: used by the n-vector sweeps too.  Latency-bound chains of
@@ -255,8 +275,7 @@ __global__ void __launch_bounds__(CELL_BLOCK) ising_init_kernel(const __grid_con
 __global__ void __launch_bounds__(512, 4) boundary_unite_kernel(const __grid_constant__ Batch B)
 {
     // the block's crossing pairs, compacted so that every thread takes an
-    // equal share: entry lx | ly << 5 | lz << 10 | (6 f + k) << 16 (at most three
-    // pairs per tetrahedron span it)
+    // equal share (at most three pairs per tetrahedron span it)
     extern __shared__ uint32_t blist[];
     __shared__ int bcount;
     __shared__ uint32_t ends[24];
@@ -279,7 +298,7 @@ __global__ void __launch_bounds__(512, 4) boundary_unite_kernel(const __grid_con
         face_cell_coords(B, threadIdx.x, lx, ly, lz);
         if (max(ox + lx, max(oy + ly, oz + lz)) < L)
             todo = R.dmask[(int64_t)(ox + lx) + (int64_t)L * ((int64_t)(oy + ly) + (int64_t)L * (oz + lz))];
-        here = (uint32_t)(lx | (ly << 5) | (lz << 10));
+        here = cell_entry(lx, ly, lz);
     }
     const int lane = threadIdx.x & 31;
     const int n = __popc(todo);
@@ -296,7 +315,7 @@ __global__ void __launch_bounds__(512, 4) boundary_unite_kernel(const __grid_con
     while (todo) {
         const int bit = __ffs(todo) - 1;
         todo &= todo - 1;
-        blist[pos++] = here | ((uint32_t)bit << 16);
+        blist[pos++] = pair_entry(here, bit);
     }
     __syncthreads();
     const int np = bcount;
@@ -304,8 +323,8 @@ __global__ void __launch_bounds__(512, 4) boundary_unite_kernel(const __grid_con
     bool ok = true;
     for (int i = threadIdx.x; i < np; i += blockDim.x) {
         const uint32_t en = blist[i];
-        const int x = ox + (int)(en & 31u), y = oy + (int)((en >> 5) & 31u), z = oz + (int)((en >> 10) & 31u);
-        uint32_t pr = ends[en >> 16];
+        const int x = ox + entry_x(en), y = oy + entry_y(en), z = oz + entry_z(en);
+        uint32_t pr = ends[entry_pair(en)];
         uint32_t g[2];
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
