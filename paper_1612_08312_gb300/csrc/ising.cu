@@ -340,8 +340,9 @@ __global__ void __launch_bounds__(512, 4) boundary_unite_kernel(const __grid_con
 }
 
 // Phase 1, second launch: the flip bit of every slot's cluster (that of its
-// root site), 32 slots to a word.  All unions are done and this pass writes no
-// link, so the walks may take the cached read-only path.
+// root site), 16 slots to a word.  The flip bits may be read through the read-
+// only path: the local kernel, which wrote them, had ended before this one
+// could start (its predecessor lets it start only after waiting for that end).
 __global__ void __launch_bounds__(SLOT_BLOCK) boundary_flip_kernel(const __grid_constant__ Batch B)
 {
     overlap_begin();

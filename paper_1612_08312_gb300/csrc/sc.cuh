@@ -330,7 +330,8 @@ __global__ void __launch_bounds__(256, 8) sc_unite_kernel(const __grid_constant_
     if (!ok) atomicOr(&S.st->status, ST_NOCONVERGE);
 }
 
-// The flip bit of every slot's cluster, 16 slots to a word.
+// The flip bit of every slot's cluster, 16 slots to a word (read-only loads of
+// the flip bits as in boundary_flip_kernel).
 __global__ void __launch_bounds__(SLOT_BLOCK) sc_slot_flip_kernel(const __grid_constant__ ScDev S)
 {
     overlap_begin();

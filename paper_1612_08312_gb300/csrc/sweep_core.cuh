@@ -580,6 +580,11 @@ __device__ __forceinline__ void local_core(const TileCtx &c, const Rep &R, const
 // the other one, so a cluster's root keeps its minimum site index.  The local
 // kernel writes every slot in use, so nothing is left over from earlier
 // sweeps.
+//
+// No load of the table takes the read-only path (__ldg), the walks after the
+// last union included: that path asks for data nobody writes while the kernel
+// exists, and an overlapped kernel exists while the one before it still links
+// slots; what overlap_wait makes visible, ordinary loads see.
 __device__ __forceinline__ bool slot_linked(uint32_t v) { return (v & SLOT_LINK) != 0; }
 
 // One find step with path splitting: x (entry v, a link) moves to its parent,
@@ -628,7 +633,7 @@ __device__ __forceinline__ bool slot_unite(uint32_t *P, uint32_t a, uint32_t b)
 __device__ __forceinline__ uint32_t slot_root(const uint32_t *P, uint32_t v)
 {
 #pragma unroll 1
-    for (int it = 0; it < (1 << 20) && slot_linked(v); ++it) v = __ldg(P + (v & ~SLOT_LINK));
+    for (int it = 0; it < (1 << 20) && slot_linked(v); ++it) v = P[v & ~SLOT_LINK];
     return v;
 }
 
@@ -636,8 +641,7 @@ __device__ __forceinline__ uint32_t slot_root(const uint32_t *P, uint32_t v)
 constexpr int SLOT_BLOCK = 128;
 
 // The flip bits of the clusters of a tile's n slots, 16 to a word: three slots
-// per thread at a time, their walks in lockstep.  All unions are done and
-// nothing here writes a link, so the walks may take the cached read-only path.
+// per thread at a time, their walks in lockstep.
 template <typename FlipBit>
 __device__ __forceinline__ void slot_flips(const uint32_t *own, const uint32_t *P, int n, uint16_t *out,
                                            const FlipBit &flip_bit)
@@ -648,13 +652,13 @@ __device__ __forceinline__ void slot_flips(const uint32_t *own, const uint32_t *
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
             const int k = k0 + j * SLOT_BLOCK + lane;
-            v[j] = k < n ? __ldg(own + k) : 0u;
+            v[j] = k < n ? own[k] : 0u;
         }
 #pragma unroll 1
         for (int it = 0; it < (1 << 20) && ((v[0] | v[1] | v[2]) & SLOT_LINK); ++it)
 #pragma unroll
             for (int j = 0; j < 3; ++j)
-                if (slot_linked(v[j])) v[j] = __ldg(P + (v[j] & ~SLOT_LINK));
+                if (slot_linked(v[j])) v[j] = P[v[j] & ~SLOT_LINK];
         uint32_t bit[3];
 #pragma unroll
         for (int j = 0; j < 3; ++j) bit[j] = flip_bit(v[j]);
