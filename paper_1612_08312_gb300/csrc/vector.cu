@@ -56,13 +56,17 @@ __host__ __device__ constexpr bool vec_stage_shared(int TX, int TY, int TZ)
 // 256 exp(-y) = 2^(8 - y log2 e) the evaluation errs by at most 2e-4 there:
 // 256 * 2^-22 of ex2, 2^-22 in its argument (256 ln 2 * 2^-22), four roundings
 // of y log2 e (256 y exp(-y) * 2^-22 <= 94 * 2^-22) and that of q.
-// FP64 projections are staged in FP32 as sums of rounded terms, 3e-7 off at
-// most (six roundings of 2^-24), so y = K2 p p' errs by 6e-7 K2 more and q by
-// 1.6e-4 K2.
+// FP64 projections are staged in FP32 as sums of rounded terms, for spins of
+// length 1 3e-7 off at most (six roundings of 2^-24), so y = K2 p p' errs by
+// 6e-7 K2 more and q by 1.6e-4 K2.  A caller may set spins of any length: a
+// block that stages one whose squared length exceeds LENGTH2_MAX (or is no
+// number) decides all its bonds by the FP64 rule.  (FP32 projections are the
+// rule's own, whatever the length.)
+constexpr float LENGTH2_MAX = 1.0001f;
 template <typename T>
-__device__ __forceinline__ float shortcut_margin(double K2)
+__device__ __forceinline__ float shortcut_margin(double K2, bool any_long)
 {
-    return sizeof(T) == 4 ? SHORTCUT_MARGIN : SHORTCUT_MARGIN + 4e-4f * (float)K2;
+    return sizeof(T) == 4 ? SHORTCUT_MARGIN : any_long ? INFINITY : SHORTCUT_MARGIN + 4e-4f * (float)K2;
 }
 
 // Registers: two 512-thread blocks' worth of warps per SM.
@@ -112,6 +116,7 @@ __global__ void __launch_bounds__(512, 2) vec_local_kernel(const __grid_constant
     for (int b = 0; b < BATCH; ++b) own_load(b, b);
     const double *axis = R.st->axis;
     const float rf[3] = {(float)axis[0], (float)axis[1], (float)axis[2]};
+    bool is_long = false;  // (FP64) a spin staged by this thread
     auto put = [&](const T w[NC][4], int h, int s0) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -119,6 +124,12 @@ __global__ void __launch_bounds__(512, 2) vec_local_kernel(const __grid_constant
 #pragma unroll
             for (int k = 1; k < NC; ++k) pr = Ar<float>::add(pr, Ar<float>::mul((float)w[k][q], rf[k]));
             proj[(s0 + q) * nh + h] = pr;
+            if (sizeof(T) == 8) {
+                float len2 = 0.0f;
+#pragma unroll
+                for (int k = 0; k < NC; ++k) len2 = fmaf((float)w[k][q], (float)w[k][q], len2);
+                is_long |= !(len2 <= LENGTH2_MAX);
+            }
         }
     };
 #pragma unroll
@@ -180,7 +191,9 @@ __global__ void __launch_bounds__(512, 2) vec_local_kernel(const __grid_constant
         put(v[0], h[0], s0[0]);
         if (two) put(v[1], h[1], s0[1]);
     }
-    __syncthreads();
+    bool any_long = false;
+    if (sizeof(T) == 8) any_long = __syncthreads_or(is_long);
+    else __syncthreads();
 
     uint32_t act[3] = {0, 0, 0};
     if (R.K2 > 0.0 && c.valid) {
@@ -194,7 +207,7 @@ __global__ void __launch_bounds__(512, 2) vec_local_kernel(const __grid_constant
         // 534 -> 327 us; FP64, whose projections and exponentials all ran in
         // FP64, L = 64 862 -> 97 us.
         const float K2l = (float)R.K2 * 1.44269504f;
-        const float margin = shortcut_margin<T>(R.K2);
+        const float margin = shortcut_margin<T>(R.K2, any_long);
         // (three calls together; then tetrahedron by tetrahedron, so that each
         // projection is loaded once)
         uint32_t ww[3][4];
