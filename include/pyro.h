@@ -94,8 +94,10 @@ typedef struct {
     uint64_t seed;     /* Philox key */
     void *stream;      /* cudaStream_t to run on; NULL = the library creates one */
     int tile[3];       /* labelling tile in cells: power-of-two edges, each dividing L, at most
-                          512 cells; {0,0,0} = default (Ising 8 x 8 x 4, n-vector 8 x 4 x 4 for
-                          most L; power-of-two edges chosen by L that need not divide it) */
+                          512 cells; {0,0,0} = default (power-of-two edges chosen by L that need
+                          not divide it, at most 512, 128 or 256 cells for Ising and 256, 64 or 256
+                          for n > 1, with growing L).  The default may also be given as
+                          pyro_get_tile reports it */
     void *workspace;   /* NULL = the library allocates (and frees) the lattice's device memory;
                           else caller-owned device memory (for instance a torch tensor's data_ptr),
                           at least pyro_workspace_bytes(cfg) bytes, 256-byte aligned, from which
@@ -191,6 +193,7 @@ int pyro_sync(pyro_handle h);
 
 /* Facts about a handle. */
 int64_t pyro_num_sites(pyro_handle h);
+/* (the tile in use; accepted back in pyro_config.tile for the same L) */
 int pyro_get_tile(pyro_handle h, int tile[3]);
 void *pyro_get_stream(pyro_handle h);
 
@@ -296,8 +299,9 @@ int pyro_batch_init(pyro_batch *out, int R, const int *L, const double *beta, in
                     int precision, int start, uint64_t seed);
 
 /* Same with a labelling tile for every replica (power-of-two edges dividing
- * every L; NULL or {0,0,0} = the default, one tile for all, chosen by the
- * sizes), e.g. from pyro_batch_autotune. */
+ * every L, or the tile that pyro_get_tile reports for one of them; NULL or
+ * {0,0,0} = the default, one tile for all, chosen by the sizes), e.g. from
+ * pyro_batch_autotune. */
 int pyro_batch_init_ex(pyro_batch *out, int R, const int *L, const double *beta, int model,
                        int precision, int start, uint64_t seed, const int tile[3]);
 

@@ -49,6 +49,17 @@ static int finish(Engine &e)
 
 static bool beta_ok(double b) { return b >= 0.0 && std::isfinite(b); }
 
+// Whether t is the default tile of the set of lattices or of one of them alone:
+// what pyro_get_tile may have reported, whose edges need not divide L.
+static bool reported_tile(const int *Ls, int R, int model, const TileShape &t)
+{
+    const auto is = [&](const TileShape &d) { return d.TX == t.TX && d.TY == t.TY && d.TZ == t.TZ; };
+    if (is(default_tile(Ls, R, model))) return true;
+    for (int r = 0; r < R; ++r)
+        if (is(default_tile(Ls + r, 1, model))) return true;
+    return false;
+}
+
 // Argument checks and the resolved tile of a set of lattices; "" if valid.
 static std::string check_args(int R, const int *Ls, const double *betas, int model, int prec, int start, double J,
                               const int tile[3], TileShape &t)
@@ -62,10 +73,13 @@ static std::string check_args(int R, const int *Ls, const double *betas, int mod
     if (prec != PYRO_FP32 && prec != PYRO_FP64) return "precision must be PYRO_FP32 or PYRO_FP64";
     if (start != PYRO_START_UP && start != PYRO_START_RANDOM) return "start must be PYRO_START_UP or PYRO_START_RANDOM";
     if (!(J > 0.0) || !std::isfinite(J)) return "J must be positive and finite";
-    t = default_tile(Ls, R, model);
-    const bool callers = tile && (tile[0] || tile[1] || tile[2]);
-    if (callers) t = TileShape{tile[0], tile[1], tile[2]};
-    return check_tile(Ls, R, model, prec, t, callers);
+    if (!tile || !(tile[0] || tile[1] || tile[2])) {
+        t = default_tile(Ls, R, model);
+        return check_tile(Ls, R, model, prec, t, false);
+    }
+    t = TileShape{tile[0], tile[1], tile[2]};
+    const std::string why = check_tile(Ls, R, model, prec, t);
+    return !why.empty() && reported_tile(Ls, R, model, t) ? check_tile(Ls, R, model, prec, t, false) : why;
 }
 
 static int create(Engine &e, int R, const int *Ls, const double *betas, int model, int prec, int start, double J,
