@@ -708,6 +708,7 @@ struct GraphEngine {
                   {(void **)&sc.pz, mask},
                   {(void **)&sc.occ, occ.empty() ? 0 : segs * 2},
                   {(void **)&sc.bytes, (size_t)N},
+                  {(void **)&sc.labels, (size_t)N * 4},  // (asking for them later can't fail)
                   {(void **)&G.partials, (size_t)nmeas * 4 * sizeof(double)},
                   {(void **)&G.st, sizeof(DevStats)}};
         cudaError_t e;
@@ -780,10 +781,6 @@ struct GraphEngine {
 
     cudaError_t sc_labels()
     {
-        if (!sc.labels) {
-            const cudaError_t e = alloc((void **)&sc.labels, (size_t)sc.N * 4);
-            if (e != cudaSuccess) return e;
-        }
         sc_labels_kernel<<<sc_tiles, sc.TX * sc.TY * sc.TZ, 0, stream>>>(sc, swept);
         ++launches;
         lab_last = sc.labels;

@@ -36,7 +36,7 @@ struct ScDev {
     const uint16_t *px, *py, *pz;    // present bonds of each direction per segment, or null
     const uint16_t *occ;             // occupied sites per segment, or null
     int8_t *bytes;                   // N spins of +-1, for the copies to and from the host
-    int32_t *labels;                 // canonical labels, or null until asked for
+    int32_t *labels;                 // canonical labels, written when asked for
     double *partials;
     DevStats *st;
     uint64_t seed, thr;
