@@ -100,7 +100,7 @@ __device__ __forceinline__ ScSpins sc_spins(const ScDev &S, const ScCtx &c)
 }
 
 // Bits 0, 3, 6 .. 45 of x as 16 bits.
-__device__ __forceinline__ uint32_t every_third(unsigned long long x)
+__host__ __device__ __forceinline__ uint32_t every_third(unsigned long long x)
 {
     x &= 0x249249249249ull;
     x = (x ^ (x >> 2)) & 0x0C30C30C30C3ull;
