@@ -200,9 +200,9 @@ void *pyro_get_stream(pyro_handle h);
 /* Number of kernel launches this handle has issued (for accounting). */
 uint64_t pyro_launch_count(pyro_handle h);
 
-/* Whether whole chunks of 32 sweeps and single sweeps replay captured CUDA
- * graphs (default on; only with a library-owned stream).  Off = one launch per
- * phase per sweep, as in between. */
+/* Whether sweeps replay captured CUDA graphs, of 32 sweeps and of one (default
+ * on; only with a library-owned stream).  Off = one launch per phase per
+ * sweep. */
 int pyro_set_graphs(pyro_handle h, int on);
 
 /* Autotuner: equilibrate a scratch lattice for 60 sweeps at beta, then

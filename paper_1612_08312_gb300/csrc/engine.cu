@@ -617,15 +617,17 @@ cudaGraphExec_t Engine::graph_for(int n)
 cudaError_t Engine::sweeps(int n)
 {
     if (n <= 0) return cudaSuccess;
-    // Whole chunks replay a graph, and so does a single sweep, whose six or
-    // seven launches would cost the host more than a small lattice's sweep
-    // costs the GPU.  In between (and for what is left of a chunk) plain
-    // launches: they overlap from sweep to sweep, graphs do not (L = 16, a sweep:
-    // 31.6 us in graphs of 32, 32.6 launched, 34.8 in graphs of one).
+    // A call replays graphs: of whole chunks, and of one sweep for what is left.
+    // Six or seven launches a sweep cost the host 10 us, more than a small
+    // lattice's sweep costs a GPU that several handles share, and a graph 1:
+    // eight Ising lattices of L = 8 driven by one thread in calls of 2 to 31
+    // sweeps take 3.6 us a sweep, launched plainly 11; FP32 XY of L = 16 6.5 and
+    // 11.  One handle alone pays for it, since plain launches overlap from sweep to
+    // sweep and graphs do not: L = 8 23.7 us for 21.5, L = 24 34.3 for 32.2.
     int left = n;
     if (use_graphs && own_stream) {
         for (const int chunk : {GRAPH_CHUNK, 1}) {
-            if (left < chunk || (chunk == 1 && left > 1)) continue;
+            if (left < chunk) continue;
             cudaGraphExec_t g = graph_for(chunk);
             for (; g && left >= chunk; left -= chunk) {
                 const cudaError_t e = cudaGraphLaunch(g, stream);
