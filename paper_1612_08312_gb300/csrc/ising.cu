@@ -41,6 +41,11 @@ __global__ void __launch_bounds__(512) ising_local_kernel(const __grid_constant_
     const TileCtx c = tile_ctx(B, R, tile);
     const uint32_t sweep = (uint32_t)R.st->sweep;
     const uint64_t seed = R.seed;
+    const ByteCompare bc(R.thr);
+    if (bc.none) {
+        local_identity(c, R, sweep, tile);
+        return;
+    }
     // the cell's spin word and those of the cells one step back along the
     // axes of each mask m (read straight from global memory, L1-cached)
     const uint16_t *spins = static_cast<const uint16_t *>(R.spins);
@@ -60,10 +65,9 @@ __global__ void __launch_bounds__(512) ising_local_kernel(const __grid_constant_
     antiparallel_groups(w[0], down_word(w), anti[0], anti[1], anti[2]);
     const uint32_t vmask = c.valid ? 0xFFFFu : 0u;  // no bond past the lattice
     uint32_t act[3];
-    const ByteCompare bc(R.thr);
-    if (bc.all || bc.none) {
+    if (bc.all) {
 #pragma unroll
-        for (int g = 0; g < 3; ++g) act[g] = bc.all ? ~anti[g] & vmask : 0u;
+        for (int g = 0; g < 3; ++g) act[g] = ~anti[g] & vmask;
     } else {
         // bond 48 c + 16 g + 4 f + q: byte 4 f + q of BOND call 3 c + g; the
         // three calls are drawn together (independent chains interleave)
