@@ -211,46 +211,55 @@ __global__ void __launch_bounds__(256, 4) sc_local_kernel(const __grid_constant_
     __syncthreads();  // labels initialised
     // ---- first pass over the bonds in the tile, as in local_core: the larger
     // of the ends' parents is linked under the other if it is a root still,
-    // else the pair is listed; four bonds at a time
+    // else the pair is listed; four bonds at a time.  At low temperatures there
+    // are more pairs than the list holds: the bonds left then have a pass of
+    // their own after the list is united.  (United at once, lane by lane: at
+    // beta = 1 L = 16 150 us a sweep, now 64, and L = 256 1,446, now 546.)
     const bool unite = c_unite_bound > 0;
     bool ok = true;
-    const auto first_pass = [&](uint32_t bits, int next) {
-#pragma unroll 1
-        while (bits) {
-            int a[4], b[4];
-            const int q0 = __ffs(bits) - 1;
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int q = bits ? __ffs(bits) - 1 : q0;
-                bits &= bits - 1;
-                a[k] = label_get(me + 4 * q);
-                b[k] = label_get(next + 4 * q);
-            }
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int lo = min(a[k], b[k]), hi = max(a[k], b[k]);
-                int old = label_link_if(unite && lo != hi, hi, lo);
-                if (!unite) old = lo;
-                if (old != hi && (old != lo || !unite)) {
-                    const int pos = atomicAdd(s.pcount, 1);
-                    if (pos < 15 * nt) s.plist[pos] = (uint32_t)lo | ((uint32_t)old << 16);
-                    else ok &= sunite2(lo, old, lo, old);  // the list is full
-                }
-            }
-        }
-    };
-    first_pass(iny ? act[1] : 0u, nexty);
-    first_pass(inz ? act[2] : 0u, nextz);
-    if (inx && last) {
-        const int a = label_get(me + 4 * (c.nv - 1)), b = label_get(nextx);
+    const auto link_or_list = [&](int a, int b) {  // false: the list is full
         const int lo = min(a, b), hi = max(a, b);
         int old = label_link_if(unite && lo != hi, hi, lo);
         if (!unite) old = lo;
-        if (old != hi && (old != lo || !unite)) {
-            const int pos = atomicAdd(s.pcount, 1);
-            if (pos < 15 * nt) s.plist[pos] = (uint32_t)lo | ((uint32_t)old << 16);
-            else ok &= sunite2(lo, old, lo, old);
+        if (old == hi || (old == lo && unite)) return true;
+        const int pos = atomicAdd(s.pcount, 1);
+        if (pos >= list_room(nt)) return false;
+        s.plist[pos] = (uint32_t)lo | ((uint32_t)old << 16);
+        return true;
+    };
+    const auto pass = [&](uint32_t bits, int next) {  // the bonds left
+        uint32_t left = 0;
+#pragma unroll 1
+        while (bits) {
+            int a[4], b[4], q[4];
+            const int q0 = __ffs(bits) - 1;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                q[k] = bits ? __ffs(bits) - 1 : q0;
+                bits &= bits - 1;
+                a[k] = label_get(me + 4 * q[k]);
+                b[k] = label_get(next + 4 * q[k]);
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (!link_or_list(a[k], b[k])) left |= 1u << q[k];
         }
+        return left;
+    };
+    uint32_t ybits = iny ? act[1] : 0u, zbits = inz ? act[2] : 0u;
+    bool xbit = inx && last;
+#pragma unroll 1
+    for (;;) {
+        ybits = pass(ybits, nexty);
+        zbits = pass(zbits, nextz);
+        if (xbit) xbit = !link_or_list(label_get(me + 4 * (c.nv - 1)), label_get(nextx));
+        __syncthreads();  // pairs listed
+        // (every pass but the last lists a whole list of pairs, so they end)
+        if (s.pcount[0] <= list_room(nt)) break;
+        ok &= unite_listed(s, nt);
+        __syncthreads();
+        if (threadIdx.x == 0) s.pcount[0] = 0;
+        __syncthreads();
     }
     if (!ok) atomicOr(&S.st->status, ST_NOCONVERGE);
     // sites a crossing bond may end on: those of segments on a face that is not

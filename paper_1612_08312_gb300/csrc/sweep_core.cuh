@@ -334,23 +334,34 @@ constexpr int IS_CODE = 1 << 20;
 // Synchronous rounds of the resolution before the walks.
 constexpr int RESOLVE_ROUNDS = 1;
 
+// Pairs the list has room for.
+__device__ __forceinline__ int list_room(int nt) { return 15 * nt; }
+
+// Unites the listed pairs, two at a time per thread (after a barrier behind the
+// listing, before one ahead of the labels' next use).  False if a bound was hit.
+__device__ __forceinline__ bool unite_listed(const CoreSmem &s, int nt)
+{
+    bool ok = true;
+    const int np = min(s.pcount[0], list_room(nt));
+    for (int e = threadIdx.x; e < np; e += 2 * nt) {
+        const uint32_t p0 = s.plist[e], p1 = e + nt < np ? s.plist[e + nt] : p0;
+        ok &= sunite2((int)(p0 & 0xFFFFu), (int)(p0 >> 16), (int)(p1 & 0xFFFFu), (int)(p1 >> 16));
+    }
+    return ok;
+}
+
 // The second half of a tile's labelling, for a thread's 16 sites named me, me +
 // 4, ..: unites the listed pairs, resolves every representative (reps) to its
 // root, gives the roots of the sites in `ends` (which a crossing bond may end
 // on) a slot each in P (the root's site: site0 + q for the thread's q-th), and
 // returns in ent the codes of the representatives (entries below IS_CODE are
-// names of roots without a slot).  Called by every thread of the block.
+// names of roots without a slot).  Called by every thread of the block, after a
+// barrier behind the listing.
 template <typename Ends>
 __device__ __forceinline__ void finish_labels(const CoreSmem &s, int nt, int me, uint32_t reps, const Ends &ends_of,
                                               int32_t site0, int32_t *P, int32_t *nslots, int *status, int ent[16])
 {
-    __syncthreads();  // pairs listed
-    bool ok = true;
-    const int np = min(s.pcount[0], 15 * nt);
-    for (int e = threadIdx.x; e < np; e += 2 * nt) {
-        const uint32_t p0 = s.plist[e], p1 = e + nt < np ? s.plist[e + nt] : p0;
-        ok &= sunite2((int)(p0 & 0xFFFFu), (int)(p0 >> 16), (int)(p1 & 0xFFFFu), (int)(p1 >> 16));
-    }
+    const bool ok = unite_listed(s, nt);
     __syncthreads();  // all unions done
     if (!ok) atomicOr(status, ST_NOCONVERGE);
     // Resolution: every representative's entry becomes its root's name.  No
@@ -564,6 +575,7 @@ __device__ __forceinline__ void local_core(const TileCtx &c, const Rep &R, const
         for (int k = 0; k < 12; ++k)
             if (rest[k]) s.plist[pos++] = rest[k];
     }
+    __syncthreads();  // pairs listed
     int ent[16];
     finish_labels(s, nt, me, reps, [&] { return crossing_sites(c); }, (int32_t)(16 * c.cell), R.P + (int64_t)tile * (16 * nt),
                   R.nslots + tile, &R.st->status, ent);
