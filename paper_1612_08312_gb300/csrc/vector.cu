@@ -299,96 +299,6 @@ __global__ void __launch_bounds__(512, 2) vec_local_kernel(const __grid_constant
     local_core(c, R, sm, act[0], act[1], act[2], sweep, tile);
 }
 
-// t <- t / sqrt(t . t), every operation correctly rounded: the bits of sqrt_
-// and div, in fewer operations for the vectors a sweep meets, whose squared
-// length q is within a few units in the last place of 1.  With M mantissa
-// bits and d = bits(q) - bits(1), sqrt(1 + x) = 1 + x/2 - x^2/8 ..: for q d
-// units of 2^-M above 1 (below: -d units of 2^-(M+1)) the correctly rounded
-// root is floor(d / 2) units from 1, the x^2/8 term being far below half a
-// unit for the d taken here; it only breaks the ties of odd d downwards.
-//
-// FP32: the quotients by s = 1 + e follow from one correctly rounded
-// reciprocal r by Markstein's theorem (IBM J. Res. Dev. 34, 1990): with the
-// faithful quotient g = fma(-e, t, t) (e^2 < 2^-27), fma(t - s g, r, g) is the
-// correctly rounded t / s, the residual t - s g being exact in one fma (not
-// for tiny t: those divide).
-template <int NC>
-__device__ __forceinline__ void normalise(float t[NC])
-{
-    float q = t[0] * t[0];
-#pragma unroll
-    for (int k = 1; k < NC; ++k) q = Ar<float>::add(q, Ar<float>::mul(t[k], t[k]));
-    const int d = __float_as_int(q) - 0x3F800000;
-    if (d > -1024 && d < 1024) {
-        const int h = d >> 1;
-        if (h == 0) return;  // the length rounds to 1
-        const float s = __int_as_float(0x3F800000 + h), e = s - 1.0f, r = __frcp_rn(s);
-        bool ok = true;
-        float o[NC];
-#pragma unroll
-        for (int k = 0; k < NC; ++k) {
-            const float g = __fmaf_rn(-e, t[k], t[k]);
-            o[k] = __fmaf_rn(__fmaf_rn(-s, g, t[k]), r, g);
-            ok &= fabsf(t[k]) > 1e-25f;
-        }
-        if (ok) {
-#pragma unroll
-            for (int k = 0; k < NC; ++k) t[k] = o[k];
-            return;
-        }
-    }
-    q = sqrtf(q);
-#pragma unroll
-    for (int k = 0; k < NC; ++k) t[k] = t[k] / q;
-}
-
-// FP64: by integer arithmetic, since roots and quotients took four fifths of
-// the FP64 flip, whose two FP64 lanes a clock per SM bound it.  Quotient of
-// t = T 2^e by s = 1 + h 2^-52, h > 0: T/s = T - T h / (2^52 + h); by
-// s = 1 - k 2^-53: T/s = T + T k / (2^53 - k).  The fraction, rounded to
-// nearest, is its quotient by the power of two alone, rounded, or one step
-// from that (checked by the remainder); no quotient of two floats lies
-// halfway.  A result past the binade of t, a zero and a denormal divide.
-template <int NC>
-__device__ __forceinline__ void normalise(double t[NC])
-{
-    using A = Ar<double>;
-    double q = A::mul(t[0], t[0]);
-#pragma unroll
-    for (int k = 1; k < NC; ++k) q = A::add(q, A::mul(t[k], t[k]));
-    constexpr long long ONE = 0x3FF0000000000000ll, FIELD = (1ll << 52) - 1;
-    const long long d = __double_as_longlong(q) - ONE;
-    if (d > -128 && d < 128) {
-        const int h = (int)d >> 1;
-        if (h == 0) return;  // the length rounds to 1
-        const int m = abs(h), sh = h > 0 ? 52 : 53;
-        const long long D = (1ll << sh) + h;
-        bool ok = true;
-        double o[NC];
-#pragma unroll
-        for (int k = 0; k < NC; ++k) {
-            const long long b = __double_as_longlong(t[k]);
-            const long long mant = b & FIELD;
-            const long long n = (mant | (1ll << 52)) * m;  // below 2^59
-            long long i = (n + (1ll << (sh - 1))) >> sh;
-            const long long r2 = 2 * (n - i * D);
-            if (h > 0) i -= r2 < -D;  // the divisor exceeds the power of two
-            else i += r2 > D;
-            const long long to = h > 0 ? mant - i : mant + i;
-            ok &= to >= 0 && to <= FIELD && ((b >> 53) & 0x3FF) != 0;  // exponent field above 1
-            o[k] = __longlong_as_double(h > 0 ? b - i : b + i);
-        }
-        if (ok) {
-#pragma unroll
-            for (int k = 0; k < NC; ++k) t[k] = o[k];
-            return;
-        }
-    }
-    q = A::sqrt_(q);
-#pragma unroll
-    for (int k = 0; k < NC; ++k) t[k] = A::div(t[k], q);
-}
-
 // s <- the reflection s - 2 (s . r) r, normalised.
 template <int NC, typename T>
 __device__ __forceinline__ void reflect(T t[NC], const T r[3])
