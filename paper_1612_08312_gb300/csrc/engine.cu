@@ -245,16 +245,20 @@ static int64_t tiles_of(int L, const TileShape &t)
 // crossing unions of its faces; w is the measured cost of the crossing phase
 // per face cell over the local phase's per cell (Ising L = 256: 640 us over 0.5
 // face cells per cell against 1,449; n = 3, L = 128: 91 over 0.5 against 268).
-// Before, the edges were the largest powers of two dividing L: one-cell tiles
-// of one thread for odd L (Ising L = 45: 951 us a sweep then, 99 with this).
+// Edges that divide L would be one cell for odd L, tiles of one thread (Ising
+// L = 45 938 us a sweep, 87 with this rule).
 //
 // cap.  Sets that do not fill the GPU are bound by a block's latency, which
 // grows with its threads; sets that do, by the crossing work, which falls with
-// the tile.  A sweep in us at 64 / 128 / 256 cells: Ising L = 32 39.5 / 39.2 / 40.2,
-// L = 64 78.9 / 72.4 / 74.5, L = 128 (phases) - / 364 / 352 and 367 at 512; n = 3
-// L = 32 50.0 / 52.2 / 55.4, L = 64 112.8 / 109.4 / 108.7, L = 128 (phases)
-// 715 / 652 / 621.  One lattice that a block of 512 cells covers has no crossing
-// work at all: L = 8 25.4, and 27.9 with two tiles of 256.
+// the tile.  A sweep in us at 64 / 128 / 256 cells: Ising L = 16 30.2 / 30.1 / 32.4,
+// L = 32 35.6 / 33.1 / 36.0, L = 64 73.2 / 68.1 / 70.1, L = 72 94.8 / 80.0 / 85.5, L = 96
+// 181 / 151 / 149, L = 128 401 / 324 / 311 and 322 at 512: 128 and 256 meet between
+// L = 80 and 96, past the line at L = 66.  n = 3, FP32 L = 16 39.8 / 42.3 / 47.5, L = 32
+// 47.0 / 48.9 / 52.0, L = 48 65.5 / 64.3 / 66.3, L = 64 109 / 106 / 106, L = 80
+// 192 / 182 / 176; FP64 L = 32 90 / 95 / 104, L = 48 182 / 192 / 211, L = 64
+// 318 / 313 / 323: 64 and 256 meet near the line at L = 40 for FP32, near L = 64 for FP64.
+// One lattice that a block of 512 cells covers has no crossing work at all: L = 8
+// 21.4, and 24.3 with two tiles of 256.
 TileShape default_tile(const int *Ls, int R, int model)
 {
     int64_t cells = 0;

@@ -172,8 +172,9 @@ __global__ void __launch_bounds__(GB_THREADS) graph_proj_kernel(const __grid_con
 // at once.)  The bonds are decided first, all sites and spins loaded together
 // (bond after bond, each waited for its own sites, spins and unions), then the
 // active ones are united in a loop of their own: chains of dependent reads,
-// for which every warp the SM holds counts (simple cubic L = 256, a sweep with
-// 48, 40 and 32 registers: 697, 636 and 568 us).
+// for which every warp the SM holds counts (Ising, a simple-cubic bond list, a
+// sweep with 48, 40 and 32 registers: L = 256 727, 674 and 615 us, L = 128 124,
+// 117 and 117; below L = 100, where the SMs are not full, 32 are 1 to 4 % slower).
 template <int NC, typename T>
 __global__ void __launch_bounds__(GB_THREADS, NC == 1 ? 8 : 4) graph_bond_kernel(const __grid_constant__ GraphDev G)
 {
@@ -571,8 +572,8 @@ struct GraphEngine {
         const int64_t nchunk = std::max(cdiv(NB, 16), cdiv(N, 128));
         nbond = (unsigned)std::max<int64_t>(1, cdiv(nchunk, GB_THREADS));
         nsite = (unsigned)cdiv(N, GB_THREADS);
-        nproj = (unsigned)std::min<int64_t>(cdiv(N, GB_THREADS), 152 * 8);
-        nmeas = (unsigned)std::min<int64_t>(cdiv(std::max(N, NB), GB_THREADS), model == PYRO_ISING ? 152 * 4 : 152 * 8);
+        nproj = (unsigned)std::min<int64_t>(cdiv(N, GB_THREADS), GPU_SMS * 8);
+        nmeas = (unsigned)std::min<int64_t>(cdiv(std::max(N, NB), GB_THREADS), model == PYRO_ISING ? GPU_SMS * 4 : GPU_SMS * 8);
         struct {
             void **p;
             size_t bytes;
@@ -639,6 +640,14 @@ struct GraphEngine {
     // Tile of the simple-cubic sweep: the power-of-two tile of at most `cap`
     // segments whose padded cost is least, each axis it does not cover adding its
     // crossing faces (as default_tile in engine.cu).
+    //
+    // cap.  A sweep in us at 64 / 128 / 256 segments, at the critical temperature:
+    // L = 16 (a lone tile at 256) 29.0 / 26.6 / 21.7, L = 32 36.4 / 36.0 / 34.8, L = 64
+    // 47.0 / 40.3 / 39.4, L = 128 66.2 / 61.2 / 60.0, L = 256 226 / 213 / 213; at
+    // beta = 1, where the trees are deep: L = 16 49 / 53 / 62, L = 32 51 / 57 / 78,
+    // L = 64 63 / 63 / 71, L = 128 91 / 99 / 112.  Lattices of several tiles that do
+    // not fill the GPU, bound by a block's latency, take 64: up to a sixth slower at
+    // the transition, up to a third faster below it.
     void sc_tile()
     {
         const int64_t segs = (int64_t)sc.SX * sc.L * sc.L;
@@ -691,7 +700,7 @@ struct GraphEngine {
         sc_tile();
         const int nt = sc.TX * sc.TY * sc.TZ;
         sc_tiles = (unsigned)sc.ntx * (unsigned)sc.nty * (unsigned)sc.ntz;
-        nmeas = (unsigned)std::min<int64_t>(cdiv((int64_t)sc_tiles * nt, 256), 152 * 4);
+        nmeas = (unsigned)std::min<int64_t>(cdiv((int64_t)sc_tiles * nt, 256), GPU_SMS * 4);
         const size_t segs = (size_t)sc.nsegs, mask = present.empty() ? 0 : segs * 2;
         struct {
             void **p;

@@ -389,7 +389,7 @@ void launch_boundary(const Batch &B, int64_t ntiles, cudaStream_t s)
     // is the kernel's time (L = 16: 41 -> 36 us a sweep, L = 45: 62 -> 53; four
     // at L = 256: crossing 685 -> 955 us)
     int threads = (nf + 31) & ~31;
-    while (2 * threads <= 512 && 2 * threads <= 4 * ((nf + 31) & ~31) && ntiles * (2 * threads) <= 152 * 2048) threads *= 2;
+    while (2 * threads <= 512 && 2 * threads <= 4 * ((nf + 31) & ~31) && ntiles * (2 * threads) <= GPU_THREADS) threads *= 2;
     const size_t smem = (size_t)nf * 12 * sizeof(uint32_t);
     launch_overlapped(boundary_unite_kernel, (unsigned)ntiles, threads, smem, s, B);
     launch_overlapped(boundary_flip_kernel, (unsigned)ntiles, SLOT_BLOCK, 0, s, B);

@@ -17,6 +17,9 @@
 
 namespace pyro {
 
+constexpr int GPU_SMS = 152;                // multiprocessors of a GB300
+constexpr int GPU_THREADS = GPU_SMS * 2048;  // threads it holds at once
+
 __device__ __forceinline__ void overlap_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void overlap_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void overlap_begin()

@@ -114,9 +114,9 @@ struct TileShape {
 // One lattice (replica) as the kernels see it.
 struct Rep {
     void *spins;       // Ising: uint16 per cell; n-vector: n planes of N values
-    uint16_t *L16;     // per site: its code, the tile-local index of its tile-local
-                       // root, or 16 nt + the root's slot if its cluster may
-                       // cross a tile face (nt = the tile's cells)
+    uint16_t *L16;     // per site: its code, the word 17 t + s of its tile-local root
+                       // (cell t of the tile, site s), or slot_code(nt) + the root's
+                       // slot if its cluster may cross a tile face (nt = the tile's cells)
     int32_t *P;        // per tile 16 nt slots: the root's site, or a link to a slot
     int32_t *nslots;   // per tile: slots in use
     uint32_t *sflip;   // per tile 16 nt bits: the flip bit of each slot's cluster
@@ -137,7 +137,8 @@ struct Rep {
 // Up to MAX_REPS lattices updated by one launch per phase.  Blocks of the
 // tiled kernels map to (replica, tile) through tile_begin; blocks of the
 // per-cell kernels (256 cells each) through block_begin.  Tile edges are
-// powers of two that divide every replica's L.
+// powers of two; they need not divide a replica's L, so that its last tiles may
+// reach past it (TileCtx::valid).
 constexpr int MAX_REPS = 64;
 constexpr int CELL_BLOCK = 256;
 

@@ -534,8 +534,8 @@ __device__ __forceinline__ void local_core(const TileCtx &c, const Rep &R, const
     // First pass over all pairs, without finds: each links the larger of its
     // ends' parents under the other if that is a root still (seven pairs of
     // ten), else it is listed, as the pair of that root's new parent and the
-    // smaller one.  Before, all pairs were listed and united with full finds
-    // in three rounds, whose barriers waited for the longest chains.
+    // smaller one.  (All pairs listed and united with full finds took three
+    // rounds, whose barriers waited for the longest chains.)
     uint32_t rest[12];
     uint32_t nrest = 0;
     const bool unite = c_unite_bound > 0;
