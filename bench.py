@@ -87,10 +87,11 @@ def kernel_source_hash() -> str:
     return h.hexdigest()[:16]
 
 
-def committed_traffic(kernel: str, nsites: int):
+def committed_traffic(kernel: str, nsites: int, tile=None):
     """DRAM bytes per launch of `kernel` on an nsites lattice, from the
     committed ncu summary (bytes per site of the captured case), if it was
-    taken on the current kernel sources; else None."""
+    taken on the current kernel sources and, where the line names one, with
+    the same labelling tile; else None."""
     path = os.path.join(ROOT, "profiles", "traffic.txt")
     if not os.path.exists(path):
         return None
@@ -98,6 +99,8 @@ def committed_traffic(kernel: str, nsites: int):
     for line in open(path):
         parts = line.split()
         if len(parts) >= 3 and not line.startswith("#") and parts[0] == kernel and parts[2] == src:
+            if tile is not None and len(parts) >= 4 and parts[3] != "x".join(str(v) for v in tile):
+                continue
             return float(parts[1]) * nsites
     return None
 
@@ -411,7 +414,7 @@ def main():
         dominant = max(prof, key=prof.get)
         alg_bytes = PHASE_BYTES_PER_SITE[dominant] * N
         achieved = alg_bytes / (prof[dominant] * 1e-3) / 1e9
-        traffic = committed_traffic(KERNEL_NAMES[dominant], N)
+        traffic = committed_traffic(KERNEL_NAMES[dominant], N, tile)
         out["roofline"] = {"bound": "hbm", "kernel": KERNEL_NAMES[dominant], "achieved": achieved, "peak": peak,
                            "unit": "GB/s", "frac": achieved / peak, "peak_kind": peak_kind, "traffic": traffic,
                            "alg_bytes_per_site": PHASE_BYTES_PER_SITE[dominant],
